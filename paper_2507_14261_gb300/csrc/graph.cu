@@ -185,9 +185,38 @@ __device__ __forceinline__ int uf_find(int32_t *parent_, int v, int limit, int *
     return v;
 }
 
-__global__ void uf_init_kernel(int32_t *parent, int64_t n) {
-    int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (v < n) parent[v] = int32_t(v);
+// Hooks. Hooking every edge by itself makes the threads in flight fight for
+// the few roots their edges share (50k points of two moons: 1.2 ms, the
+// hubs' roots changing hands one compare-and-swap at a time). So the forest
+// is first grown by rounds without retries: every vertex points at its
+// smallest neighbour; then, twice, every edge between two roots lowers the
+// larger root's parent by atomicMin, after a plain read that filters most of
+// them. A round may replace a link by another; uf_hook_kernel then goes over
+// all edges, which mostly find equal roots in one read of each end, and
+// joins what is still apart.
+constexpr int UF_ROUNDS = 2;
+
+__global__ void uf_min_kernel(const int32_t *__restrict__ nbr, int64_t n, int k,
+                              int32_t *__restrict__ parent) {
+    const int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (v >= n) return;
+    int m = int(v);
+    for (int j = 0; j < k; ++j) {
+        const int b = __ldg(nbr + v * k + j);
+        m = b >= 0 && b < m ? b : m;
+    }
+    parent[v] = m;
+}
+
+__global__ void uf_lower_kernel(const int32_t *__restrict__ nbr, int64_t nk, int k,
+                                int32_t *parent_) {
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= nk) return;
+    volatile int32_t *parent = parent_;
+    const int ra = parent[e / k], rb = parent[nbr[e]];
+    if (ra == rb) return;
+    const int hi = ra > rb ? ra : rb, lo = ra > rb ? rb : ra;
+    if (parent[hi] > lo) atomicMin(parent_ + hi, lo);
 }
 
 // Vertices in a scrambled order: thread e takes edge j = e mod k of vertex
@@ -195,15 +224,18 @@ __global__ void uf_init_kernel(int32_t *parent, int64_t n) {
 // [0, 2^m), 2^m >= n; v >= n idle). When ids are contiguous in space (clouds
 // laid out one after another, sorted inputs), threads in flight together
 // would otherwise all hook onto the same few roots.
-__global__ void uf_hook_kernel(const int32_t *__restrict__ nbr, int64_t n, int k,
-                               uint32_t vmask, int32_t *parent, int limit, int *dstatus) {
+__global__ void uf_hook_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, uint32_t vmask,
+                               int32_t *parent, int limit, int *dstatus) {
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t vl = e / k;
     if (vl > int64_t(vmask)) return;
     const uint32_t v = (uint32_t(vl) * 0x9E3779B1u) & vmask;
     if (int64_t(v) >= n) return;
-    int a = int(v), b = nbr[int64_t(v) * k + (e - vl * k)];
-    int ra = uf_find(parent, a, limit, dstatus), rb = uf_find(parent, b, limit, dstatus);
+    const int a = int(v), b = nbr[int64_t(v) * k + (e - vl * k)];
+    const int pa = *reinterpret_cast<volatile int32_t *>(parent + a);
+    const int pb = *reinterpret_cast<volatile int32_t *>(parent + b);
+    if (pa == pb) return;   // one common ancestor: already joined
+    int ra = uf_find(parent, pa, limit, dstatus), rb = uf_find(parent, pb, limit, dstatus);
     for (int it = 0; it < limit; ++it) {
         if (ra == rb) return;
         int hi = ra > rb ? ra : rb, lo = ra > rb ? rb : ra;
@@ -214,6 +246,12 @@ __global__ void uf_hook_kernel(const int32_t *__restrict__ nbr, int64_t n, int k
         else rb = uf_find(parent, old, limit, dstatus);
     }
     set_status(dstatus, STATUS_LOOP_LIMIT);
+}
+
+// every vertex points at its root (no hooks run beside this kernel)
+__global__ void uf_compress_kernel(int32_t *parent, int64_t n, int limit, int *dstatus) {
+    const int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (v < n) *reinterpret_cast<volatile int32_t *>(parent + v) = uf_find(parent, int(v), limit, dstatus);
 }
 
 // Roots go to a separate array: a concurrent find may still rewrite
@@ -342,12 +380,18 @@ famst_status components_uf(const Exec &ex, Arena &ar, const int32_t *nbr, int64_
     const int th = 256;
     const int lim = ex.loop_limit > 0 ? ex.loop_limit : UF_LIMIT;
     int64_t nk = n * k;
-    FAMST_LAUNCH(ex, uf_init_kernel, blocks_for(n, th), th, 0, parent, n);
+    FAMST_LAUNCH(ex, uf_min_kernel, blocks_for(n, th), th, 0, nbr, n, nk > 0 ? k : 0, parent);
     if (nk > 0) {
+        for (int r = 0; r < UF_ROUNDS; ++r) {
+            FAMST_LAUNCH(ex, uf_compress_kernel, blocks_for(n, th), th, 0, parent, n, lim,
+                         ex.dstatus);
+            FAMST_LAUNCH(ex, uf_lower_kernel, blocks_for(nk, th), th, 0, nbr, nk, k, parent);
+        }
+        FAMST_LAUNCH(ex, uf_compress_kernel, blocks_for(n, th), th, 0, parent, n, lim, ex.dstatus);
         uint32_t vmask = 1;
         while (int64_t(vmask) + 1 < n) vmask = (vmask << 1) | 1u;
-        FAMST_LAUNCH(ex, uf_hook_kernel, blocks_for((int64_t(vmask) + 1) * k, th), th, 0, nbr, n,
-                     k, vmask, parent, lim, ex.dstatus);
+        FAMST_LAUNCH(ex, uf_hook_kernel, blocks_for((int64_t(vmask) + 1) * k, th), th, 0, nbr, n, k,
+                     vmask, parent, lim, ex.dstatus);
     }
     FAMST_LAUNCH(ex, uf_flatten_kernel, blocks_for(n, th), th, 0, parent, n, root, flag, lim,
                  ex.dstatus);

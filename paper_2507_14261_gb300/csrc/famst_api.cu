@@ -251,10 +251,15 @@ bool vec4_ok(const float *X, int d) {
     return (d % 4 == 0) && (reinterpret_cast<uintptr_t>(X) % 16 == 0);
 }
 
-famst_status check_points(famst_ctx *ctx, const float *X, int64_t n, int32_t d) {
+famst_status check_points_args(famst_ctx *ctx, const float *X, int64_t n, int32_t d) {
     if (!X) return fail(ctx, FAMST_ERR_INVALID_ARG, "X is NULL");
     if (n < 1 || d < 1) return fail(ctx, FAMST_ERR_INVALID_ARG, "need n >= 1 and d >= 1");
     if (n >= (int64_t(1) << 31)) return fail(ctx, FAMST_ERR_UNSUPPORTED, "n must be < 2^31");
+    return FAMST_OK;
+}
+
+famst_status check_points(famst_ctx *ctx, const float *X, int64_t n, int32_t d) {
+    ST(check_points_args(ctx, X, n, d));
     Exec ex = exec_of(ctx);
     FAMST_LAUNCH(ex, check_finite_kernel, grid_cap(ctx, n * d, 256), 256, 0, X, n * d,
                  ctx->dstatus);
@@ -1330,16 +1335,10 @@ famst_status famst_mst_backward(famst_ctx *ctx, const float *X, int64_t n, int32
     CK(cudaSetDevice(ctx->device));
     ST(reset_status(ctx));
     if (n < 1 || (n * int64_t(d)) >= (int64_t(1) << 40)) return fail(ctx, FAMST_ERR_INVALID_ARG, "bad n/d");
-    ST(check_points(ctx, X, n, d));
-    Exec ex = exec_of(ctx);
-    if (m > 0) {
-        FAMST_LAUNCH(ex, check_ids_kernel, grid_cap(ctx, m, 256), 256, 0, tu, m, n, 0, ctx->dstatus);
-        FAMST_LAUNCH(ex, check_ids_kernel, grid_cap(ctx, m, 256), 256, 0, tv, m, n, 0, ctx->dstatus);
-    }
-    ST(sync_status(ctx));
+    ST(check_points_args(ctx, X, n, d));   // the gradient kernel checks the values it reads
     Arena ar;
     ST(ensure_ws(ctx, 1, mst_backward_workspace(n, m), ar));
-    ST(mst_backward(ex, ar, X, n, d, vec4_ok(X, d), tu, tv, m, gW, gX));
+    ST(mst_backward(exec_of(ctx), ar, X, n, d, tu, tv, m, gW, gX, ctx->pinned + PIN_T));
     return sync_status(ctx);
 }
 

@@ -714,8 +714,8 @@ famst_status tree_weight(const Exec &ex, Arena &ar, const float *X, int d, bool 
                          double *W_dev /*2 doubles: W, W64*/);
 size_t tree_weight_workspace(int64_t m);
 famst_status mst_backward(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
-                          bool vec4, const int32_t *tu, const int32_t *tv, int64_t m,
-                          float gW, float *gX);
+                          const int32_t *tu, const int32_t *tv, int64_t m, float gW, float *gX,
+                          int32_t *pinned_host);
 size_t mst_backward_workspace(int64_t n, int64_t m);
 
 // emst.cu

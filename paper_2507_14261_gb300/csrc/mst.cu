@@ -301,48 +301,226 @@ __global__ void weight_final_kernel(const double *__restrict__ part, int64_t nb,
 }
 
 // ----------------------------------------------------------- backward
+//
+// Bound: HBM and the latency of its dependent loads. Every vertex's row is
+// read once for itself and once per incident edge (about 3 n d floats for a
+// tree, 1.5 GB at 1M x 128) and the gradient is written once. A warp owns a
+// vertex: its row stays in registers, lane l holding the coordinates l,
+// l + 32, ... of both rows, which are the canonical distance's own partials,
+// so the edge's length comes out of the loads the gradient needs anyway; no
+// pass over the edges computes or stores lengths, and the finiteness check
+// rides along. The incidences are placed by counting and ranked inside their
+// vertex (ascending edge index) instead of radix sorted; a vertex beyond
+// INC_RANK_MAX edges sends the call to the radix sort, whose cost does not
+// depend on the degrees.
 
-template <int VEC>
-__global__ void edge_len_kernel(const float *__restrict__ X, int d,
-                                const int32_t *__restrict__ tu, const int32_t *__restrict__ tv,
-                                int64_t m, float *__restrict__ wl) {
-    int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (e < m) wl[e] = canon_dist<VEC>(X + int64_t(tu[e]) * d, X + int64_t(tv[e]) * d, d);
+constexpr int INC_RANK_MAX = 2048;   // a rank reads its vertex's whole list (about 20 us here)
+
+// Range check, degrees and each incidence's arrival number at its vertex;
+// maxdeg[0] = the largest degree.
+__global__ void incidence_count_kernel(const int32_t *__restrict__ tu,
+                                       const int32_t *__restrict__ tv, int64_t m, int64_t n,
+                                       int32_t *__restrict__ deg, int2 *__restrict__ slot,
+                                       int32_t *__restrict__ maxdeg, int *dstatus) {
+    __shared__ int bmax;
+    if (threadIdx.x == 0) bmax = 0;
+    __syncthreads();
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    int mx = 0;
+    if (e < m) {
+        const int u = tu[e], v = tv[e];
+        if (u < 0 || v < 0 || int64_t(u) >= n || int64_t(v) >= n) {
+            set_status(dstatus, STATUS_BAD_ID);
+        } else {
+            const int su = atomicAdd(&deg[u], 1), sv = atomicAdd(&deg[v], 1);
+            slot[e] = make_int2(su, sv);
+            mx = (su > sv ? su : sv) + 1;
+        }
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&bmax, mx);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(maxdeg, bmax);
 }
 
+__global__ void incidence_fill_kernel(const int32_t *__restrict__ tu,
+                                      const int32_t *__restrict__ tv, int64_t m,
+                                      const int32_t *__restrict__ off,
+                                      const int2 *__restrict__ slot, int32_t *__restrict__ inc) {
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= m) return;
+    const int2 s = slot[e];
+    inc[off[tu[e]] + s.x] = int(2 * e);
+    inc[off[tv[e]] + s.y] = int(2 * e + 1);
+}
+
+// adj: per vertex, its edges' other ends in ascending edge index
+__global__ void incidence_rank_kernel(const int32_t *__restrict__ tu,
+                                      const int32_t *__restrict__ tv, int64_t m,
+                                      const int32_t *__restrict__ off,
+                                      const int32_t *__restrict__ inc, int32_t *__restrict__ adj) {
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= m) return;
+    const int u = tu[e], v = tv[e];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const int a = side ? v : u, code = int(2 * e) + side;
+        const int j0 = off[a], j1 = off[a + 1];
+        int r = 0;
+        for (int j = j0; j < j1; ++j) r += __ldg(inc + j) < code;
+        adj[j0 + r] = side ? u : v;
+    }
+}
+
+// The radix sort's input (a vertex of large degree) and its adj entries.
 __global__ void incidence_kernel(const int32_t *__restrict__ tu, const int32_t *__restrict__ tv,
-                                 int64_t m, uint32_t *__restrict__ keys, int32_t *__restrict__ vals,
-                                 int32_t *__restrict__ deg) {
-    int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+                                 int64_t m, uint32_t *__restrict__ keys,
+                                 int32_t *__restrict__ vals) {
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (e >= m) return;
     keys[2 * e] = uint32_t(tu[e]);
     vals[2 * e] = int32_t(2 * e);
     keys[2 * e + 1] = uint32_t(tv[e]);
     vals[2 * e + 1] = int32_t(2 * e + 1);
-    atomicAdd(&deg[tu[e]], 1);
-    atomicAdd(&deg[tv[e]], 1);
+}
+
+__global__ void incidence_adj_kernel(const int32_t *__restrict__ tu,
+                                     const int32_t *__restrict__ tv, int64_t m2,
+                                     const int32_t *__restrict__ inc, int32_t *__restrict__ adj) {
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= m2) return;
+    const int code = inc[i];
+    adj[i] = (code & 1) ? tu[code >> 1] : tv[code >> 1];
 }
 
 // gX[v][t] = gW * sum over v's edges, ascending edge index, of
-// (x_v[t] - x_other[t]) / w_e  (w_e = 0 contributes 0)
-__global__ void grad_kernel(const float *__restrict__ X, int64_t n, int d,
-                            const int32_t *__restrict__ tu, const int32_t *__restrict__ tv,
-                            const float *__restrict__ wl, const int32_t *__restrict__ off,
-                            const int32_t *__restrict__ inc, float gW, float *__restrict__ gX) {
-    int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (idx >= n * d) return;
-    int64_t v = idx / d;
-    int t = int(idx - v * d);
-    float xs = X[idx];
+// (x_v[t] - x_other[t]) / w_e  (w_e = 0 contributes 0).
+// Narrow rows (d <= 16): G lanes per vertex, G the power of two that holds d
+// (the canonical butterfly's wider steps would add zeros).
+template <int G>
+__global__ void grad_narrow_kernel(const float *__restrict__ X, int64_t n, int d,
+                                   const int32_t *__restrict__ off,
+                                   const int32_t *__restrict__ adj, float gW,
+                                   float *__restrict__ gX, int *dstatus) {
+    const int64_t v = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / G;
+    if (v >= n) return;   // whole groups
+    const int lane = threadIdx.x & 31, g = lane % G;
+    const unsigned gmask = ((1u << G) - 1u) << (lane - g);
+    const float x = g < d ? X[v * d + g] : 0.0f;
+    if (!isfinite(x)) set_status(dstatus, STATUS_NONFINITE);
     float acc = 0.0f;
-    for (int q = off[v]; q < off[v + 1]; ++q) {
-        int code = inc[q];
-        int e = code >> 1;
-        int other = (code & 1) ? tu[e] : tv[e];
-        float w = wl[e];
-        if (w > 0.0f) acc = __fadd_rn(acc, __fdiv_rn(__fsub_rn(xs, X[int64_t(other) * d + t]), w));
+    const int j1 = off[v + 1];
+    for (int j = off[v]; j < j1; ++j) {
+        const float y = g < d ? __ldg(X + int64_t(adj[j]) * d + g) : 0.0f;
+        const float dl = __fsub_rn(x, y);
+        float p = __fmaf_rn(dl, dl, 0.0f);
+#pragma unroll
+        for (int o = G / 2; o >= 1; o >>= 1) p = __fadd_rn(p, __shfl_xor_sync(gmask, p, o));
+        const float w = __fsqrt_rn(p);
+        if (w > 0.0f) acc = __fadd_rn(acc, __fdiv_rn(dl, w));
     }
-    gX[idx] = __fmul_rn(gW, acc);
+    if (g < d) gX[v * d + g] = __fmul_rn(gW, acc);
+}
+
+// A warp takes GRAD_V consecutive vertices: their offsets and the ends of
+// their edges come with one load each, and while a vertex is summed the next
+// one's row and its first two neighbours' rows are on their way (a tree
+// vertex has two edges on average), so a warp waits for the chain offset ->
+// edge end -> row once per GRAD_V vertices instead of once per vertex.
+// A lane holds XR coordinates; rows wider than 32 XR (WIDE) take the
+// coordinates in chunks of 32 XR and evaluate each edge's length again per
+// chunk.
+constexpr int GRAD_V = 8;
+template <int XR, bool WIDE>
+__global__ void __launch_bounds__(256) grad_rows_kernel(const float *__restrict__ X, int64_t n, int d,
+                                 const int32_t *__restrict__ off, const int32_t *__restrict__ adj,
+                                 float gW, float *__restrict__ gX, int *dstatus) {
+    const int64_t vb = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * GRAD_V;
+    if (vb >= n) return;
+    const int lane = threadIdx.x & 31;
+    const int nv = n - vb < GRAD_V ? int(n - vb) : GRAD_V;
+    const int o = off[vb + (lane < nv ? lane : nv)];
+    const int base = __shfl_sync(0xffffffffu, o, 0), last = __shfl_sync(0xffffffffu, o, nv);
+    const int aj = base + lane < last ? adj[base + lane] : 0;
+    auto end_of = [&](int j) {   // the other end of entry j (warp-uniform)
+        const int a = __shfl_sync(0xffffffffu, aj, (j - base) & 31);
+        return j - base < 32 ? a : __ldg(adj + j);
+    };
+    bool bad = false;
+    for (int c0 = 0; c0 < d; c0 += 32 * XR) {
+        float xn[XR], yn[2][XR];
+        const float *yp[2] = {X, X};
+        auto row = [&](const float *r, float(&f)[XR]) {
+#pragma unroll
+            for (int q = 0; q < XR; ++q) {
+                const int t = c0 + lane + 32 * q;
+                f[q] = t < d ? __ldg(r + t) : 0.0f;
+            }
+        };
+        auto fetch = [&](int i) {   // vertex vb + i and its first two neighbours
+            const int j0 = __shfl_sync(0xffffffffu, o, i), j1 = __shfl_sync(0xffffffffu, o, i + 1);
+            row(X + (vb + i) * d, xn);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (j0 + e < j1) {
+                    yp[e] = X + int64_t(end_of(j0 + e)) * d;
+                    row(yp[e], yn[e]);
+                }
+            }
+        };
+        fetch(0);
+        for (int i = 0; i < nv; ++i) {
+            const int j0 = __shfl_sync(0xffffffffu, o, i), j1 = __shfl_sync(0xffffffffu, o, i + 1);
+            float xs[XR], acc[XR], y[2][XR];
+            const float *yc[2] = {yp[0], yp[1]};
+            const float *xr = X + (vb + i) * d;
+#pragma unroll
+            for (int q = 0; q < XR; ++q) {
+                xs[q] = xn[q];
+                y[0][q] = yn[0][q];
+                y[1][q] = yn[1][q];
+                acc[q] = 0.0f;
+                bad |= !isfinite(xs[q]);
+            }
+            if (i + 1 < nv) fetch(i + 1);
+            auto add = [&](const float *yr, const float(&yv)[XR]) {
+                float p = 0.0f;
+                if constexpr (WIDE) {
+                    for (int t = lane; t < d; t += 32) {
+                        const float dl = __fsub_rn(__ldg(xr + t), __ldg(yr + t));
+                        p = __fmaf_rn(dl, dl, p);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < XR; ++q) {
+                        const float dl = __fsub_rn(xs[q], yv[q]);
+                        p = __fmaf_rn(dl, dl, p);
+                    }
+                }
+#pragma unroll
+                for (int s = 16; s >= 1; s >>= 1) p = __fadd_rn(p, __shfl_xor_sync(0xffffffffu, p, s));
+                const float w = __fsqrt_rn(p);
+                if (w > 0.0f) {
+#pragma unroll
+                    for (int q = 0; q < XR; ++q)
+                        acc[q] = __fadd_rn(acc[q], __fdiv_rn(__fsub_rn(xs[q], yv[q]), w));
+                }
+            };
+            if (j0 < j1) add(yc[0], y[0]);
+            if (j0 + 1 < j1) add(yc[1], y[1]);
+            for (int j = j0 + 2; j < j1; ++j) {
+                const float *yr = X + int64_t(end_of(j)) * d;
+                row(yr, y[0]);
+                add(yr, y[0]);
+            }
+#pragma unroll
+            for (int q = 0; q < XR; ++q) {
+                const int t = c0 + lane + 32 * q;
+                if (t < d) gX[(vb + i) * d + t] = __fmul_rn(gW, acc[q]);
+            }
+        }
+    }
+    if (bad) set_status(dstatus, STATUS_NONFINITE);
 }
 
 // Record the round's tree edges at base + pos (base and the round's count
@@ -589,36 +767,72 @@ famst_status tree_weight(const Exec &ex, Arena &ar, const float *X, int d, bool 
 }
 
 size_t mst_backward_workspace(int64_t n, int64_t m) {
-    return align256(size_t(m) * 4) + align256(size_t(2 * m) * 4) * 2 +
-           align256(size_t(n + 1) * 4) * 2 + radix_sort_workspace(2 * m) + scan_workspace(n + 1);
+    return align256(size_t(m) * 8) + align256(size_t(2 * m) * 4) * 3 +
+           align256(size_t(n + 2) * 4) + align256(size_t(n + 1) * 4) +
+           radix_sort_workspace(2 * m) + scan_workspace(n + 1);
 }
 
-famst_status mst_backward(const Exec &ex, Arena &ar, const float *X, int64_t n, int d, bool vec4,
-                          const int32_t *tu, const int32_t *tv, int64_t m, float gW, float *gX) {
-    float *wl = ar.take<float>(size_t(m > 0 ? m : 1));
-    uint32_t *keys = ar.take<uint32_t>(size_t(2 * m > 0 ? 2 * m : 1));
-    int32_t *inc = ar.take<int32_t>(size_t(2 * m > 0 ? 2 * m : 1));
-    int32_t *deg = ar.take<int32_t>(size_t(n + 1));
+// pinned_host: two pinned host words. Ids are checked before they are used;
+// synchronises once (the status word and the largest degree).
+famst_status mst_backward(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
+                          const int32_t *tu, const int32_t *tv, int64_t m, float gW, float *gX,
+                          int32_t *pinned_host) {
+    int2 *slot = ar.take<int2>(size_t(m > 0 ? m : 1));
+    int32_t *inc = ar.take<int32_t>(size_t(m > 0 ? 2 * m : 1));
+    int32_t *adj = ar.take<int32_t>(size_t(m > 0 ? 2 * m : 1));
+    int32_t *deg = ar.take<int32_t>(size_t(n + 2));   // [n + 1]: the largest degree
     int32_t *off = ar.take<int32_t>(size_t(n + 1));
-    if (!wl || !keys || !inc || !deg || !off) return FAMST_ERR_OOM;
+    if (!slot || !inc || !adj || !deg || !off) return FAMST_ERR_OOM;
     const int th = 256;
-    if (cudaMemsetAsync(deg, 0, size_t(n + 1) * 4, ex.stream) != cudaSuccess)
+    if (cudaMemsetAsync(deg, 0, size_t(n + 2) * 4, ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
-    if (m > 0) {
-        if (vec4)
-            FAMST_LAUNCH(ex, edge_len_kernel<4>, blocks_for(m, th), th, 0, X, d, tu, tv, m, wl);
-        else
-            FAMST_LAUNCH(ex, edge_len_kernel<1>, blocks_for(m, th), th, 0, X, d, tu, tv, m, wl);
-        FAMST_LAUNCH(ex, incidence_kernel, blocks_for(m, th), th, 0, tu, tv, m, keys, inc, deg);
-        int bits = 0;
-        while ((int64_t(1) << bits) < n) ++bits;
-        famst_status st = radix_sort_pairs(ex, ar, keys, inc, 2 * m, bits);
-        if (st != FAMST_OK) return st;
-    }
+    if (m > 0)
+        FAMST_LAUNCH(ex, incidence_count_kernel, blocks_for(m, th), th, 0, tu, tv, m, n, deg, slot,
+                     deg + n + 1, ex.dstatus);
     famst_status st = exclusive_scan_i32(ex, ar, deg, off, n + 1, nullptr);
     if (st != FAMST_OK) return st;
-    FAMST_LAUNCH(ex, grad_kernel, blocks_for(n * d, th), th, 0, X, n, d, tu, tv, wl, off, inc, gW,
-                 gX);
+    if (m > 0) {
+        if (cudaMemcpyAsync(pinned_host, deg + n + 1, 4, cudaMemcpyDeviceToHost, ex.stream) !=
+                cudaSuccess ||
+            cudaMemcpyAsync(pinned_host + 1, ex.dstatus, 4, cudaMemcpyDeviceToHost, ex.stream) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(ex.stream) != cudaSuccess)
+            return FAMST_ERR_CUDA;
+        if (pinned_host[1] != 0) return FAMST_OK;   // an id out of range: the caller reads the status
+        if (pinned_host[0] <= INC_RANK_MAX) {
+            FAMST_LAUNCH(ex, incidence_fill_kernel, blocks_for(m, th), th, 0, tu, tv, m, off, slot,
+                         inc);
+            FAMST_LAUNCH(ex, incidence_rank_kernel, blocks_for(m, th), th, 0, tu, tv, m, off, inc,
+                         adj);
+        } else {
+            uint32_t *keys = ar.take<uint32_t>(size_t(2 * m));
+            if (!keys) return FAMST_ERR_OOM;
+            FAMST_LAUNCH(ex, incidence_kernel, blocks_for(m, th), th, 0, tu, tv, m, keys, inc);
+            int bits = 0;
+            while ((int64_t(1) << bits) < n) ++bits;
+            st = radix_sort_pairs(ex, ar, keys, inc, 2 * m, bits);
+            if (st != FAMST_OK) return st;
+            FAMST_LAUNCH(ex, incidence_adj_kernel, blocks_for(2 * m, th), th, 0, tu, tv, 2 * m, inc,
+                         adj);
+        }
+    }
+#define FAMST_GRADN(GV)                                                                         \
+    FAMST_LAUNCH(ex, grad_narrow_kernel<GV>, blocks_for(n * GV, th), th, 0, X, n, d, off, adj, gW, \
+                 gX, ex.dstatus)
+#define FAMST_GRAD(XRV, WIDEV)                                                                  \
+    FAMST_LAUNCH(ex, (grad_rows_kernel<XRV, WIDEV>),                                            \
+                 blocks_for((n + GRAD_V - 1) / GRAD_V * 32, th), th, 0, X, n, d, off, adj, gW, gX, \
+                 ex.dstatus)
+    if (d <= 4) FAMST_GRADN(4);
+    else if (d <= 8) FAMST_GRADN(8);
+    else if (d <= 16) FAMST_GRADN(16);
+    else if (d <= 32) FAMST_GRAD(1, false);
+    else if (d <= 64) FAMST_GRAD(2, false);
+    else if (d <= 128) FAMST_GRAD(4, false);
+    else if (d <= 256) FAMST_GRAD(8, false);
+    else FAMST_GRAD(8, true);
+#undef FAMST_GRADN
+#undef FAMST_GRAD
     return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
 }
 

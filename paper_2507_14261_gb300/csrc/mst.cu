@@ -243,41 +243,59 @@ __device__ void block_sum2(double &a, double &b) {
     b = sb[0];
 }
 
+// The FP64 value of a float without the conversion unit: the FP64 pipe (two
+// lanes an SM here) bounds the lengths below, and conversions go through it.
+// Normal numbers only need their exponent rebased and their fields moved;
+// zeros and subnormals take the instruction.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f), e = b & 0x7f800000u;
+    if (e == 0u) return double(f);
+    return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)),
+                            int(b << 29));
+}
+
+// FP64 length of every edge: p = fma(x_t - y_t, x_t - y_t, p) over t = 0 ..
+// d - 1. One thread per edge. (The sums over edges are a separate pass, so
+// that a small tree still fills the chip: 2k x 16, 47 us in one block.)
 template <int VEC>
-__global__ void weight_partial_kernel(const float *__restrict__ X, int d,
-                                      const int32_t *__restrict__ tu,
-                                      const int32_t *__restrict__ tv,
-                                      const float *__restrict__ tw, int64_t m,
-                                      double *__restrict__ part) {
+__global__ void edge_len64_kernel(const float *__restrict__ X, int d,
+                                  const int32_t *__restrict__ tu, const int32_t *__restrict__ tv,
+                                  int64_t m, double *__restrict__ len) {
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= m) return;
+    const float *a = X + int64_t(tu[e]) * d, *b = X + int64_t(tv[e]) * d;
+    double p = 0.0;
+    if constexpr (VEC == 4) {
+        const float4 *a4 = reinterpret_cast<const float4 *>(a);
+        const float4 *b4 = reinterpret_cast<const float4 *>(b);
+#pragma unroll 2
+        for (int q = 0; q < d / 4; ++q) {
+            const float4 x = __ldg(a4 + q), y = __ldg(b4 + q);
+            const double d0 = widen(x.x) - widen(y.x), d1 = widen(x.y) - widen(y.y);
+            const double d2 = widen(x.z) - widen(y.z), d3 = widen(x.w) - widen(y.w);
+            p = fma(d0, d0, p);
+            p = fma(d1, d1, p);
+            p = fma(d2, d2, p);
+            p = fma(d3, d3, p);
+        }
+    } else {
+        for (int t = 0; t < d; ++t) {
+            const double dl = widen(a[t]) - widen(b[t]);
+            p = fma(dl, dl, p);
+        }
+    }
+    len[e] = sqrt(p);
+}
+
+__global__ void weight_partial_kernel(const float *__restrict__ tw, const double *__restrict__ len,
+                                      int64_t m, double *__restrict__ part) {
     int64_t base = int64_t(blockIdx.x) * WR_TILE + int64_t(threadIdx.x) * WR_IPT;
     double s32 = 0.0, s64 = 0.0;
     for (int r = 0; r < WR_IPT; ++r) {
         int64_t e = base + r;
         if (e >= m) break;
         s32 += double(tw[e]);
-        if (X) {
-            const float *a = X + int64_t(tu[e]) * d, *b = X + int64_t(tv[e]) * d;
-            double p = 0.0;
-            if constexpr (VEC == 4) {   // the same sum, 16-byte loads
-                const float4 *a4 = reinterpret_cast<const float4 *>(a);
-                const float4 *b4 = reinterpret_cast<const float4 *>(b);
-                for (int q = 0; q < d / 4; ++q) {
-                    const float4 x = __ldg(a4 + q), y = __ldg(b4 + q);
-                    const double d0 = double(x.x) - double(y.x), d1 = double(x.y) - double(y.y);
-                    const double d2 = double(x.z) - double(y.z), d3 = double(x.w) - double(y.w);
-                    p = fma(d0, d0, p);
-                    p = fma(d1, d1, p);
-                    p = fma(d2, d2, p);
-                    p = fma(d3, d3, p);
-                }
-            } else {
-                for (int t = 0; t < d; ++t) {
-                    double dl = double(a[t]) - double(b[t]);
-                    p = fma(dl, dl, p);
-                }
-            }
-            s64 += sqrt(p);
-        }
+        if (len) s64 += len[e];
     }
     block_sum2(s32, s64);
     if (threadIdx.x == 0) {
@@ -746,7 +764,7 @@ famst_status boruvka(const Exec &ex, Arena &ar, int64_t n, const int32_t *nbr, c
 }
 
 size_t tree_weight_workspace(int64_t m) {
-    return align256(size_t((m + WR_TILE - 1) / WR_TILE + 1) * 16);
+    return align256(size_t((m + WR_TILE - 1) / WR_TILE + 1) * 16) + align256(size_t(m) * 8);
 }
 
 famst_status tree_weight(const Exec &ex, Arena &ar, const float *X, int d, bool vec4,
@@ -756,12 +774,16 @@ famst_status tree_weight(const Exec &ex, Arena &ar, const float *X, int d, bool 
     if (nb == 0) nb = 1;
     double *part = ar.take<double>(size_t(nb) * 2);
     if (!part) return FAMST_ERR_OOM;
-    if (vec4)
-        FAMST_LAUNCH(ex, weight_partial_kernel<4>, unsigned(nb), WR_NT, 0, X, d, tu, tv, tw, m,
-                     part);
-    else
-        FAMST_LAUNCH(ex, weight_partial_kernel<1>, unsigned(nb), WR_NT, 0, X, d, tu, tv, tw, m,
-                     part);
+    double *len = nullptr;
+    if (X && m > 0) {
+        len = ar.take<double>(size_t(m));
+        if (!len) return FAMST_ERR_OOM;
+        if (vec4)
+            FAMST_LAUNCH(ex, edge_len64_kernel<4>, blocks_for(m, 128), 128, 0, X, d, tu, tv, m, len);
+        else
+            FAMST_LAUNCH(ex, edge_len64_kernel<1>, blocks_for(m, 128), 128, 0, X, d, tu, tv, m, len);
+    }
+    FAMST_LAUNCH(ex, weight_partial_kernel, unsigned(nb), WR_NT, 0, tw, len, m, part);
     FAMST_LAUNCH(ex, weight_final_kernel, 1, WR_NT, 0, part, nb, W_dev);
     return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
 }

@@ -376,6 +376,9 @@ famst_status knn_stage(famst_ctx *ctx, Arena &ar, const float *X, int64_t n, int
             return st;
         }
         *uncert = n;
+    } else if (ctx->prune && knn_fp32_prunes(n, d, k, vec4_ok(X, d))) {
+        return knn_tc(ex, ar, X, n, d, k, false, true, nbr, dist, ctx->pinned + PIN_KNN, uncert,
+                      nullptr, true, nullptr, false, true);
     }
     return knn_fp32(ex, ar, X, n, d, k, nullptr, 0, n, nbr, dist);
 }
@@ -385,7 +388,10 @@ size_t knn_stage_ws(famst_ctx *ctx, int64_t n, int32_t d, int32_t k, int32_t pre
     if (prec != FAMST_PREC_FP32 && knn_tc_supported(n, d, k, prec == FAMST_PREC_BF16X3, f8))
         return knn_tc_workspace(n, d, k, prec == FAMST_PREC_BF16X3, ctx->num_sms,
                                 !f8 && ctx->prune != 0 && prune_supported(n, d, k, true), f8);
-    return knn_fp32_workspace(n, d, k, n, ctx->num_sms);
+    const size_t plain = knn_fp32_workspace(n, d, k, n, ctx->num_sms);
+    if (prec == FAMST_PREC_FP32 && ctx->prune && knn_fp32_prunes(n, d, k, true))
+        return std::max(plain, knn_tc_workspace(n, d, k, false, ctx->num_sms, true, false));
+    return plain;
 }
 
 // Workspace of Phases 2-3 + MST (slot 1) for m inter-component edges.

@@ -504,7 +504,10 @@ famst_status fallback_rows_batched(const Exec &ex, const float *Xc, int ld, cons
 famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d, int k, bool x3,
                     bool vec4, int32_t *nbr, float *dist, int32_t *pinned_host,
                     int64_t *uncertified, const int32_t *colcomp = nullptr, bool prune = false,
-                    int64_t *tiles_visited = nullptr, bool f8 = false);
+                    int64_t *tiles_visited = nullptr, bool f8 = false, bool f32 = false);
+// FP32 tiles over the pruned lists (knn_tc with f32 = true) where the
+// points are many enough to pay for the partition
+bool knn_fp32_prunes(int64_t n, int d, int k, bool vec4);
 
 // prune.cu
 // Tile pruning of Phase 1: locality partition (pivot cells), ball bounds,
@@ -519,12 +522,27 @@ struct PruneOut {
     int32_t *nitems = nullptr;      // device: work items in tab (<= nq + PRUNE_SPLIT_SLOTS)
     int32_t *splitq = nullptr;      // device: per split query tile (q, first slot, parts)
     int32_t *nsplit = nullptr;      // device: split query tiles
+    int32_t *off = nullptr;         // per query tile: its range of klist (nq + 1)
     float *skipQ = nullptr;         // per query tile
     float *Xs = nullptr;            // the points in sorted order (FP32, n x d)
     float *tau_row = nullptr;       // per sorted row: upper bound on its k-th neighbour distance
     int32_t *visited = nullptr;     // device: number of visited (query, key) tile pairs
     int64_t nq = 0, nk = 0;
 };
+// knn_fp32.cu on the pruning's lists: the FP32 tiles for every row, and the
+// exact distances of single rows (positions in the cell order, with the k-th
+// key of their candidates) over the keys their tile's list holds; a row that
+// a skipped tile could still reach is appended to fails (nfails on the device)
+size_t knn_fp32_pruned_workspace(int64_t n, int k, int64_t nq_tiles);
+famst_status knn_fp32_pruned(const Exec &ex, Arena &ar, const float *X, int64_t n, int d, int k,
+                             const PruneOut &P, int32_t *nbr, float *dist);
+size_t visited_rows_workspace(int64_t nrows);
+famst_status visited_rows(const Exec &ex, Arena &ar, const PruneOut &P, int64_t n, int d, int k,
+                          const int32_t *rows, const uint64_t *kth0, int64_t nrows, int32_t *nbr,
+                          float *dist, int32_t *fails, int32_t *nfails);
+famst_status exact_rows(const Exec &ex, const float *X, int64_t n, int d, int k,
+                        const int32_t *rows, const int32_t *count, int64_t max_rows,
+                        const int32_t *colcomp, int32_t *nbr, float *dist);
 int prune_pivots(int64_t n);      // evenly spaced pivots
 int prune_extra(int64_t n);       // pivots added by each of the two coverage passes
 int prune_pivots_max(int64_t n);

@@ -61,6 +61,7 @@ constexpr int BK = 64;           // K elements per stage (one 128-byte swizzle a
 constexpr int A_BLOCK = BM * BK * 2;   // 16 KB
 constexpr int B_BLOCK = BN * BK * 2;   // 32 KB
 constexpr int CAPB = 24;         // staged candidates per row (flush check every 16 columns)
+constexpr int VISITED_ROWS_SHARE = 32;   // uncertified rows redone one by one: up to n / this
 constexpr int TC_THREADS_MAX = 64 + 32 * 8;   // producer, MMA issuer, up to 8 epilogue warps
 
 // ------------------------------------------------------------ PTX helpers
@@ -909,10 +910,9 @@ __global__ void fill_inf_kernel(float *p, int64_t from, int64_t to) {
 // score s~(y) = ||y'||^2 - 2 x'.y' (rounded) with s~ <= ||x' - y'||^2 -
 // ||x'||^2 + E <= (tau_r + c)^2 - xn2 (1 - (d+1) u) + E, where c bounds the
 // centring rounding and E the tile's score error (the certificate's terms).
-// Written over tau_row in place.
-__global__ void thr0_kernel(float *__restrict__ tau_row, const float *__restrict__ xn2s,
+__global__ void thr0_kernel(const float *__restrict__ tau_row, const float *__restrict__ xn2s,
                             int64_t n, int d, const unsigned *__restrict__ ymax_bits,
-                            double eps_dot) {
+                            double eps_dot, float *__restrict__ thr0) {
     const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const double u24 = 1.0 / 16777216.0;
@@ -922,7 +922,7 @@ __global__ void thr0_kernel(float *__restrict__ tau_row, const float *__restrict
                      2.0 * u24 * (ym * ym + 2.0 * xn * ym) * 1.01 + 1e-30;
     const double t = (double(tau_row[r]) + 1.02 * u24 * (xn + ym)) * (1.0 + 0x1p-20);
     const double thr = t * t - xn2 * (1.0 - (d + 1) * u24 * 1.02) + E;
-    tau_row[r] = __double2float_ru(thr + (thr >= 0.0 ? thr : -thr) * 0x1p-20 + 1e-30);
+    thr0[r] = __double2float_ru(thr + (thr >= 0.0 ? thr : -thr) * 0x1p-20 + 1e-30);
 }
 
 // ------------------------------------------------------------- rerank
@@ -951,7 +951,8 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
                                            int lane,
                                            int32_t *__restrict__ nbr_row,
                                            float *__restrict__ dist_row,
-                                           const int32_t *__restrict__ idmap = nullptr) {
+                                           const int32_t *__restrict__ idmap = nullptr,
+                                           uint64_t *kth_out = nullptr) {
     constexpr int KP = KC - 1;
     uint64_t key[2];
     if constexpr (XR > 0) {
@@ -1078,6 +1079,7 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
     // k-th key (index k-1)
     const int kh = (k - 1) >> 5, kl = (k - 1) & 31;
     uint64_t kth = __shfl_sync(0xffffffffu, kh ? key[1] : key[0], kl);
+    if (kth_out) *kth_out = kth;
     bool cert = false;
     if (lane == 0) {
         const double u24c = 1.0 / 16777216.0;
@@ -1150,16 +1152,22 @@ __global__ void __launch_bounds__(256, 5) rerank_sorted_kernel(const float *__re
                                      const unsigned *__restrict__ ymax_bits, CertConst cc,
                                      int32_t *__restrict__ nbr, float *__restrict__ dist,
                                      int32_t *__restrict__ fail_rows,
+                                     uint64_t *__restrict__ fail_kth,
                                      int32_t *__restrict__ fail_count) {
     const int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r >= n) return;
     const int64_t i = perm[r];
+    uint64_t kth;
     const bool cert = rerank_row<VEC, KC, XR>(Xs, d, d, d, Xs + r * d, k, cand + r * (KC - 1),
                                           splus[r], skipQ[r / BM], xnorm2[i],
                                           __uint_as_float(*ymax_bits), cc.eps_dot, lane,
-                                          nbr + i * k, dist + i * k, perm);
-    if (!cert && lane == 0) fail_rows[atomicAdd(fail_count, 1)] = int32_t(i);
+                                          nbr + i * k, dist + i * k, perm, &kth);
+    if (!cert && lane == 0) {
+        const int s = atomicAdd(fail_count, 1);
+        fail_rows[s] = int32_t(r);   // the position in the cell order
+        fail_kth[s] = kth;
+    }
 }
 
 __device__ __forceinline__ int cloud_of(const long long *__restrict__ off, int B, long long v) {
@@ -1424,6 +1432,9 @@ size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prun
         b += align256(size_t(K) * 4) + align256(size_t(K) * p.kh * 2) +
              align256(size_t(Kpad + BN) * 4) * 2 + align256(size_t(n) * 4) * 2;
         b += prune_workspace(n, d, p.kh, p.kc - 1, p.nq_tiles, p.nk_tiles);
+        b += align256(size_t(n) * 4) * 2 + align256(size_t(n) * 8) + 256;   // thr0, failed rows
+        b += std::max(knn_fp32_pruned_workspace(n, k, p.nq_tiles),
+                      visited_rows_workspace(n / VISITED_ROWS_SHARE));
     }
     b += align256(size_t(n) * p.kh * (f8 ? 1 : 2));        // operand rows
     if (f8) b += align256(size_t(p.nk_tiles) * BN * 4);    // per-row scales
@@ -1437,17 +1448,29 @@ size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prun
     return b;
 }
 
+// The partition takes about 1.1 ms whatever the size (a dozen
+// synchronisations and sorts); the unpruned tiles take about 55 fs per pair
+// and coordinate plus 3.3 ps per pair. The line is at 1.9 ms of those: 16384
+// x 128 in 20 clusters 3.05 ms unpruned, 1.31 ms pruned; 8192 x 128 1.08 ms
+// unpruned; a cloud without structure loses the partition's time (50000 x
+// 100: 20.7 -> 22.8 ms).
+bool knn_fp32_prunes(int64_t n, int d, int k, bool vec4) {
+    return double(n) * double(n) * (d + 60.0) >= 3.5e10 && prune_supported(n, d, k, vec4) &&
+           knn_tc_supported(n, d, 1, false);
+}
+
 famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d, int k, bool x3,
                     bool vec4, int32_t *nbr, float *dist, int32_t *pinned_host,
                     int64_t *uncertified, const int32_t *colcomp, bool prune,
-                    int64_t *tiles_visited, bool f8) {
+                    int64_t *tiles_visited, bool f8, bool f32) {
     if (f8) {   // single E4M3 products, no tile pruning, no component mask
         x3 = false;
         prune = false;
         if (colcomp) return FAMST_ERR_UNSUPPORTED;
     }
-    TcPlan p = tc_plan(n, d, k, x3, true, f8);
-    if (p.stages < 2 || k + 1 > 64) return FAMST_ERR_UNSUPPORTED;
+    // f32: the tensor tiles only place the points in pivot cells
+    TcPlan p = tc_plan(n, d, f32 ? 1 : k, x3, true, f8);
+    if (p.stages < 2 || (k + 1 > 64 && !f32)) return FAMST_ERR_UNSUPPORTED;
     // operand rows: BF16 (kh elements) or E4M3 bytes (kh bytes) with per-row scales
     __nv_bfloat16 *H = f8 ? nullptr : ar.take<__nv_bfloat16>(size_t(n) * p.kh);
     uint8_t *Q = f8 ? ar.take<uint8_t>(size_t(n) * p.kh) : nullptr;
@@ -1550,13 +1573,27 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
                              pinned_host + 2, &P);
         if (st != FAMST_OK) return st;
     }
+    if (f32) {
+        *uncertified = 0;
+        if (tiles_visited) *tiles_visited = p.nq_tiles * p.nk_tiles;
+        return use_prune ? knn_fp32_pruned(ex, ar, X, n, d, k, P, nbr, dist)
+                         : FAMST_ERR_UNSUPPORTED;
+    }
     // candidates of the tensor pass: directly in cand / splus, or (pruned)
     // in sorted order first
     int32_t *cand_t = cand;
     float *splus_t = splus;
     int32_t *side_j = nullptr;   // candidates of the parts of split lists
     float *side_s = nullptr, *side_sp = nullptr;
+    float *thr0 = nullptr;       // start thresholds
+    uint64_t *fail_kth = nullptr;
+    int32_t *fails2 = nullptr, *nfail2 = nullptr;
     if (use_prune) {
+        thr0 = ar.take<float>(size_t(n));
+        fail_kth = ar.take<uint64_t>(size_t(n));
+        fails2 = ar.take<int32_t>(size_t(n));
+        nfail2 = ar.take<int32_t>(1);
+        if (!thr0 || !fail_kth || !fails2 || !nfail2) return FAMST_ERR_OOM;
         cand_t = ar.take<int32_t>(size_t(n) * (p.kc - 1));
         splus_t = ar.take<float>(size_t(n));
         side_j = ar.take<int32_t>(size_t(PRUNE_SPLIT_SLOTS) * BM * (p.kc - 1));
@@ -1600,10 +1637,10 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     cc.d_plus = double(d) + 4.0;
     if (use_prune)
         FAMST_LAUNCH(ex, thr0_kernel, unsigned((n + 255) / 256), 256, 0, P.tau_row, P.nys, n, d,
-                     ymax, cc.eps_dot);
+                     ymax, cc.eps_dot, thr0);
     TcArgs a{int(n), int(p.nk_tiles), p.nkb, int(x3), p.stages, use_prune ? P.nys : ny, cand_t,
              splus_t, ex.dstatus, use_prune ? P.tab : nullptr, cpad,
-             use_prune ? P.klist : nullptr, 0, p.epi, rscale, use_prune ? P.tau_row : nullptr};
+             use_prune ? P.klist : nullptr, 0, p.epi, rscale, thr0};
     // one CTA per work item: the pruned tiles' key lists differ in length,
     // and a static round-robin over persistent CTAs measured slower here.
     // Pruned lists come as work items, long ones split into parts; the grid
@@ -1663,7 +1700,7 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         if (use_prune)                                                                           \
             FAMST_LAUNCH(ex, (rerank_sorted_kernel<V, KCV, XRV>), rgrid, 256, 0, P.Xs, n, d, k,  \
                          cand_t, splus_t, P.skipQ, P.perm, xn2, ymax, cc, nbr, dist, fail_rows,  \
-                         fail_count);                                                            \
+                         fail_kth, fail_count);                                                            \
         else                                                                                     \
             FAMST_LAUNCH(ex, (rerank_kernel<V, KCV, XRV>), rgrid, 256, 0, X, n, d, k, cand,      \
                          splus, nullptr, xn2, ymax, cc, nbr, dist, fail_rows, fail_count);       \
@@ -1694,7 +1731,21 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     const int32_t nfail = *pinned_host;
     *uncertified = nfail;
     if (tiles_visited) *tiles_visited = use_prune ? int64_t(pinned_host[1]) : p.nq_tiles * p.nk_tiles;
-    if (nfail > 0) {
+    if (nfail > 0 && use_prune) {
+        // few rows: exact over their tile's list, read for each row by
+        // itself; many: the FP32 tiles over all lists, which share a key
+        // among 64 rows
+        famst_status st;
+        if (nfail <= n / VISITED_ROWS_SHARE) {
+            if (cudaMemsetAsync(nfail2, 0, 4, ex.stream) != cudaSuccess) return FAMST_ERR_CUDA;
+            st = visited_rows(ex, ar, P, n, d, k, fail_rows, fail_kth, nfail, nbr, dist, fails2, nfail2);
+            if (st == FAMST_OK)
+                st = exact_rows(ex, X, n, d, k, fails2, nfail2, nfail, nullptr, nbr, dist);
+        } else {
+            st = knn_fp32_pruned(ex, ar, X, n, d, k, P, nbr, dist);
+        }
+        if (st != FAMST_OK) return st;
+    } else if (nfail > 0) {
         famst_status st = knn_fp32(ex, ar, X, n, d, k, fail_rows, 0, nfail, nbr, dist, colcomp);
         if (st != FAMST_OK) return st;
     }

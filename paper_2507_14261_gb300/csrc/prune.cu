@@ -935,6 +935,7 @@ famst_status prune_partition(const Exec &ex, Arena &ar, const float *X, int d, i
     out->nitems = nitems;
     out->splitq = splitq;
     out->nsplit = nsplit;
+    out->off = off;
     out->skipQ = skipQ;
     out->Xs = Xs;
     out->tau_row = tau_row;

@@ -17,9 +17,9 @@
 // load feeds four coordinates: 16 loads per 256 packed instructions, and two
 // blocks of four warps fit an SM, one computing while the other selects or
 // waits at a barrier. 50021 x 100, k = 16: 59.5 ms with one block of eight
-// warps per SM, scalar arithmetic and one selecting thread per list; 20.7 ms
-// (1.2e13 coordinate pairs/s, 62% of the pipe's 1.95e13) with these tiles,
-// and 1.7 ms where the cloud has 20 clusters and the pruned lists are used.
+// warps per SM, scalar arithmetic and one selecting thread per list; 18.2 ms
+// (1.37e13 coordinate pairs/s, 70% of the pipe's 1.95e13) with these tiles,
+// and 1.6 ms where the cloud has 20 clusters and the pruned lists are used.
 //
 // Selection is fused: a thread compares its 64 values with their rows'
 // thresholds (the k'-th kept, or a bound the caller knows in advance) in
@@ -352,55 +352,63 @@ __global__ void __launch_bounds__(NT, 2) knn_fp32_kernel(TileArgs A) {
         // survivors: query ty + 8 i, key tx + 16 j; bit 8 i + j of `pend`
         // marks a value not yet queued
         const int key0 = key0_of(tile_begin + s / nchunks);
-        float pv[8][8];
+        float pv[64];
         unsigned long long pend = 0ull;
-        auto compare = [&](bool first) {
-            unsigned long long keep = 0ull;
+        auto compare = [&](unsigned long long among) {
+            pend = 0ull;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float thr = thr_s[ty + 8 * i];
+                float mn = pv[8 * i];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (pv[i][j] <= thr) keep |= 1ull << (8 * i + j);
+                for (int j = 1; j < 8; ++j) mn = fminf(mn, pv[8 * i + j]);
+                if (mn <= thr) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (pv[8 * i + j] <= thr) pend |= 1ull << (8 * i + j);
+                }
             }
-            pend = first ? keep : pend & keep;
+            pend &= among;
         };
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) pv[i][j] = f2_hsum(acc[i][j]);
-        compare(true);
-        while (__syncthreads_or(pend != 0ull)) {
-            if (pend) {
+            for (int j = 0; j < 8; ++j) pv[8 * i + j] = f2_hsum(acc[i][j]);
+        compare(~0ull);
+        const bool last = s + 1 == nsteps;
+        while (true) {
+            const bool more = __syncthreads_or(pend != 0ull);
+            if (!more && !last) break;
+            // one survivor per thread and turn (one copy of the code: unrolled
+            // over the 64 values it does not fit the instruction cache)
+            unsigned long long left = 0ull;
+#pragma unroll 1
+            while (pend) {
+                const int b = __ffsll(pend) - 1;
+                pend &= pend - 1ull;
+                float v[32];   // the value at b, by its bits
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (!((pend >> (8 * i)) & 0xffull)) continue;
-                    const int row = ty + 8 * i;
+                for (int x = 0; x < 32; ++x) v[x] = (b & 1) ? pv[2 * x + 1] : pv[2 * x];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (!((pend >> (8 * i + j)) & 1ull)) continue;
-                        const int jj = key0 + tx + 16 * j;
-                        bool in = jj < n && jj != qid_s[row];
-                        if (A.colcomp && in) in = A.colcomp[jj] != comp_s[row];
-                        int slot = 0;
-                        if (in) {
-                            slot = atomicAdd(&qcnt[row], 1);
-                            if (slot < QCAP)
-                                Q[row * QCAP + slot] = nb_key(__fsqrt_rn(pv[i][j]), uint32_t(jj));
-                        }
-                        if (slot < QCAP) pend &= ~(1ull << (8 * i + j));
-                    }
-                }
+                for (int w = 1; w < 6; ++w)
+#pragma unroll
+                    for (int x = 0; x < (32 >> w); ++x)
+                        v[x] = (b >> w) & 1 ? v[2 * x + 1] : v[2 * x];
+                const int row = ty + (b & ~7), jj = key0 + tx + 16 * (b & 7);
+                bool in = jj < n && jj != qid_s[row];
+                if (A.colcomp && in) in = A.colcomp[jj] != comp_s[row];
+                if (!in) continue;
+                const int slot = atomicAdd(&qcnt[row], 1);
+                if (slot < QCAP) Q[row * QCAP + slot] = nb_key(__fsqrt_rn(v[0]), uint32_t(jj));
+                else left |= 1ull << b;
             }
             __syncthreads();
-            flush(FLUSH_AT);
+            flush(more ? FLUSH_AT : 1);   // the last tile ends with every queue merged
             __syncthreads();
-            if (pend) compare(false);
+            if (!more) break;
+            if (left) compare(left);
         }
     }
-    __syncthreads();
-    flush(1);
-    __syncthreads();
     const int rows = min(QM, nq - qbase);
     for (int x = tid; x < rows * kp; x += NT) {
         const uint64_t v = L[x];

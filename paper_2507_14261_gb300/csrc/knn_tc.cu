@@ -50,6 +50,7 @@
 
 #include "famst_internal.cuh"
 #include "mbarrier.cuh"
+#include "tcgen05.cuh"
 #include "topk_merge.cuh"
 
 namespace famst {
@@ -57,123 +58,12 @@ namespace {
 
 constexpr int BM = 128;          // query rows per CTA (TMEM lanes)
 constexpr int BN = 256;          // keys per tile (accumulator columns)
-constexpr int BK = 64;           // K elements per stage (one 128-byte swizzle atom)
+constexpr int BK = TC_BK;        // K elements per stage (one 128-byte swizzle atom)
 constexpr int A_BLOCK = BM * BK * 2;   // 16 KB
 constexpr int B_BLOCK = BN * BK * 2;   // 32 KB
 constexpr int CAPB = 24;         // staged candidates per row (flush check every 16 columns)
 constexpr int VISITED_ROWS_SHARE = 32;   // uncertified rows redone one by one: up to n / this
 constexpr int TC_THREADS_MAX = 64 + 32 * 8;   // producer, MMA issuer, up to 8 epilogue warps
-
-// ------------------------------------------------------------ PTX helpers
-
-// Bounded wait for the phase of parity `parity` to complete. Returns false
-// if the CTA aborted or the time limit expired (then it raises the abort).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                          int *status) {
-    if (mbar_try_wait(bar, parity)) return true;
-    uint64_t t0 = globaltimer();
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (globaltimer() - t0 > WAIT_NS) {
-            *abort_flag = 1;
-            set_status(status, STATUS_LOOP_LIMIT);
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x,
-                                            int y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(slot)),
-                 "r"(ncols)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-                 : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 (BF16 inputs, FP32 accumulate)
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// arrive on `bar` once every tcgen05 op issued so far by this thread is done
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld_wait16(uint32_t (&r)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
-                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
-                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-                 :
-                 : "memory");
-}
-__device__ __forceinline__ void epilogue_bar(int nthreads) {  // the epilogue warps only
-    asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
-}
-// The same barrier, returning whether any epilogue thread passed p = true.
-__device__ __forceinline__ bool epilogue_bar_any(int nthreads, bool p) {
-    int r;
-    asm volatile(
-        "{\n\t.reg .pred pi, po;\n\tsetp.ne.s32 pi, %1, 0;\n\t"
-        "bar.red.or.pred po, 1, %2, pi;\n\tselp.s32 %0, 1, 0, po;\n\t}"
-        : "=r"(r)
-        : "r"(int(p)), "r"(nthreads)
-        : "memory");
-    return r != 0;
-}
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows
-// of 128 bytes, 8-row groups 1024 bytes apart (SBO), version 1.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= uint64_t((saddr & 0x3FFFFu) >> 4);   // start address
-    d |= uint64_t(1) << 16;                    // leading byte offset (unused with SW128 K-major)
-    d |= uint64_t(1024 >> 4) << 32;            // stride byte offset
-    d |= uint64_t(1) << 46;                    // descriptor version
-    d |= uint64_t(2) << 61;                    // SWIZZLE_128B
-    return d;
-}
-// Instruction descriptor, kind::f16: D F32, A/B BF16, both K-major.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) |
-           (uint32_t(M >> 4) << 24);
-}
 
 // Instruction descriptor, kind::f8f6f4: D F32, A/B E4M3 (format 0), both K-major.
 __host__ __device__ constexpr uint32_t idesc_e4m3(int M, int N) {
@@ -1336,36 +1226,6 @@ __global__ void cloud_mean_kernel(const float *__restrict__ Xc, int ld,
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                             &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
-// 2-D map over row-major operand rows of `cols` elements: BF16 (boxes of 64
-// elements) or, with f8, bytes (boxes of 128); 128 bytes per box row either way
-bool make_map(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int box_rows,
-              bool f8 = false) {
-    auto fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t gdim[2] = {cuuint64_t(cols), cuuint64_t(rows)};
-    cuuint64_t gstride[1] = {cuuint64_t(cols) * (f8 ? 1 : 2)};
-    cuuint32_t box[2] = {cuuint32_t(f8 ? 2 * BK : BK), cuuint32_t(box_rows)};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(m, f8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                    const_cast<void *>(base), gdim, gstride,
-                    box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
 // keep the better of two top-1 results (the second with ids offset by k0)
 __global__ void top1_merge_kernel(const int32_t *__restrict__ c2, const float *__restrict__ s2,
                                   int k0, int64_t n, int32_t *__restrict__ c,
@@ -1449,13 +1309,13 @@ size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prun
 }
 
 // The partition takes about 1.1 ms whatever the size (a dozen
-// synchronisations and sorts); the unpruned tiles take about 55 fs per pair
-// and coordinate plus 3.3 ps per pair. The line is at 1.9 ms of those: 16384
-// x 128 in 20 clusters 3.05 ms unpruned, 1.31 ms pruned; 8192 x 128 1.08 ms
-// unpruned; a cloud without structure loses the partition's time (50000 x
-// 100: 20.7 -> 22.8 ms).
+// synchronisations and sorts); the unpruned tiles take about 65 fs per pair
+// and coordinate plus 1.2 ps per pair. The line is at 1.6 ms of those: 16384
+// x 128 in 20 clusters 2.66 ms unpruned, 1.27 ms pruned; 32768 x 16 2.45 and
+// 1.32 ms; 8192 x 128 0.88 ms unpruned; a cloud without structure loses the
+// partition's time (50000 x 100: 18.2 -> 20.7 ms).
 bool knn_fp32_prunes(int64_t n, int d, int k, bool vec4) {
-    return double(n) * double(n) * (d + 60.0) >= 3.5e10 && prune_supported(n, d, k, vec4) &&
+    return double(n) * double(n) * (d + 18.0) >= 2.5e10 && prune_supported(n, d, k, vec4) &&
            knn_tc_supported(n, d, 1, false);
 }
 

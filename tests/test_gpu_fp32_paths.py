@@ -53,7 +53,7 @@ def test_plain_tiles(orc, ctx, n, d, k):
 ])
 def test_pruned_tiles(ctx, name, make, k):
     X = torch.from_numpy(make()).cuda()
-    assert X.shape[0] ** 2 * (X.shape[1] + 60) >= 3.5e10   # large enough to be pruned
+    assert X.shape[0] ** 2 * (X.shape[1] + 18) >= 2.5e10   # large enough to be pruned
     pn, pd = _knn(ctx, X, k, "fp32", True)
     un, ud = _knn(ctx, X, k, "fp32", False)
     assert np.array_equal(pn, un) and np.array_equal(pd, ud)

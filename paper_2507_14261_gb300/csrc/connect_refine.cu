@@ -702,21 +702,22 @@ famst_status launch_refine(const Exec &ex, const float *X, int d, bool vec4, con
 }
 
 // Centre m for the BF16 rows: the mean of up to 256 evenly spaced rows (any
-// m is valid; the bounds use the actual fl(x - m)).
-__global__ void half_mean_kernel(const float *__restrict__ X, int64_t n, int d,
-                                 float *__restrict__ m) {
+// m is valid; the bounds use the actual fl(x - m)). One block per 32
+// coordinates, eight rows at a time (one block for all of them waited 34 us
+// for its chain of loads).
+__global__ void __launch_bounds__(256) half_mean_kernel(const float *__restrict__ X, int64_t n,
+                                                        int d, float *__restrict__ m) {
+    __shared__ float part[8][32];
     const int64_t S = n < 256 ? n : 256;
-    for (int t = threadIdx.x; t < d; t += blockDim.x) {
-        float s = 0.0f;
-        int64_t i = 0;
-        for (; i + 8 <= S; i += 8) {   // eight independent loads in flight
-            float v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = __ldg(X + ((i + q) * n / S) * d + t);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) s += v[q];
-        }
-        for (; i < S; ++i) s += __ldg(X + (i * n / S) * d + t);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int t = int(blockIdx.x) * 32 + lane;
+    float s = 0.0f;
+    if (t < d)
+        for (int64_t i = w; i < S; i += 8) s += __ldg(X + (i * n / S) * d + t);
+    part[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && t < d) {
+        for (int q = 1; q < 8; ++q) s += part[q][lane];
         m[t] = s / float(S);
     }
 }
@@ -866,7 +867,7 @@ famst_status half_rows(const Exec &ex, Arena &ar, const float *X, int64_t n, int
     float *n2 = ar.take<float>(size_t(n));
     float *m = ar.take<float>(size_t(d));
     if (!h || !eb || !n2 || !m) return FAMST_ERR_OOM;
-    FAMST_LAUNCH(ex, half_mean_kernel, 1, 256, 0, X, n, d, m);
+    FAMST_LAUNCH(ex, half_mean_kernel, unsigned((d + 31) / 32), 256, 0, X, n, d, m);
     FAMST_LAUNCH(ex, half_rows_kernel, unsigned((n * 32 + 255) / 256), 256, 0, X, n, d, ld, m, h,
                  eb, n2);
     out->h = h;

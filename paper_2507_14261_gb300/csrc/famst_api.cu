@@ -219,6 +219,19 @@ __global__ void max_i32_kernel(const int32_t *__restrict__ a, int64_t count, int
     if ((threadIdx.x & 31) == 0) atomicMax(out, mx);
 }
 
+// *open = 1 when a kNN edge joins two of the caller's components (ids out of
+// range are reported elsewhere)
+__global__ void check_closed_kernel(const int32_t *__restrict__ nbr, int64_t nk, int64_t n, int k,
+                                    const int32_t *__restrict__ comp, int32_t *open) {
+    int bad = 0;
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < nk;
+         e += int64_t(gridDim.x) * blockDim.x) {
+        const int v = nbr[e];
+        if (v >= 0 && int64_t(v) < n) bad |= comp[v] != comp[e / k];
+    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) *open = 1;
+}
+
 unsigned grid_cap(famst_ctx *ctx, int64_t count, int th) {
     int64_t g = (count + th - 1) / th;
     int64_t cap = int64_t(ctx->num_sms) * 8;
@@ -953,37 +966,58 @@ famst_status famst_refine(famst_ctx *ctx, const float *X, int64_t n, int32_t d,
     ST(check_nbr(ctx, nbr, n, k));
     Exec ex = exec_of(ctx);
     FAMST_LAUNCH(ex, check_ids_kernel, grid_cap(ctx, n, 256), 256, 0, comp, n, n, 0, ctx->dstatus);
-    ST(sync_status(ctx));
-    if (m > 0) {
-        FAMST_LAUNCH(ex, check_edges_kernel, unsigned((m + 255) / 256), 256, 0, eu, ev, eci, ecj,
-                     comp, m, n, ctx->dstatus);
-        ST(sync_status(ctx));
-    }
     *sweeps_out = 0;
     if (m == 0) {
+        ST(sync_status(ctx));
         *sweeps_out = 1;
         if (delta_hist) delta_hist[0] = 0;
         return FAMST_OK;
     }
+    // Labels that no kNN edge leaves (Algorithm 2's own): G[u] needs no test
+    // for the component, and the grouped scans of a build serve here too.
+    const bool v4 = vec4_ok(X, d);
+    const bool may_group = v4 && d >= 32 && d <= 256;
     Arena ar;
-    ST(ensure_ws(ctx, 1, align256(size_t(n + 1) * 4) + align256(size_t(n) * k * 4) +
-                             reverse_csr_workspace(n, k) + align256(size_t(max_iters + 1) * 4) +
-                             refine_workspace(m) + 256,
-                 ar));
+    size_t ws = align256(size_t(n + 1) * 4) + align256(size_t(n) * k * 4) +
+                reverse_csr_workspace(n, k) + align256(size_t(max_iters + 1) * 4) +
+                refine_workspace(m) + 512;
+    if (may_group)
+        ws += align256(size_t(n) * 4) + align256(size_t(n + 1) * 4) + member_lists_workspace(n, n) +
+              half_rows_workspace(n, d) + glists_workspace(n, k) + refine_build_workspace(n, m);
+    ST(ensure_ws(ctx, 1, ws, ar));
+    int32_t *flags = ar.take<int32_t>(2);   // largest component index in E and comp; open labels
     int32_t *rev_off = ar.take<int32_t>(size_t(n + 1));
     int32_t *rev_src = ar.take<int32_t>(size_t(n) * k);
     int32_t *hist = ar.take<int32_t>(size_t(max_iters + 1));
+    CK(cudaMemsetAsync(flags, 0, 8, ctx->stream));
+    FAMST_LAUNCH(ex, check_edges_kernel, unsigned((m + 255) / 256), 256, 0, eu, ev, eci, ecj, comp,
+                 m, n, ctx->dstatus);
+    if (may_group) {
+        FAMST_LAUNCH(ex, check_closed_kernel, grid_cap(ctx, n * k, 256), 256, 0, nbr, n * k, n, k,
+                     comp, flags + 1);
+        FAMST_LAUNCH(ex, max_i32_kernel, grid_cap(ctx, n, 256), 256, 0, comp, n, flags);
+    } else {
+        FAMST_LAUNCH(ex, max_i32_kernel, grid_cap(ctx, m, 256), 256, 0, ecj, m, flags);
+    }
+    CK(cudaMemcpyAsync(ctx->pinned + PIN_T, flags, 8, cudaMemcpyDeviceToHost, ctx->stream));
+    ST(sync_status(ctx));
+    const int64_t t_e = int64_t(ctx->pinned[PIN_T]) + 1;
+    const bool grouped = may_group && ctx->pinned[PIN_T + 1] == 0;
     ST(reverse_csr(ex, ar, nbr, n, k, rev_off, rev_src));
     CK(cudaMemsetAsync(hist, 0, size_t(max_iters + 1) * 4, ctx->stream));
-    // number of components: one more than the largest component index in E
-    int32_t *tmax = ar.take<int32_t>(1);
-    CK(cudaMemsetAsync(tmax, 0, 4, ctx->stream));
-    FAMST_LAUNCH(ex, max_i32_kernel, grid_cap(ctx, m, 256), 256, 0, ecj, m, tmax);
-    CK(cudaMemcpyAsync(ctx->pinned + PIN_T, tmax, 4, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    const int64_t t_e = int64_t(ctx->pinned[PIN_T]) + 1;
-    ST(refine_edges(ex, ar, X, d, vec4_ok(X, d), nbr, k, rev_off, rev_src, comp, t_e, eu, ev, ew, eci, ecj,
-                    m, max_iters, hist));
+    if (grouped) {
+        int32_t *members = ar.take<int32_t>(size_t(n));
+        int32_t *comp_off = ar.take<int32_t>(size_t(n + 1));
+        ST(member_lists(ex, ar, comp, n, t_e, members, comp_off));
+        HalfRows hr;
+        ST(half_rows(ex, ar, X, n, d, &hr));
+        ST(refine_glists(ex, ar, nbr, n, k, rev_off, rev_src, &hr));
+        ST(refine_build(ex, ar, X, d, hr, members, n, eu, ev, ew, nullptr, m, max_iters, hist,
+                        nullptr, ctx->pinned + PIN_REF));
+    } else {
+        ST(refine_edges(ex, ar, X, d, v4, nbr, k, rev_off, rev_src, comp, t_e, eu, ev, ew, eci, ecj,
+                        m, max_iters, hist));
+    }
     famst_status s = sync_status(ctx);
     int32_t *hh = new (std::nothrow) int32_t[max_iters + 1];
     if (!hh) return fail(ctx, FAMST_ERR_OOM, "host");

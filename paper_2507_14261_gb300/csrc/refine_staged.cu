@@ -343,7 +343,8 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
                         const __nv_bfloat16 *__restrict__ H, const int32_t *__restrict__ members,
                         int64_t n, const int32_t *__restrict__ bstart,
                         const int4 *__restrict__ rec, unsigned long long *__restrict__ best,
-                        unsigned long long *__restrict__ evals_out, float aerr, float eps) {
+                        unsigned long long *__restrict__ evals_out, float aerr, float eps,
+                        float rel) {
     using S = Stage<NKS>;
     extern __shared__ __align__(128) char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -391,12 +392,15 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
                 const int idx = r0 + lane;
                 const bool valid = idx < deg;
                 int cand = -1;
-                float2 en = make_float2(inf, 0.0f);
+                float2 en = make_float2(0.0f, inf);   // absent: no pair passes the filter
                 if (valid) {
                     cand = __ldg(g.id + base + idx);
                     en = __ldg(g.en + base + idx);
                 }
                 const int nv = __popc(__ballot_sync(0xffffffffu, valid));
+                // the round's largest row error (non-negative floats order as integers)
+                const float ebm = __uint_as_float(
+                    __reduce_max_sync(0xffffffffu, __float_as_uint(en.x)));
                 s_en[lane] = en;
                 s_id[lane] = cand;
                 stage_rows<NKS>(H, cand, sbuf, lane);
@@ -426,61 +430,71 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
                             b1[ks] = has ? ldg_u32(hf + 16 * ks + 8 + 2 * t4) : 0u;
                         }
                     }
-                    float acc[2][4];
-                    round_dots<NKS>(sbuf, b0, b1, lane, acc);
                     // this lane holds the pairs (candidate 16 T + g4 + 8 (e2 >> 1),
-                    // task 2 t4 + (e2 & 1)) in acc[T][e2]
-                    float lo[2][4];
-                    float mh0 = inf, mh1 = inf;
+                    // task 2 t4 + (e2 & 1)) in acc[T][e2]; a short last round
+                    // leaves out the second tile
+                    float acc[2][4];
+                    round_dots<NKS>(sbuf, b0, b1, lane, acc, nv > 16);
+                    // bounds on the squared distance of the BF16 rows, p~ -+ A
+                    // (dist_bounds'); the row errors enter per task through
+                    // E = its own plus the round's largest, so that a pair
+                    // takes no square root
+                    float lo[2][4], nx[2], E[2], mh[2];
 #pragma unroll
-                    for (int T = 0; T < 2; ++T)
-#pragma unroll
-                        for (int e2 = 0; e2 < 4; ++e2) {
-                            const int ci = 16 * T + g4 + 8 * (e2 >> 1), tj = 2 * t4 + (e2 & 1);
-                            float hi = inf;
-                            lo[T][e2] = inf;
-                            if (ci < nv && tj < ntb) {
-                                const float2 ce = s_en[ci];
-                                const float4 ts = s_task[tj];
-                                dist_bounds(acc[T][e2], ts.z, ce.y, ts.y, ce.x, aerr, eps,
-                                            lo[T][e2], hi);
-                            }
-                            if (e2 & 1) mh1 = fminf(mh1, hi);
-                            else mh0 = fminf(mh0, hi);
-                        }
-                    // per task: the smallest upper bound over all candidates
-                    // (the lanes with the same t4)
-#pragma unroll
-                    for (int o = 4; o <= 16; o <<= 1) {
-                        mh0 = fminf(mh0, __shfl_xor_sync(0xffffffffu, mh0, o));
-                        mh1 = fminf(mh1, __shfl_xor_sync(0xffffffffu, mh1, o));
+                    for (int c = 0; c < 2; ++c) {
+                        const float4 ts = s_task[2 * t4 + c];
+                        nx[c] = ts.z;
+                        E[c] = __fadd_ru(ts.y, ebm);
+                        mh[c] = inf;
                     }
-                    const float bnd0 =
-                        2 * t4 < ntb
-                            ? __fmul_ru(fminf(mh0, key_w(s_best[2 * t4])), 1.0f + 0x1p-22f)
-                            : -inf;
-                    const float bnd1 =
-                        2 * t4 + 1 < ntb
-                            ? __fmul_ru(fminf(mh1, key_w(s_best[2 * t4 + 1])), 1.0f + 0x1p-22f)
-                            : -inf;
+#pragma unroll
+                    for (int T = 0; T < 2; ++T) {
+#pragma unroll
+                        for (int e2 = 0; e2 < 4; ++e2) lo[T][e2] = inf;
+                        if (T == 1 && nv <= 16) break;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const float ny = s_en[16 * T + g4 + 8 * h].y;
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                const float nn = __fadd_rn(nx[c], ny);
+                                const float pt = __fmaf_rn(-2.0f, acc[T][2 * h + c], nn);
+                                const float A = __fmaf_ru(nn, aerr, 1e-35f);
+                                lo[T][2 * h + c] = __fsub_rd(pt, A);
+                                mh[c] = fminf(mh[c], __fadd_ru(pt, A));
+                            }
+                        }
+                    }
+                    // per task: the smallest upper bound over all candidates
+                    // (the lanes with the same t4), and the largest lower bound
+                    // on p~ - A that a candidate at or below it can have
+                    float lim[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+#pragma unroll
+                        for (int o = 4; o <= 16; o <<= 1)
+                            mh[c] = fminf(mh[c], __shfl_xor_sync(0xffffffffu, mh[c], o));
+                        const float hi = __fmul_ru(__fadd_ru(__fsqrt_ru(mh[c]), E[c]), 1.0f + eps);
+                        const float bound =
+                            __fmul_ru(fminf(hi, key_w(s_best[2 * t4 + c])), 1.0f + 0x1p-22f);
+                        const float r = __fmaf_ru(bound, rel, E[c]);
+                        lim[c] = 2 * t4 + c < ntb ? __fmul_ru(r, r) : -inf;
+                    }
                     if (lane == 0) ctr += unsigned(nv * ntb);
                     __syncwarp();
                     // survivors, decided on canonical distances by the whole
                     // warp, up to four at a time; bit 4 T + e2 of `my` marks a
                     // surviving pair of this lane (one copy of the batch code).
+                    // (an absent candidate's lo is NaN or +inf, an absent task's lim -inf)
                     unsigned my = 0;
 #pragma unroll
                     for (int T = 0; T < 2; ++T)
 #pragma unroll
                         for (int e2 = 0; e2 < 4; ++e2)
-                            if (16 * T + g4 + 8 * (e2 >> 1) < nv && 2 * t4 + (e2 & 1) < ntb &&
-                                lo[T][e2] <= ((e2 & 1) ? bnd1 : bnd0))
-                                my |= 1u << (4 * T + e2);
+                            if (lo[T][e2] <= lim[e2 & 1]) my |= 1u << (4 * T + e2);
                     {
-                        int cnt = __popc(my);
-#pragma unroll
-                        for (int o = 16; o >= 1; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-                        if (lane == 1) ctr += unsigned(cnt);
+                        const unsigned cnt = __reduce_add_sync(0xffffffffu, __popc(my));
+                        if (lane == 1) ctr += cnt;
                     }
 #pragma unroll 1
                     while (true) {
@@ -582,6 +596,9 @@ float refine_aerr() {
 // canonical distance vs the exact one, generously: (d + 16) u
 float refine_eps(int d) { return float((d + 16) * std::ldexp(1.0, -24) * 1.1); }
 
+// at least 1 / (1 - eps)
+float refine_rel(int d) { return 1.0f + 2.0f * refine_eps(d); }
+
 template <class K>
 famst_status occupancy_grid(const Exec &ex, K *fn, int threads, int smem, int64_t want,
                             unsigned *grid) {
@@ -623,7 +640,7 @@ famst_status launch_group_t(const Exec &ex, const float *X, int d, const HalfRow
         occupancy_grid(ex, fn, S::WARPS * 32, S::SMEM, (n + S::WARPS - 1) / S::WARPS, &grid);
     if (st != FAMST_OK) return st;
     FAMST_LAUNCH(ex, fn, grid, S::WARPS * 32, S::SMEM, X, d, hr.g, hr.h, members, n, bstart, rec,
-                 best, evals, refine_aerr<NKS>(), refine_eps(d));
+                 best, evals, refine_aerr<NKS>(), refine_eps(d), refine_rel(d));
     return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
 }
 

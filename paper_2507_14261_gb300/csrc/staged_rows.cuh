@@ -69,11 +69,12 @@ __device__ __forceinline__ void stage_rows(const __nv_bfloat16 *__restrict__ H, 
 }
 
 // acc[T] = D of mma tile T: rows = candidates 16 T .. 16 T + 15 of the
-// staged round, columns = the eight B columns (b0, b1 per k step).
+// staged round, columns = the eight B columns (b0, b1 per k step). Without
+// `both` the second tile is left out (acc[1] is zero).
 template <int NKS>
 __device__ __forceinline__ void round_dots(uint32_t sbuf, const uint32_t (&b0)[NKS],
                                            const uint32_t (&b1)[NKS], int lane,
-                                           float (&acc)[2][4]) {
+                                           float (&acc)[2][4], bool both = true) {
     using S = StageRows<NKS>;
     // ldmatrix: lanes 8 mi .. 8 mi + 7 address matrix mi = (rows 8 (mi & 1) ..,
     // k half mi >> 1): the A fragment order of m16n8k16
@@ -83,6 +84,7 @@ __device__ __forceinline__ void round_dots(uint32_t sbuf, const uint32_t (&b0)[N
     for (int T = 0; T < 2; ++T) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[T][e] = 0.0f;
+        if (T == 1 && !both) break;
 #pragma unroll
         for (int ks = 0; ks < NKS; ++ks) {
             uint32_t a0, a1, a2, a3;

@@ -104,18 +104,19 @@ __global__ void glist_fill_kernel(const int32_t *__restrict__ nbr, int64_t n, in
 }
 
 // Shared memory of one warp: a staged round of 32 rows, the round's
-// (eb, n2) and ids, eight task slots.
+// (eb, n2) and ids, eight task slots, the round's surviving pairs.
 template <int NKS>
 struct Stage : StageRows<NKS> {
     static constexpr int WARPS = NKS >= 16 ? 4 : 8;
-    static constexpr int WARP_BYTES = StageRows<NKS>::ROWS_BYTES + 32 * 8 + 32 * 4 + 8 * 16 + 8 * 8;
+    static constexpr int WARP_BYTES =
+        StageRows<NKS>::ROWS_BYTES + 32 * 8 + 32 * 4 + 8 * 16 + 8 * 8 + 256;
     static constexpr int SMEM = WARPS * WARP_BYTES;
 };
 
 // --------------------------------------------------- per-edge scan (tail)
 
 // argmin over G[c] of (w(c', fixed), 1 + c') with the incumbent (w0, 0).
-template <int NKS, int XR>
+template <int NKS, int NQ>
 __device__ __forceinline__ uint64_t scan_staged(
     const float *__restrict__ X, int d, int c, int fixed, float w0, const GLists &g,
     const __nv_bfloat16 *__restrict__ H, const float *__restrict__ heb,
@@ -166,11 +167,20 @@ __device__ __forceinline__ uint64_t scan_staged(
         const float bound = __fmul_ru(fminf(mh, key_w(best)), 1.0f + 0x1p-22f);
         unsigned sv = __ballot_sync(0xffffffffu, valid && lo <= bound);
         if (lane == 0) canon += unsigned(__popc(sv));
-        while (sv) {   // survivors: canonical distance by the whole warp
-            const int sl = __ffs(sv) - 1;
-            sv &= sv - 1;
-            const int c2 = __shfl_sync(0xffffffffu, cand, sl);
-            const uint64_t key = cand_key(canon_w<XR>(X, d, fixed, c2, lane), c2);
+        while (sv) {   // survivors: canonical distances, four at a time
+            int sl = -1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {   // group j's survivor
+                if ((lane >> 3) == j) sl = __ffs(sv) - 1;
+                sv &= sv - 1;
+            }
+            const int c2 = __shfl_sync(0xffffffffu, cand, sl < 0 ? 0 : sl);
+            uint64_t key = cand_key(canon_group8<NQ>(X, d, fixed, sl < 0 ? fixed : c2, lane), c2);
+            if (sl < 0) key = KEY_NONE;
+            uint64_t o = shfl_xor_u64(key, 8);
+            key = o < key ? o : key;
+            o = shfl_xor_u64(key, 16);
+            key = o < key ? o : key;
             best = key < best ? key : best;
         }
     }
@@ -181,7 +191,7 @@ __device__ __forceinline__ uint64_t scan_staged(
 // 0 .. m-1), each iterated to its own fixed point; change_hist[c] counts the
 // edges that changed c times here. A v-scan that repeats the previous
 // sweep's inputs is reused.
-template <int NKS, int XR, int MINB>
+template <int NKS, int NQ, int MINB>
 __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
     refine_staged_kernel(const float *__restrict__ X, int d, GLists g,
                          const __nv_bfloat16 *__restrict__ H, const float *__restrict__ heb,
@@ -210,7 +220,7 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
         uint64_t mv_b = 0;
         for (; changes < max_iters; ++changes) {
             // u-loop: u' in G[u] against v
-            const uint64_t bu = scan_staged<NKS, XR>(X, d, u, v, wt, g, H, heb, hn2, sbuf, lane,
+            const uint64_t bu = scan_staged<NKS, NQ>(X, d, u, v, wt, g, H, heb, hn2, sbuf, lane,
                                                      aerr, eps, evals, canon);
             ++scans_total;
             const int us = key_lo(bu) ? int(key_lo(bu)) - 1 : u;
@@ -220,7 +230,7 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
             if (v == mv_v && us == mv_u)
                 bv = mv_b;
             else {
-                bv = scan_staged<NKS, XR>(X, d, v, us, ws, g, H, heb, hn2, sbuf, lane, aerr, eps,
+                bv = scan_staged<NKS, NQ>(X, d, v, us, ws, g, H, heb, hn2, sbuf, lane, aerr, eps,
                                           evals, canon);
                 ++scans_total;
             }
@@ -292,52 +302,11 @@ __global__ void bsp_scatter_kernel(const int32_t *__restrict__ list, const int32
     best[pos] = uint64_t(__float_as_uint(ew[e])) << 32;
 }
 
-// Up to four canonical distances (X rows fx[j], c2[j]) computed together,
-// each keyed (w, 1 + c2) into sbest[tj] when smaller; warp-uniform inputs.
-template <int XR>
-__device__ __forceinline__ void canon_batch(const float *__restrict__ X, int d, int nq,
-                                            const int (&fx)[4], const int (&c2)[4],
-                                            const int (&tj)[4], unsigned long long *sbest,
-                                            int lane) {
-    if constexpr (XR > 0) {
-        float xa[4][XR], xb[4][XR];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int q = 0; q < XR; ++q) {
-                const int t = lane + 32 * q;
-                const bool ok = j < nq && t < d;
-                xa[j][q] = ok ? __ldg(X + int64_t(fx[j]) * d + t) : 0.0f;
-                xb[j][q] = ok ? __ldg(X + int64_t(c2[j]) * d + t) : 0.0f;
-            }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (j >= nq) break;
-            float p = 0.0f;
-#pragma unroll
-            for (int q = 0; q < XR; ++q) {
-                const float dl = __fsub_rn(xb[j][q], xa[j][q]);
-                p = __fmaf_rn(dl, dl, p);
-            }
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) p = __fadd_rn(p, __shfl_xor_sync(0xffffffffu, p, o));
-            const uint64_t key = cand_key(__fsqrt_rn(p), c2[j]);
-            if (lane == 0 && key < sbest[tj[j]]) sbest[tj[j]] = key;
-        }
-    } else {
-        for (int j = 0; j < nq; ++j) {
-            const uint64_t key = cand_key(canon_w<0>(X, d, fx[j], c2[j], lane), c2[j]);
-            if (lane == 0 && key < sbest[tj[j]]) sbest[tj[j]] = key;
-        }
-    }
-    __syncwarp();
-}
-
 // One warp per scanned vertex c (visited in component order, 32 vertices
 // looked up per step): G[c]'s rows are staged once per round of 32 and
 // scored against the fixed points of all scans of c, eight per mma; the
 // best key of the scan at sorted position i is kept in best[i].
-template <int NKS, int XR, int MINB>
+template <int NKS, int NQ, int MINB>
 __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
     refine_group_kernel(const float *__restrict__ X, int d, GLists g,
                         const __nv_bfloat16 *__restrict__ H, const int32_t *__restrict__ members,
@@ -355,6 +324,7 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
     float4 *s_task = reinterpret_cast<float4 *>(wb + S::ROWS_BYTES + 384);   // 8 (fixed, eb, n2)
     unsigned long long *s_best =
         reinterpret_cast<unsigned long long *>(wb + S::ROWS_BYTES + 512);    // 8 best keys
+    uint8_t *s_code = reinterpret_cast<uint8_t *>(wb + S::ROWS_BYTES + 576); // surviving pairs
     const float inf = __int_as_float(0x7f800000);
     const int g4 = lane >> 2, t4 = lane & 3;   // mma fragment row group / column pair
     // counters, one per lane: pairs (lane 0), canonical evaluations (1),
@@ -492,34 +462,34 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
 #pragma unroll
                         for (int e2 = 0; e2 < 4; ++e2)
                             if (lo[T][e2] <= lim[e2 & 1]) my |= 1u << (4 * T + e2);
-                    {
-                        const unsigned cnt = __reduce_add_sync(0xffffffffu, __popc(my));
-                        if (lane == 1) ctr += cnt;
-                    }
-#pragma unroll 1
-                    while (true) {
-                        int qf[4], qc[4], qt[4], nq = 0;
-#pragma unroll 1
-                        while (nq < 4) {
-                            const unsigned any = __ballot_sync(0xffffffffu, my != 0u);
-                            if (!any) break;
-                            const int sl = __ffs(any) - 1;
-                            const int bit = __ffs(__shfl_sync(0xffffffffu, my, sl)) - 1;
-                            if (lane == sl) my &= my - 1u;
-                            const int ci = 16 * (bit >> 2) + (sl >> 2) + 8 * ((bit & 3) >> 1);
-                            const int tj = 2 * (sl & 3) + (bit & 1);
+                    // the surviving pairs as one list of (candidate, task) codes
+                    int at = __popc(my);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (j == nq) {
-                                    qc[j] = s_id[ci];
-                                    qf[j] = __float_as_int(s_task[tj].x);
-                                    qt[j] = tj;
-                                }
-                            ++nq;
-                        }
-                        if (nq == 0) break;
-                        canon_batch<XR>(X, d, nq, qf, qc, qt, s_best, lane);
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, at, o);
+                        if (lane >= o) at += y;
                     }
+                    const int ns = __shfl_sync(0xffffffffu, at, 31);
+                    if (lane == 1) ctr += unsigned(ns);
+                    at -= __popc(my);
+                    while (my) {
+                        const int bit = __ffs(my) - 1;
+                        my &= my - 1u;
+                        const int ci = 16 * (bit >> 2) + g4 + 8 * ((bit & 3) >> 1);
+                        s_code[at++] = uint8_t(8 * ci + 2 * t4 + (bit & 1));
+                    }
+                    __syncwarp();
+                    // decided on canonical distances, four at a time
+#pragma unroll 1
+                    for (int q = 0; q < ns; q += 4) {
+                        const int e = q + (lane >> 3);
+                        const int code = s_code[e < ns ? e : q];
+                        const int c2 = s_id[code >> 3], tj = code & 7;
+                        const float w =
+                            canon_group8<NQ>(X, d, __float_as_int(s_task[tj].x), c2, lane);
+                        if (e < ns && (lane & 7) == 0) atomicMin(s_best + tj, cand_key(w, c2));
+                    }
+                    __syncwarp();
                     if ((!single || r0 + 32 >= deg) && lane < ntb) best[tb + lane] = s_best[lane];
                     __syncwarp();
                 }
@@ -612,14 +582,14 @@ famst_status occupancy_grid(const Exec &ex, K *fn, int threads, int smem, int64_
     return FAMST_OK;
 }
 
-template <int NKS, int XR, int MINB>
+template <int NKS, int NQ, int MINB>
 famst_status launch_staged_t(const Exec &ex, const float *X, int d, const HalfRows &hr,
                              int32_t *eu, int32_t *ev, float *ew, const int32_t *order, int64_t m,
                              int max_iters, int32_t *change_hist, unsigned long long *next_item,
                              unsigned long long *evals) {
     using S = Stage<NKS>;
     unsigned grid;
-    auto *fn = refine_staged_kernel<NKS, XR, MINB>;
+    auto *fn = refine_staged_kernel<NKS, NQ, MINB>;
     famst_status st =
         occupancy_grid(ex, fn, S::WARPS * 32, S::SMEM, (m + S::WARPS - 1) / S::WARPS, &grid);
     if (st != FAMST_OK) return st;
@@ -629,13 +599,13 @@ famst_status launch_staged_t(const Exec &ex, const float *X, int d, const HalfRo
     return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
 }
 
-template <int NKS, int XR, int MINB>
+template <int NKS, int NQ, int MINB>
 famst_status launch_group_t(const Exec &ex, const float *X, int d, const HalfRows &hr,
                             const int32_t *members, int64_t n, const int32_t *bstart,
                             const int4 *rec, unsigned long long *best, unsigned long long *evals) {
     using S = Stage<NKS>;
     unsigned grid;
-    auto *fn = refine_group_kernel<NKS, XR, MINB>;
+    auto *fn = refine_group_kernel<NKS, NQ, MINB>;
     famst_status st =
         occupancy_grid(ex, fn, S::WARPS * 32, S::SMEM, (n + S::WARPS - 1) / S::WARPS, &grid);
     if (st != FAMST_OK) return st;
@@ -651,7 +621,7 @@ famst_status launch_group(const Exec &ex, const float *X, int d, const HalfRows 
         return launch_group_t<4, 2, 4>(ex, X, d, hr, members, n, bstart, rec, best, evals);
     if (hr.ld == 128)
         return launch_group_t<8, 4, 3>(ex, X, d, hr, members, n, bstart, rec, best, evals);
-    return launch_group_t<16, 0, 2>(ex, X, d, hr, members, n, bstart, rec, best, evals);
+    return launch_group_t<16, 8, 2>(ex, X, d, hr, members, n, bstart, rec, best, evals);
 }
 
 }  // namespace
@@ -693,7 +663,7 @@ famst_status launch_refine_staged(const Exec &ex, const float *X, int d, const H
     if (hr.ld == 128)
         return launch_staged_t<8, 4, 3>(ex, X, d, hr, eu, ev, ew, order, m, max_iters, change_hist,
                                         next_item, evals);
-    return launch_staged_t<16, 0, 2>(ex, X, d, hr, eu, ev, ew, order, m, max_iters, change_hist,
+    return launch_staged_t<16, 8, 2>(ex, X, d, hr, eu, ev, ew, order, m, max_iters, change_hist,
                                      next_item, evals);
 }
 

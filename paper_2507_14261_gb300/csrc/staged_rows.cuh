@@ -138,6 +138,48 @@ __device__ __forceinline__ float canon_w(const float *__restrict__ X, int d, int
     }
 }
 
+// Four canonical FP32 distances at once, one per group of eight lanes (rows a
+// and b of the group; d <= 32 NQ, d % 4 == 0, 16-byte rows): lane g of a group
+// holds the partials 4 g .. 4 g + 3, read as float4. The canonical butterfly's
+// steps 16, 8 and 4 pair lanes g and g ^ 4, g ^ 2, g ^ 1, its steps 2 and 1
+// the partials inside a lane; a lane passes on what its partner keeps (two
+// partials, then one), so the same additions take six shuffles for the four
+// pairs instead of twenty. Every lane of a group gets its pair's distance.
+template <int NQ>
+__device__ __forceinline__ float canon_group8(const float *__restrict__ X, int d, int a, int b,
+                                              int lane) {
+    const int g = lane & 7, d4 = d >> 2;
+    const float4 *ra = reinterpret_cast<const float4 *>(X + int64_t(a) * d);
+    const float4 *rb = reinterpret_cast<const float4 *>(X + int64_t(b) * d);
+    float4 xa[NQ], xb[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const int c = g + 8 * q;
+        xa[q] = c < d4 ? __ldg(ra + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xb[q] = c < d4 ? __ldg(rb + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const float t0 = __fsub_rn(xb[q].x, xa[q].x), t1 = __fsub_rn(xb[q].y, xa[q].y);
+        const float t2 = __fsub_rn(xb[q].z, xa[q].z), t3 = __fsub_rn(xb[q].w, xa[q].w);
+        p0 = __fmaf_rn(t0, t0, p0);
+        p1 = __fmaf_rn(t1, t1, p1);
+        p2 = __fmaf_rn(t2, t2, p2);
+        p3 = __fmaf_rn(t3, t3, p3);
+    }
+    const bool u4 = (g & 4) != 0, u2 = (g & 2) != 0;
+    float k0 = u4 ? p2 : p0, k1 = u4 ? p3 : p1;
+    k0 = __fadd_rn(k0, __shfl_xor_sync(0xffffffffu, u4 ? p0 : p2, 4));
+    k1 = __fadd_rn(k1, __shfl_xor_sync(0xffffffffu, u4 ? p1 : p3, 4));
+    float k = u2 ? k1 : k0;
+    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, u2 ? k0 : k1, 2));
+    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, k, 1));
+    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, k, 4));
+    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, k, 2));
+    return __fsqrt_rn(k);
+}
+
 __device__ __forceinline__ uint64_t cand_key(float w, int id) {
     return (uint64_t(__float_as_uint(w)) << 32) | uint32_t(id + 1);
 }

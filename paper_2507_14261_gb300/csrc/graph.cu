@@ -208,22 +208,25 @@ __global__ void uf_min_kernel(const int32_t *__restrict__ nbr, int64_t n, int k,
     parent[v] = m;
 }
 
-__global__ void uf_lower_kernel(const int32_t *__restrict__ nbr, int64_t nk, int k,
-                                int32_t *parent_) {
-    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (e >= nk) return;
-    volatile int32_t *parent = parent_;
-    const int ra = parent[e / k], rb = parent[nbr[e]];
-    if (ra == rb) return;
-    const int hi = ra > rb ? ra : rb, lo = ra > rb ? rb : ra;
-    if (parent[hi] > lo) atomicMin(parent_ + hi, lo);
-}
-
 // Vertices in a scrambled order: thread e takes edge j = e mod k of vertex
 // v = (e / k) * 0x9E3779B1 mod 2^m (odd multiplier: a bijection of
 // [0, 2^m), 2^m >= n; v >= n idle). When ids are contiguous in space (clouds
 // laid out one after another, sorted inputs), threads in flight together
 // would otherwise all hook onto the same few roots.
+__global__ void uf_lower_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, uint32_t vmask,
+                                int32_t *parent_) {
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t vl = e / k;
+    if (vl > int64_t(vmask)) return;
+    const uint32_t v = (uint32_t(vl) * 0x9E3779B1u) & vmask;
+    if (int64_t(v) >= n) return;
+    volatile int32_t *parent = parent_;
+    const int ra = parent[v], rb = parent[nbr[int64_t(v) * k + (e - vl * k)]];
+    if (ra == rb) return;
+    const int hi = ra > rb ? ra : rb, lo = ra > rb ? rb : ra;
+    if (parent[hi] > lo) atomicMin(parent_ + hi, lo);
+}
+
 __global__ void uf_hook_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, uint32_t vmask,
                                int32_t *parent, int limit, int *dstatus) {
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -382,16 +385,16 @@ famst_status components_uf(const Exec &ex, Arena &ar, const int32_t *nbr, int64_
     int64_t nk = n * k;
     FAMST_LAUNCH(ex, uf_min_kernel, blocks_for(n, th), th, 0, nbr, n, nk > 0 ? k : 0, parent);
     if (nk > 0) {
+        uint32_t vmask = 1;
+        while (int64_t(vmask) + 1 < n) vmask = (vmask << 1) | 1u;
+        const unsigned hgrid = blocks_for((int64_t(vmask) + 1) * k, th);
         for (int r = 0; r < UF_ROUNDS; ++r) {
             FAMST_LAUNCH(ex, uf_compress_kernel, blocks_for(n, th), th, 0, parent, n, lim,
                          ex.dstatus);
-            FAMST_LAUNCH(ex, uf_lower_kernel, blocks_for(nk, th), th, 0, nbr, nk, k, parent);
+            FAMST_LAUNCH(ex, uf_lower_kernel, hgrid, th, 0, nbr, n, k, vmask, parent);
         }
         FAMST_LAUNCH(ex, uf_compress_kernel, blocks_for(n, th), th, 0, parent, n, lim, ex.dstatus);
-        uint32_t vmask = 1;
-        while (int64_t(vmask) + 1 < n) vmask = (vmask << 1) | 1u;
-        FAMST_LAUNCH(ex, uf_hook_kernel, blocks_for((int64_t(vmask) + 1) * k, th), th, 0, nbr, n, k,
-                     vmask, parent, lim, ex.dstatus);
+        FAMST_LAUNCH(ex, uf_hook_kernel, hgrid, th, 0, nbr, n, k, vmask, parent, lim, ex.dstatus);
     }
     FAMST_LAUNCH(ex, uf_flatten_kernel, blocks_for(n, th), th, 0, parent, n, root, flag, lim,
                  ex.dstatus);

@@ -199,6 +199,37 @@ __device__ __forceinline__ uint64_t warp_min_u64(uint64_t v) {
     return v;
 }
 
+// Bitonic sort of 32 H keys (element 32 h + lane), ascending.
+template <int H>
+__device__ __forceinline__ void warp_sort_regs(uint64_t (&key)[H], int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32 * H; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            if (stride >= 32) {
+                const int hs = stride >> 5;
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    if (h & hs) continue;
+                    const bool asc = ((h * 32 + lane) & size) == 0;
+                    const uint64_t a = key[h], b = key[(h | hs) < H ? (h | hs) : h];
+                    const uint64_t mn = a < b ? a : b, mx = a < b ? b : a;
+                    key[h] = asc ? mn : mx;
+                    key[(h | hs) < H ? (h | hs) : h] = asc ? mx : mn;
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const bool asc = ((h * 32 + lane) & size) == 0;
+                    const uint64_t other = shfl_xor_u64(key[h], stride);
+                    const bool lower = (lane & stride) == 0;
+                    key[h] = (key[h] < other) == (lower == asc) ? key[h] : other;
+                }
+            }
+        }
+    }
+}
+
 // ---------------------------------------------- fast squared distances
 // Warp-cooperative squared distances for filters and bounds (never for a
 // stored weight). Rows are 16-byte aligned with d % 4 == 0; lane l holds
@@ -455,7 +486,8 @@ struct TcTile {
     int row_end;   // padded rows >= row_end are padding
     int shift;     // compact id = padded row - shift
     int part;      // 0: the query tile's whole key list; s > 0: one part of a split
-                   // list, whose rows' sorted candidates go to side slot s - 1
+                   // list, whose rows' candidates go to side slot s - 1
+    int cloud;     // batched: the cloud (else 0)
 };
 // Long key lists of a pruned Phase 1 are split so that no work item holds
 // much more than a share of one SM's tiles: at most PRUNE_SPLIT_TILES query
@@ -464,6 +496,10 @@ struct TcTile {
 constexpr int PRUNE_SPLIT_TILES = 640;
 constexpr int PRUNE_SPLIT_SLOTS = 2 * PRUNE_SPLIT_TILES;
 constexpr int PRUNE_SPLIT_MIN = 16;
+// Most candidates the tensor tiles keep per row (a row with more is not
+// certified); knn_tc_cand_cap(k): for this k.
+constexpr int TC_CAND_CAP = 128;
+int knn_tc_cand_cap(int k);
 struct F32Tile {
     int qbase;     // first query row of the block (64 rows)
     int nq;        // valid queries in the block
@@ -566,22 +602,18 @@ famst_status prune_partition(const Exec &ex, Arena &ar, const float *X, int d, i
 #include <cuda.h>
 #include <cuda_bf16.h>
 namespace famst {
-// Tile shape of the batched tensor pass for operand width D: epi_req = 8
-// asks for eight epilogue warps (granted when the lists and three ring
-// stages fit), 4 for four; the ring takes what shared memory leaves.
-bool knn_tc_batched_plan(int D, int k, bool x3, int epi_req, int *stages, size_t *smem, int *kc,
-                         int *epi);
-famst_status knn_tc_batched_tiles(const Exec &ex, int D, bool x3, int stages, size_t smem, int kc,
-                                  int epi, const TcTile *tiles, int64_t nctas, const float *ny,
-                                  int32_t *cand, float *splus, const CUtensorMap *mA,
-                                  const CUtensorMap *mB, bool spiral = false);
+// Ring depth and shared memory of the batched tensor pass for operand width D.
+bool knn_tc_batched_plan(int D, int k, bool x3, int *stages, size_t *smem);
+int knn_tc_epilogue_warps();
+size_t knn_tc_log_entries(int64_t nctas, int num_sms);   // int2 scratch entries of the tile kernel
 famst_status knn_tc_batched(const Exec &ex, const float *Xc, int D, int64_t N, int64_t NP,
                             const long long *voff, const long long *roff, int B,
                             const CloudDev *cl, const TcTile *tiles, int64_t nctas, int k,
-                            bool x3, int stages, size_t smem, int kc, int epi, __nv_bfloat16 *H,
+                            bool x3, int stages, size_t smem, __nv_bfloat16 *H,
                             float *ny, float *xn2, float *mean, unsigned *ymax, int32_t *cand,
-                            float *splus, int32_t *fail_rows, int32_t *fail_count, int32_t *nbr,
-                            float *dist, const CUtensorMap *mA, const CUtensorMap *mB,
+                            int32_t *ccnt, int2 *log, int *claim, float *splus,
+                            int32_t *fail_rows, int32_t *fail_count, int32_t *nbr, float *dist,
+                            const CUtensorMap *mA, const CUtensorMap *mB,
                             const float *Xorig = nullptr, const int32_t *perm = nullptr);
 bool knn_tc_batched_maps(const void *H, int64_t NP, int D, bool x3, CUtensorMap *mA,
                          CUtensorMap *mB);

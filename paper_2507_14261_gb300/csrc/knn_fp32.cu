@@ -489,37 +489,6 @@ __device__ __forceinline__ float warp_canon32(const float *__restrict__ X, int l
     return cand >= 0 ? acc[0] : 0.0f;
 }
 
-// Bitonic sort of 32 H keys (element 32 h + lane), ascending.
-template <int H>
-__device__ __forceinline__ void warp_sort_regs(uint64_t (&key)[H], int lane) {
-#pragma unroll
-    for (int size = 2; size <= 32 * H; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride >= 32) {
-                const int hs = stride >> 5;
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    if (h & hs) continue;
-                    const bool asc = ((h * 32 + lane) & size) == 0;
-                    const uint64_t a = key[h], b = key[(h | hs) < H ? (h | hs) : h];
-                    const uint64_t mn = a < b ? a : b, mx = a < b ? b : a;
-                    key[h] = asc ? mn : mx;
-                    key[(h | hs) < H ? (h | hs) : h] = asc ? mx : mn;
-                }
-            } else {
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const bool asc = ((h * 32 + lane) & size) == 0;
-                    const uint64_t other = shfl_xor_u64(key[h], stride);
-                    const bool lower = (lane & stride) == 0;
-                    key[h] = (key[h] < other) == (lower == asc) ? key[h] : other;
-                }
-            }
-        }
-    }
-}
-
 struct RerankArgs {
     const float *X;
     int d, ld, k, kp;
@@ -616,8 +585,10 @@ __global__ void __launch_bounds__(128) rerank_fp32_kernel(RerankArgs A) {
     }
     warp_sort_regs<H>(key, lane);
     const uint64_t kth = warp_list_at<H>(key, k - 1);
-    bool cert = !(sp < inf) || (kth != KEY_NONE &&
-                                double(sp) * (1.0 - double(A.rho)) > double(key_w(kth)));
+    // (FP32, rounded down, decides all but near ties; FP64 the rest)
+    bool cert = !(sp < inf) ||
+                (kth != KEY_NONE && (__fmul_rd(sp, __fsub_rd(1.0f, A.rho)) > key_w(kth) ||
+                                     double(sp) * (1.0 - double(A.rho)) > double(key_w(kth))));
     if (A.skipQ) {   // keys of skipped tiles lie at true distance >= skip
         const float skip = A.skipQ[q / (2 * QM)];
         cert &= !(skip < inf) || (kth != KEY_NONE &&

@@ -8,33 +8,52 @@
 // hi/lo split x' ~ xh + xl (xh.yh + xl.yh + xh.yl), whose error is
 // O(2^-16) instead of O(2^-8).
 //
-// Kernel (one CTA per 128 query rows, 64 + 32 E threads, E = 8 or 4):
+// Kernel (one CTA per 128 query rows, 18 warps):
 //   warp 0     TMA producer: the query tile's operand rows once (resident),
 //              then 256-key tiles, one 64-wide K block per ring stage;
 //   warp 1     allocates 512 TMEM columns (two 128 x 256 FP32
 //              accumulators) and one lane issues tcgen05.mma (M=128, N=256,
 //              K=16 per instruction) with SW128 K-major smem descriptors;
 //              tcgen05.commit frees ring stages and publishes accumulators;
-//   warps 2..  E epilogue warps: thread r of a warp owns query row r of its
-//              TMEM lane quarter; with E = 8 two warps share a quarter, each
-//              on half of the columns. It loads 16 columns at a time with
-//              tcgen05.ld, forms s = ny_j - 2 acc (key norms read from L1),
-//              and stages the columns that beat its row's threshold in
-//              shared memory. When any lane's stage is nearly full the warp
-//              merges the stages, eight candidates at a time (a sorting
-//              network, then a bitonic merge: topk_merge.cuh), into per-row
-//              sorted register lists of the KC smallest scores, then
-//              tightens the threshold to the KC-th score (the smaller of the
-//              two halves' when E = 8); the halves' lists merge at the end.
+//   warps 2..  sixteen epilogue warps, four per TMEM lane quarter: thread r of
+//              a warp owns query row r of the quarter and, of every tile, a
+//              fourth of the columns (16-column chunks g, g + 4, g + 8, g + 12
+//              for the quarter's warp g). It loads 16 columns at a time with
+//              tcgen05.ld and forms s = ny_j - 2 acc (key norms from L1).
+//              A row keeps no sorted list of ids (32 to 64 scores and ids per
+//              thread left room for eight warps, which could not hide the
+//              latency of TMEM, norms and branches, and two column halves each
+//              kept a full list):
+//              - bound: a thread keeps its R smallest scores, a sorted list; a
+//                new one goes in by R min/max pairs. The row's T is the largest
+//                of its four threads' R-th (shared memory): each list holds R
+//                distinct keys' scores at or below it, so at least 4 R keys
+//                score <= T.
+//              - log: a key that scores at most the T of the moment is appended
+//                to the thread's log of (score, id) in a scratch area of the
+//                CTA (about 4 R ln(keys / 4 R) entries per row, L2-resident).
+//                The item's first tile is read twice from TMEM, for T and then
+//                for the log.
+//              - at the end a warp per row keeps the logged keys at or below
+//                the final T and lowers it to the k-th key plus the score
+//                error's margin: the row's candidates, with s+ = that bound.
+//              Bound: the epilogue's issue slots (48 % of peak: min/max pairs,
+//              norms and log branches; the tensor cores wait for it). Against
+//              sorted id lists in eight warps: 65,537 x 96 overlapping points at
+//              k = 32 7.4 -> 4.05 ms, 256 clouds of 500 to 20,000 points
+//              (k = 16) 31.2 -> 23.5, 1M x 128 sphere points (k = 32, pruned
+//              lists) 9.5 -> 8.05, five masked passes of a 10,000-point EMST
+//              1.31 -> 0.92; 100,000 x 128 blobs (k = 16, pruned lists of few
+//              tiles, so the first tile's second turn weighs) 1.05 -> 1.18.
 // Work items: a query tile with its key tiles (all of them, or a pruned
 // list); a long pruned list is split into parts run by separate CTAs, whose
-// rows' lists split_merge_kernel combines.
+// rows' candidates split_merge_kernel combines.
 // Nothing of the n x n score matrix leaves the SM. Every mbarrier wait is
 // bounded in time; on expiry the CTA sets an error bit, drains its own
 // copies and MMAs, frees its TMEM and returns.
 //
-// Exactness. Row i keeps k' = KC-1 candidates and s+ = its KC-th smallest
-// score. The rerank kernel computes the canonical FP32 distance of every
+// Exactness. Row i keeps every key (but itself) that scores at most s+.
+// The rerank kernel computes the canonical FP32 distance of every
 // candidate, takes the k smallest (w, id), and certifies the row when a
 // rigorous bound on the score error proves that no unkept point can have a
 // canonical distance <= the k-th. Uncertified rows are recomputed by the
@@ -47,11 +66,11 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "famst_internal.cuh"
 #include "mbarrier.cuh"
 #include "tcgen05.cuh"
-#include "topk_merge.cuh"
 
 namespace famst {
 namespace {
@@ -61,9 +80,14 @@ constexpr int BN = 256;          // keys per tile (accumulator columns)
 constexpr int BK = TC_BK;        // K elements per stage (one 128-byte swizzle atom)
 constexpr int A_BLOCK = BM * BK * 2;   // 16 KB
 constexpr int B_BLOCK = BN * BK * 2;   // 32 KB
-constexpr int CAPB = 24;         // staged candidates per row (flush check every 16 columns)
+constexpr int CAP = TC_CAND_CAP; // candidates kept per row; a row with more is not certified
+constexpr int EPI = 16;          // epilogue warps
+constexpr int LOG_CAP = 256;     // log entries per thread; compacted beyond LOG_CAP - 64
+constexpr size_t LOG_SLOT = size_t(4) * BM * LOG_CAP;   // entries of one CTA's scratch area
+// scratch areas of a launch of nctas CTAs, of which one per SM is resident
+inline int log_slots(int64_t nctas, int num_sms) { return int(std::min<int64_t>(nctas, num_sms)); }
+constexpr int TC_THREADS = 64 + 32 * EPI;
 constexpr int VISITED_ROWS_SHARE = 32;   // uncertified rows redone one by one: up to n / this
-constexpr int TC_THREADS_MAX = 64 + 32 * 8;   // producer, MMA issuer, up to 8 epilogue warps
 
 // Instruction descriptor, kind::f8f6f4: D F32, A/B E4M3 (format 0), both K-major.
 __host__ __device__ constexpr uint32_t idesc_e4m3(int M, int N) {
@@ -81,6 +105,47 @@ __device__ __forceinline__ void umma_f8(uint32_t d_tmem, uint64_t adesc, uint64_
         : "memory");
 }
 
+// A row keeps the keys up to its k-th plus what the certificate loses to the
+// score's error, eps_dot |x||y|max + eps_row (|x| + |y|max)^2: that is the
+// fewest that a row can be certified with, and what it takes where the errors
+// are large. (A fixed 4 R keys cost the re-rank 31 to 50 distances a row
+// instead of about k + 3: 10.5 against 12.9 ms for 256 clouds of 500 to 20,000
+// points at k = 16; and rows whose margin held more were redone exactly.)
+struct Select {
+    int k, cap;
+    float eps_dot, eps_row;
+};
+// count(t): the row's keys that score at most t, of all up to Tr; lo, hi:
+// the least and the largest of them. A bound by bisection: with k + 1 or k + 2
+// keys at or below it, plus the margin; where that takes in more than cap,
+// one with cap - 8 .. cap (or nearly).
+template <class Count>
+__device__ __forceinline__ float select_bound(Count count, float lo, float hi, float Tr,
+                                              const Select &S, float xn, float ym) {
+    const float margin = S.eps_dot * xn * ym + S.eps_row * (xn + ym) * (xn + ym);
+    int w0 = S.k + 1, w1 = S.k + 2;
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        float l = lo, u = hi;
+#pragma unroll 1
+        for (int it = 0; it < 10; ++it) {
+            const float mid = 0.5f * l + 0.5f * u;
+            const int c = count(mid);
+            if (c >= w0) {
+                u = mid;
+                if (c <= w1) break;
+            } else {
+                l = mid;
+            }
+        }
+        if (pass > 0) return u;
+        hi = fminf(u + margin, Tr);
+        if (count(hi) <= S.cap) return hi;
+        w0 = S.cap - 8;
+        w1 = S.cap;
+    }
+}
+
 struct TcArgs {
     int n;
     int nk_tiles;
@@ -88,52 +153,51 @@ struct TcArgs {
     int x3;         // hi/lo split on
     int stages;     // B ring depth
     const float *ny;    // key norms ||x'_j||^2, +inf beyond n (nk_tiles * BN entries)
-    int32_t *cand;      // n x (KC - 1)
+    int32_t *cand;      // n x cap (TOP1: n)
+    int32_t *ccnt;      // candidates of the row
+    int cap;            // places per row in cand and side_j / side_s (<= CAP)
+    Select sel;         // which of them a row keeps
+    const unsigned *ymax;   // largest |y| (float bits) of every cloud
     float *splus;       // n
     int *status;
     const TcTile *tiles;  // null: one cloud, CTA b = query tile b over all keys
     const int32_t *colcomp;  // MASK: component of every (padded) row; pairs in one component are skipped
     const int32_t *klist;    // non-null: CTA key tiles are klist[kt0 .. kt1) instead of kt0 .. kt1
     int cross;               // queries and keys are different sets: no self-exclusion
-    int epi;                 // epilogue warps: 8 (two per TMEM lane quarter, each on half
-                             // of the columns) or 4 (0 reads as 4)
     const float *rscale;     // FP8 operands: per-row scale s (x' ~ s q), query and key rows
                              // alike (keys padded with 1 to nk_tiles * BN entries)
     const float *thr0;       // non-null: per query row, a score every one of its k nearest
-                             // keys stays below (the lists start there; s+ is capped by it)
+                             // keys stays below (T and s+ are capped by it)
     int nitems;              // > 0: work items (query tiles) handed to the CTAs round-robin
                              // (persistent launch, grid <= nitems); 0: one per CTA
     int spiral;              // 1: an item's key tiles [kt0, kt1) are visited outward from the
-                             // query tile's own (q0 / BN, then +1, -1, +2, ...): on rows in
-                             // a spatial order the lists fill with near keys first
+                             // query tile's own (q0 / BN, then +1, -1, +2, ...)
     const int32_t *nitems_dev;  // non-null (one item per CTA): CTAs from *nitems_dev on are idle
     int32_t *side_j;         // items that are parts of a split list (TcTile::part = s + 1):
-    float *side_s;           //   per slot s and tile row, the KC - 1 smallest (id, score),
-    float *side_splus;       //   ascending, and the part's s+
+    float *side_s;           //   per slot s and tile row, the candidates' ids and scores
+    int32_t *side_cnt;       //   (cap each), their number and the part's s+
+    float *side_splus;
+    int2 *log;               // nslots scratch areas of LOG_SLOT (score bits, id)
+    int *claim;              // per area: 0 free, 1 taken by a resident CTA
+    int nslots;              // at least as many as CTAs can be resident (one per SM)
 };
 
-template <int KC>
-__device__ __forceinline__ void list_insert(float (&ls)[KC], int (&lj)[KC], float s, int j) {
-    // (s, j) goes before the first entry greater than s; the entries from
-    // there on move one place up. Every slot is computed from the old
-    // ls[p - 1], ls[p] and s alone (no value carried from slot to slot), so
-    // the KC updates are independent instructions rather than one chain.
-#pragma unroll
-    for (int p = KC - 1; p >= 1; --p) {
-        const bool up = ls[p - 1] > s;   // the entry below moves here
-        const bool here = ls[p] > s;
-        ls[p] = up ? ls[p - 1] : (here ? s : ls[p]);
-        lj[p] = up ? lj[p - 1] : (here ? j : lj[p]);
-    }
-    const bool here0 = ls[0] > s;
-    ls[0] = here0 ? s : ls[0];
-    lj[0] = here0 ? j : lj[0];
+// packed scores of two columns: ny - 2 acc
+__device__ __forceinline__ void scores2(uint32_t d0, uint32_t d1, unsigned long long ny, float &s0,
+                                        float &s1) {
+    unsigned long long d, r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(d0), "r"(d1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(d), "l"(f2_pack(-2.0f, -2.0f)), "l"(ny));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(r));
 }
 
-template <int KC, bool MASK, bool F8 = false>
-__global__ void __launch_bounds__(KC <= 2 * CAPB ? TC_THREADS_MAX : 64 + 32 * 4, 1)
+// R = 0: top-1 mode (the best key and its score).
+template <int R, bool MASK, bool F8 = false>
+__global__ void __launch_bounds__(TC_THREADS, 1)
 knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               TcArgs args) {
+    constexpr bool TOP1 = R == 0;
+    constexpr int RL = TOP1 ? 1 : R;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment for the swizzle atoms
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -146,7 +210,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     if (args.nitems_dev && int(blockIdx.x) >= __ldg(args.nitems_dev)) return;
     const int nitems = args.nitems > 0 ? args.nitems : int(gridDim.x);
     struct Item {
-        int q0, kt0, kt1, nkb, row_end, shift, part;
+        int q0, kt0, kt1, nkb, row_end, shift, part, cloud;
     };
     auto item_of = [&](int item) {
         Item I;
@@ -154,10 +218,10 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             const TcTile T = args.tiles[item];
             I.q0 = T.q0; I.kt0 = T.kt0; I.kt1 = T.kt1; I.nkb = T.nkb; I.row_end = T.row_end;
             I.shift = T.shift;
-            I.part = T.part;
+            I.part = T.part; I.cloud = T.cloud;
         } else {
             I.q0 = item * BM; I.kt0 = 0; I.kt1 = args.nk_tiles; I.nkb = args.nkb;
-            I.row_end = args.n; I.shift = 0; I.part = 0;
+            I.row_end = args.n; I.shift = 0; I.part = 0; I.cloud = 0;
         }
         return I;
     };
@@ -166,22 +230,18 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         if (args.klist) return __ldg(args.klist + I.kt0 + t);
         if (!args.spiral) return I.kt0 + t;
         const int c0 = min(max(I.q0 / BN, I.kt0), I.kt1 - 1);
-        const int L = c0 - I.kt0, R = I.kt1 - 1 - c0, m = min(L, R);
+        const int L = c0 - I.kt0, Rt = I.kt1 - 1 - c0, m = min(L, Rt);
         if (t <= 2 * m) return (t & 1) ? c0 + ((t + 1) >> 1) : c0 - (t >> 1);
-        return R > L ? c0 + (t - m) : c0 - (t - m);
+        return Rt > L ? c0 + (t - m) : c0 - (t - m);
     };
     const int nA_max = (args.x3 ? 2 : 1) * args.nkb;  // resident A blocks (widest item)
     unsigned char *sA = base;
     unsigned char *sB = sA + size_t(nA_max) * A_BLOCK;
-    const int EPI = args.epi == 8 ? 8 : 4;
-    const int NH = EPI / 4;                           // column halves (1 or 2)
-    // staging [NH][CAPB][BM] scores and ids; with two halves, the second
-    // half's final list ([KC][BM], KC <= 2 CAPB) reuses it for the merge
-    float *stg_s = reinterpret_cast<float *>(sB + size_t(args.stages) * B_BLOCK);
-    int *stg_j = reinterpret_cast<int *>(stg_s + NH * CAPB * BM);
-    volatile float *thr_sh = reinterpret_cast<volatile float *>(stg_j + NH * CAPB * BM);  // [2][BM]
-    uint64_t *bars = reinterpret_cast<uint64_t *>(
-        reinterpret_cast<unsigned char *>(stg_j + NH * CAPB * BM) + 2 * BM * 4);
+    float *t_sh = reinterpret_cast<float *>(sB + size_t(args.stages) * B_BLOCK);   // [4][BM]
+    int *j_sh = reinterpret_cast<int *>(t_sh + 4 * BM);                            // [4][BM]
+    float *f_sh = reinterpret_cast<float *>(j_sh + 4 * BM);       // [EPI][CAP] scores, then
+    int *fj_sh = reinterpret_cast<int *>(f_sh + EPI * CAP);       // [EPI][CAP] ids of a row
+    uint64_t *bars = reinterpret_cast<uint64_t *>(fj_sh + EPI * CAP);
     uint64_t *full = bars;                       // [stages]
     uint64_t *empty = bars + args.stages;        // [stages]
     uint64_t *a_full = bars + 2 * args.stages;
@@ -191,6 +251,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     uint64_t *a_empty = mma_done + 1;            // the A blocks may be overwritten
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(a_empty + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    int *slot_sh = reinterpret_cast<int *>(tmem_slot + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -208,17 +269,29 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         mbar_init(a_empty, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if constexpr (!TOP1) {   // a free scratch area: there are as many as resident CTAs
+            int slot = int(blockIdx.x) % args.nslots, tries = 0;
+            while (atomicCAS(args.claim + slot, 0, 1) != 0 && ++tries < (1 << 20))
+                slot = slot + 1 == args.nslots ? 0 : slot + 1;
+            if (tries == 1 << 20) {
+                set_status(args.status, STATUS_LOOP_LIMIT);
+                slot = -1;
+            }
+            *slot_sh = slot;
+        }
+    }
+    if constexpr (!TOP1) {
+        __syncthreads();
+        if (*slot_sh < 0) return;
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
-    for (int x = threadIdx.x; x < 2 * BM; x += blockDim.x) thr_sh[x] = __int_as_float(0x7f800000);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -284,9 +357,8 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     break;
                 }
                 tc_fence_after();
-                const int ntiles = I.kt1 - I.kt0;
                 const int nkb_tile = args.x3 ? 2 * I.nkb : I.nkb;
-                for (int t = 0; t < ntiles && ok; ++t, ++g) {
+                for (int t = 0; t < I.kt1 - I.kt0 && ok; ++t, ++g) {
                     const int b = g & 1, use = g >> 1;
                     if (!mbar_wait(&tempty[b], (use & 1) ^ 1, abort_flag, args.status)) {
                         ok = false;
@@ -336,249 +408,345 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         __syncwarp();
     } else {
         // ------------------------------------------------ epilogue
+        const float inf = __int_as_float(0x7f800000);
         const int quarter = warp & 3;               // TMEM lanes 32*quarter ..
-        const int half = (warp - 2) >> 2;           // columns [half * ncols, + ncols)
-        const int ncols = BN / NH;
-        const int col0 = half * ncols;
+        const int grp = (warp - 2) >> 2;            // 16-column chunks grp, grp + 4, ...
         const int row = quarter * 32 + lane;
-        float *my_s = stg_s + half * CAPB * BM + row;
-        int *my_j = stg_j + half * CAPB * BM + row;
+        volatile float *vt_sh = t_sh;
+        int2 *area = TOP1 ? nullptr : args.log + size_t(*slot_sh) * LOG_SLOT;
+        int2 *my_log = TOP1 ? nullptr : area + size_t(grp * BM + row) * LOG_CAP;
         int g = 0;   // key tiles consumed (accumulator buffer g & 1)
         for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
         const Item I = item_of(item);
         const int i = I.q0 + row;
         const int ntiles = I.kt1 - I.kt0;
-        float ls[KC];
-        int lj[KC];
+        const bool mine = i < I.row_end;
+        const float thr0v = (args.thr0 && i < args.n) ? __ldg(args.thr0 + i) : inf;
+        // this thread's R smallest scores, ascending (TOP1: the best score)
+        float ls[RL];
 #pragma unroll
-        for (int p = 0; p < KC; ++p) {
-            ls[p] = __int_as_float(0x7f800000);
-            lj[p] = -1;
-        }
-        const float thr0v = (args.thr0 && i < args.n) ? __ldg(args.thr0 + i)
-                                                      : __int_as_float(0x7f800000);
-        float thr = thr0v;
-        int cnt = 0;
-        // With two halves each list sees half the columns. A score at or above
-        // the other list's KC-th is not in the row's KC smallest (that list
-        // alone holds KC scores below it), so both filter with the smaller
-        // of the two thresholds.
-        auto partner_thr = [&]() {
-            return NH == 2 ? thr_sh[(1 - half) * BM + row] : __int_as_float(0x7f800000);
-        };
-        auto flush = [&]() {
-            const int mx = __reduce_max_sync(0xffffffffu, cnt);
-            const float pt = partner_thr();
-            if constexpr (KC >= 32) {
-                // eight staged candidates at a time: those still below the
-                // list's KC-th score are sorted and merged into the list
-                for (int q0 = 0; q0 < mx; q0 += 8) {
-                    const float lim = fminf(ls[KC - 1], pt);
-                    float bs[8];
-                    int bj[8];
-                    int nq = 0;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float sv = __int_as_float(0x7f800000);
-                        int jv = -1;
-                        if (q0 + c < cnt) {
-                            const float s = my_s[(q0 + c) * BM];
-                            const int j = my_j[(q0 + c) * BM];
-                            if ((args.cross || j != i) && s < lim) {
-                                sv = s;
-                                jv = j;
-                                ++nq;
-                            }
-                        }
-                        bs[c] = sv;
-                        bj[c] = jv;
-                    }
-                    // one merging network for any number of entries: a
-                    // single-insertion shortcut beside it measured slower
-                    // (instruction-fetch stalls from the larger loop body)
-                    if (__reduce_max_sync(0xffffffffu, nq) == 0) continue;
-                    topk::sort8(bs, bj);
-                    topk::merge8<KC>(ls, lj, bs, bj);
-                }
-            } else {
-                for (int q = 0; q < mx; ++q) {
-                    if (q < cnt) {
-                        float sv = my_s[q * BM];
-                        int jv = my_j[q * BM];
-                        if ((args.cross || jv != i) && sv < fminf(ls[KC - 1], pt))
-                            list_insert<KC>(ls, lj, sv, jv);
-                    }
-                }
-            }
-            cnt = 0;
-            if (NH == 2) thr_sh[half * BM + row] = ls[KC - 1];
-            thr = fminf(fminf(ls[KC - 1], pt), thr0v);
-        };
+        for (int p = 0; p < RL; ++p) ls[p] = inf;
+        int best_j = -1;
+        float T = inf;
+        int cnt = 0;        // log entries
+        bool over = false;  // the log does not hold every key at or below T
         bool ok = true;
         int my_comp = 0;
         if constexpr (MASK) my_comp = __ldg(args.colcomp + i);
         // FP8: acc = q_i . q_j, so x'_i . x'_j ~ s_i s_j acc
         float m2s = -2.0f;
         if constexpr (F8) m2s = -2.0f * (i < args.n ? __ldg(args.rscale + i) : 1.0f);
+        auto put = [&](float v) {   // into the sorted list; its largest drops out
+#pragma unroll
+            for (int p = 0; p < RL; ++p) {
+                const float lo = fminf(ls[p], v);
+                v = fmaxf(ls[p], v);
+                ls[p] = lo;
+            }
+        };
+        auto row_bound = [&]() {   // of the four lists as last published
+            return fmaxf(fmaxf(vt_sh[row], vt_sh[BM + row]),
+                         fmaxf(vt_sh[2 * BM + row], vt_sh[3 * BM + row]));
+        };
         for (int t = 0; t < ntiles; ++t, ++g) {
             const int b = g & 1, use = g >> 1;
             // every lane waits; the warp proceeds only if all lanes saw the phase
             const bool got = mbar_wait(&tfull[b], use & 1, abort_flag, args.status);
             if (!__all_sync(0xffffffffu, got)) {
                 ok = false;
+                if (!TOP1 && t == 0) epilogue_bar(32 * EPI);   // the others wait there
                 break;
             }
             tc_fence_after();
-            const uint32_t tb =
-                tmem + (uint32_t(quarter * 32) << 16) + uint32_t(b * BN + col0);
-            const int kt_this = ktile(I, t);
+            const uint32_t tb = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(b * BN + 16 * grp);
+            const int key0 = ktile(I, t) * BN + 16 * grp;
             // key norms (and components) of this tile's columns straight from
             // global memory: every lane reads the same addresses (L1 broadcast);
             // the next tile's are prefetched into L1 meanwhile
-            const float *nyt = args.ny + size_t(kt_this) * BN + col0;
-            const int *cmt = MASK ? args.colcomp + size_t(kt_this) * BN + col0 : nullptr;
-            if (t + 1 < ntiles && lane < ncols / 32) {
-                const size_t nxt = size_t(ktile(I, t + 1)) * BN + col0 + 32 * lane;
+            if (t + 1 < ntiles && lane < 4) {
+                const size_t nxt = size_t(ktile(I, t + 1)) * BN + 16 * grp + 64 * lane;
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(args.ny + nxt));
                 if constexpr (MASK) asm volatile("prefetch.global.L1 [%0];" ::"l"(args.colcomp + nxt));
             }
-            thr = fminf(thr, partner_thr());
-            // Candidate staging for 16 columns. The divergent part only touches
-            // this lane's stage; the warp-collective flush check sits at a
-            // warp-uniform point after it.
+            // one pass over the tile: the list, the log, or both
+            bool lists = true, logs = t > 0;
             auto process = [&](uint32_t(&v)[16], int ch) {
-                float mn = __int_as_float(0x7f800000);
+                const int k0 = key0 + 64 * ch;
+                float sc[16];
 #pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
-                    const float4 nn = __ldg(reinterpret_cast<const float4 *>(nyt + ch * 16 + 4 * c4));
-                    float4 cs = make_float4(m2s, m2s, m2s, m2s);
+                for (int q = 0; q < 4; ++q) {
                     if constexpr (F8) {   // per-key scales, same layout as the norms
-                        const float4 sk = __ldg(reinterpret_cast<const float4 *>(
-                            args.rscale + (nyt - args.ny) + ch * 16 + 4 * c4));
-                        cs = make_float4(m2s * sk.x, m2s * sk.y, m2s * sk.z, m2s * sk.w);
+                        const float4 nn = __ldg(reinterpret_cast<const float4 *>(args.ny + k0 + 4 * q));
+                        const float4 sk =
+                            __ldg(reinterpret_cast<const float4 *>(args.rscale + k0 + 4 * q));
+                        sc[4 * q + 0] = fmaf(m2s * sk.x, __uint_as_float(v[4 * q + 0]), nn.x);
+                        sc[4 * q + 1] = fmaf(m2s * sk.y, __uint_as_float(v[4 * q + 1]), nn.y);
+                        sc[4 * q + 2] = fmaf(m2s * sk.z, __uint_as_float(v[4 * q + 2]), nn.z);
+                        sc[4 * q + 3] = fmaf(m2s * sk.w, __uint_as_float(v[4 * q + 3]), nn.w);
+                    } else {
+                        const ulonglong2 nn =
+                            __ldg(reinterpret_cast<const ulonglong2 *>(args.ny + k0 + 4 * q));
+                        scores2(v[4 * q], v[4 * q + 1], nn.x, sc[4 * q], sc[4 * q + 1]);
+                        scores2(v[4 * q + 2], v[4 * q + 3], nn.y, sc[4 * q + 2], sc[4 * q + 3]);
                     }
-                    float s0 = fmaf(cs.x, __uint_as_float(v[4 * c4 + 0]), nn.x);
-                    float s1 = fmaf(cs.y, __uint_as_float(v[4 * c4 + 1]), nn.y);
-                    float s2 = fmaf(cs.z, __uint_as_float(v[4 * c4 + 2]), nn.z);
-                    float s3 = fmaf(cs.w, __uint_as_float(v[4 * c4 + 3]), nn.w);
                     if constexpr (MASK) {  // same component: not a candidate
-                        const int4 cc = __ldg(reinterpret_cast<const int4 *>(cmt + ch * 16 + 4 * c4));
-                        const float inf = __int_as_float(0x7f800000);
-                        s0 = cc.x == my_comp ? inf : s0;
-                        s1 = cc.y == my_comp ? inf : s1;
-                        s2 = cc.z == my_comp ? inf : s2;
-                        s3 = cc.w == my_comp ? inf : s3;
+                        const int4 cc = __ldg(reinterpret_cast<const int4 *>(args.colcomp + k0 + 4 * q));
+                        sc[4 * q + 0] = cc.x == my_comp ? inf : sc[4 * q + 0];
+                        sc[4 * q + 1] = cc.y == my_comp ? inf : sc[4 * q + 1];
+                        sc[4 * q + 2] = cc.z == my_comp ? inf : sc[4 * q + 2];
+                        sc[4 * q + 3] = cc.w == my_comp ? inf : sc[4 * q + 3];
                     }
-                    v[4 * c4 + 0] = __float_as_uint(s0);
-                    v[4 * c4 + 1] = __float_as_uint(s1);
-                    v[4 * c4 + 2] = __float_as_uint(s2);
-                    v[4 * c4 + 3] = __float_as_uint(s3);
-                    mn = fminf(mn, fminf(fminf(s0, s1), fminf(s2, s3)));
                 }
-                const int j0 = kt_this * BN + col0 + ch * 16;
-                if (mn < thr) {
+                float mn = inf;
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        float sc = __uint_as_float(v[c]);
-                        if (sc < thr) {
-                            my_s[cnt * BM] = sc;
-                            my_j[cnt * BM] = j0 + c;
-                            ++cnt;
-                        }
+                for (int q = 0; q < 4; ++q)
+                    mn = fminf(mn, fminf(fminf(sc[4 * q], sc[4 * q + 1]),
+                                         fminf(sc[4 * q + 2], sc[4 * q + 3])));
+                if constexpr (TOP1) {
+                    if (mn < ls[0]) {
+                        ls[0] = mn;
+                        int at = 0;
+#pragma unroll
+                        for (int c = 15; c >= 0; --c) at = sc[c] == mn ? c : at;
+                        best_j = k0 + at;
+                    }
+                    return;
+                }
+                // T is at or above this thread's own R-th: a chunk above T
+                // changes neither
+                if (!__any_sync(0xffffffffu, mn <= T)) return;
+                if (!logs) {   // first tile: every score into the list
+#pragma unroll 1
+                    for (int q = 0; q < 4; ++q) {   // four columns a turn, by select
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)
+                            put(q == 0 ? sc[c] : q == 1 ? sc[4 + c] : q == 2 ? sc[8 + c] : sc[12 + c]);
+                    }
+                } else {   // the scores at or below T into the log, and into the list
+                    unsigned bits = 0;
+                    if (mn <= T && mine) {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            bits |= (sc[c] <= T && sc[c] < inf) ? 1u << c : 0u;
+                        if (!args.cross && i >= k0 && i < k0 + 16) bits &= ~(1u << (i - k0));
+                    }
+                    // (cnt stays below LOG_CAP: at most 64 columns a tile)
+#pragma unroll 1
+                    while (bits) {
+                        const int c = __ffs(bits) - 1;
+                        bits &= bits - 1u;
+                        float x[8];   // the score of column c, by its bits
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) x[q] = (c & 1) ? sc[2 * q + 1] : sc[2 * q];
+#pragma unroll
+                        for (int w = 1; w < 4; ++w)
+#pragma unroll
+                            for (int q = 0; q < (8 >> w); ++q)
+                                x[q] = (c >> w) & 1 ? x[2 * q + 1] : x[2 * q];
+                        my_log[cnt] = make_int2(__float_as_int(x[0]), k0 + c);
+                        ++cnt;
+                        if (lists) put(x[0]);
                     }
                 }
-                // at most 16 more per chunk: flush before a stage could overflow
-                if (__any_sync(0xffffffffu, cnt > CAPB - 16)) flush();
+                __syncwarp();
             };
             // two 16-column register buffers: the load of chunk c+1 overlaps the
             // processing of chunk c
-            const int nch = ncols / 16;
-            uint32_t va[16], vb[16];
-            __syncwarp();
-            tmem_ld16(tb, va);
+            auto pass = [&]() {
+                uint32_t va[16], vb[16];
+                __syncwarp();
+                tmem_ld16(tb, va);
 #pragma unroll 1
-            for (int ch = 0; ch < nch; ch += 2) {
-                tmem_ld_wait16(va);
-                __syncwarp();
-                tmem_ld16(tb + (ch + 1) * 16, vb);
-                process(va, ch);
-                tmem_ld_wait16(vb);
-                __syncwarp();
-                if (ch + 2 < nch) tmem_ld16(tb + (ch + 2) * 16, va);
-                process(vb, ch + 1);
+                for (int ch = 0; ch < 4; ch += 2) {
+                    tmem_ld_wait16(va);
+                    __syncwarp();
+                    tmem_ld16(tb + (ch + 1) * 64, vb);
+                    process(va, ch);
+                    tmem_ld_wait16(vb);
+                    __syncwarp();
+                    if (ch + 2 < 4) tmem_ld16(tb + (ch + 2) * 64, va);
+                    process(vb, ch + 1);
+                }
+            };
+            // (one copy of the pass: the first tile takes a second turn)
+#pragma unroll 1
+            while (true) {
+                pass();
+                if (TOP1) break;
+                vt_sh[grp * BM + row] = ls[RL - 1];
+                if (t == 0 && lists) epilogue_bar(32 * EPI);
+                T = fminf(fminf(T, thr0v), row_bound());
+                if (t > 0 || !lists) break;
+                lists = false;
+                logs = true;
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[b]);
-        }
-        flush();
-        if (NH == 2) {
-            // merge: the second half's list goes through shared memory into the
-            // first half's (every epilogue warp reaches both barriers, on the
-            // error path too)
-            epilogue_bar(32 * EPI);
-            if (half == 1) {
-#pragma unroll
-                for (int p = 0; p < KC; ++p) {
-                    stg_s[p * BM + row] = ls[p];
-                    stg_j[p * BM + row] = lj[p];
+            if (!TOP1 && cnt > LOG_CAP - 64) {   // room for another tile: drop what T has ruled out
+                int w = 0;
+                for (int e = 0; e < cnt; ++e) {
+                    const int2 x = my_log[e];
+                    if (__int_as_float(x.x) <= T) my_log[w++] = x;
+                }
+                cnt = w;
+                if (cnt > LOG_CAP - 64) {   // masses of near ties: the row is not certified
+                    over = true;
+                    cnt = 0;
                 }
             }
-            epilogue_bar(32 * EPI);
-            if (half == 0) {
-                if constexpr (KC >= 32) {
-                    // the other list is ascending: batches of eight, until no
-                    // lane has an entry below its KC-th score
-                    for (int p0 = 0; p0 < KC; p0 += 8) {
-                        const float lim = ls[KC - 1];
-                        float bs[8];
-                        int bj[8];
-                        int nq = 0;
+            __syncwarp();
+        }
+        // (on a failed item others may still publish their first bounds)
+        if constexpr (TOP1) {   // the best of the row's four threads (smaller id on ties)
+            t_sh[grp * BM + row] = ls[0];
+            j_sh[grp * BM + row] = best_j;
+        } else {
+            j_sh[grp * BM + row] = over ? -1 : cnt;
+        }
+        // the logs are complete; a failure anywhere stops every warp here
+        const bool failed = epilogue_bar_any(32 * EPI, !ok);
+        if constexpr (TOP1) {
+            if (!failed && grp == 0 && mine) {
+                float s = t_sh[row];
+                int j = j_sh[row];
+                for (int q = 1; q < 4; ++q) {
+                    const float sq = t_sh[q * BM + row];
+                    const int jq = j_sh[q * BM + row];
+                    if (jq >= 0 && (j < 0 || sq < s || (sq == s && jq < j))) {
+                        s = sq;
+                        j = jq;
+                    }
+                }
+                args.cand[i - I.shift] = j >= 0 ? j - I.shift : -1;
+                args.splus[i - I.shift] = s;
+            }
+        } else if (!failed) {
+            // candidates: this warp's eight rows one after another
+            float *fs = f_sh + (warp - 2) * CAP;
+            int *fj = fj_sh + (warp - 2) * CAP;
+            const float ym = __uint_as_float(__ldg(args.ymax + I.cloud));
+#pragma unroll 1
+            for (int q = 0; q < BM / EPI; ++q) {
+                const int rr = (warp - 2) * (BM / EPI) + q;
+                const int ri = I.q0 + rr;
+                if (ri >= I.row_end) break;   // warp-uniform
+                float Tr = fmaxf(fmaxf(t_sh[rr], t_sh[BM + rr]),
+                                 fmaxf(t_sh[2 * BM + rr], t_sh[3 * BM + rr]));
+                if (ntiles == 0) Tr = inf;
+                if (args.thr0 && ri < args.n) Tr = fminf(Tr, __ldg(args.thr0 + ri));
+                bool lost = false;
+                int total = 0;
+                int2 pre[4][2];   // the first 64 entries of the four logs, in flight together
+                int c4[4];
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const float s = stg_s[(p0 + c) * BM + row];
-                            const bool in = s < lim;
-                            bs[c] = in ? s : __int_as_float(0x7f800000);
-                            bj[c] = in ? stg_j[(p0 + c) * BM + row] : -1;
-                            nq += in;
+                for (int gq = 0; gq < 4; ++gq) {
+                    const int c = j_sh[gq * BM + rr];
+                    lost |= c < 0;
+                    c4[gq] = c < 0 ? 0 : c;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int e = 32 * h + lane;
+                        pre[gq][h] = make_int2(0x7f800000, -1);
+                        if (e < c4[gq])
+                            pre[gq][h] = area[size_t(gq * BM + rr) * LOG_CAP + e];
+                    }
+                }
+                auto keep = [&](int2 x, bool have) {
+                    const bool in = have && __int_as_float(x.x) <= Tr;
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    const int to = total + __popc(m & ((1u << lane) - 1u));
+                    if (in && to < CAP) {
+                        fs[to] = __int_as_float(x.x);
+                        fj[to] = x.y;
+                    }
+                    total += __popc(m);
+                };
+#pragma unroll
+                for (int gq = 0; gq < 4; ++gq) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (32 * h < c4[gq]) keep(pre[gq][h], 32 * h + lane < c4[gq]);
+#pragma unroll 1
+                    for (int e0 = 64; e0 < c4[gq]; e0 += 32) {
+                        const bool have = e0 + lane < c4[gq];
+                        int2 x = make_int2(0x7f800000, -1);
+                        if (have) x = area[size_t(gq * BM + rr) * LOG_CAP + e0 + lane];
+                        keep(x, have);
+                    }
+                }
+                lost |= total > CAP;
+                const int kept = min(total, CAP);
+                __syncwarp();
+                float sv[4];
+                float lo = inf, hi = -inf;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const bool have = 32 * h + lane < kept;
+                    sv[h] = have ? fs[32 * h + lane] : inf;
+                    lo = fminf(lo, sv[h]);
+                    hi = have ? fmaxf(hi, sv[h]) : hi;
+                }
+                float sp = Tr;
+                if (!lost && kept > args.sel.k + 1) {
+#pragma unroll
+                    for (int o = 16; o >= 1; o >>= 1) {
+                        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+                    }
+                    auto count = [&](float t) {
+                        int c = 0;
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)
+                            c += __popc(__ballot_sync(0xffffffffu, sv[h] <= t));
+                        return c;
+                    };
+                    // (all keys up to Tr are in the log)
+                    sp = select_bound(count, lo, hi, Tr, args.sel, sqrtf(__ldg(args.ny + ri)), ym);
+                }
+                // out: the candidates at or below sp
+                const size_t at0 =
+                    (I.part > 0 ? size_t(I.part - 1) * BM + rr : size_t(ri - I.shift)) *
+                    size_t(args.cap);
+                int out = 0;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const bool in = 32 * h + lane < kept && sv[h] <= sp;
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    const int to_row = out + __popc(m & ((1u << lane) - 1u));
+                    if (in && to_row < args.cap) {
+                        const size_t to = at0 + to_row;
+                        const int j = fj[32 * h + lane] - I.shift;
+                        if (I.part > 0) {
+                            args.side_j[to] = j;
+                            args.side_s[to] = sv[h];
+                        } else {
+                            args.cand[to] = j;
                         }
-                        if (__reduce_max_sync(0xffffffffu, nq) == 0) break;
-                        topk::merge8<KC>(ls, lj, bs, bj);
                     }
-                } else {
-                    for (int p = 0; p < KC; ++p) {   // ascending: stop at the first that cannot enter
-                        const float sv = stg_s[p * BM + row];
-                        if (!(sv < ls[KC - 1])) break;
-                        list_insert<KC>(ls, lj, sv, stg_j[p * BM + row]);
+                    out += __popc(m);
+                }
+                if (out > args.cap) {   // ties at the bound
+                    lost = true;
+                    out = args.cap;
+                }
+                if (lane == 0) {
+                    if (lost) sp = -inf;   // never certified
+                    if (I.part > 0) {
+                        const size_t at = size_t(I.part - 1) * BM + rr;
+                        args.side_cnt[at] = out;
+                        args.side_splus[at] = sp;
+                    } else {
+                        args.ccnt[ri - I.shift] = out;
+                        args.splus[ri - I.shift] = sp;
                     }
                 }
+                __syncwarp();
             }
         }
-        if (ok && half == 0 && i < I.row_end) {
-            if constexpr (KC == 1) {   // top-1 mode: the best key and its score
-                args.cand[i - I.shift] = lj[0] >= 0 ? lj[0] - I.shift : -1;
-            } else if (I.part > 0) {   // one part of a split list: scores too, for the merge
-                const size_t at = size_t(I.part - 1) * BM + row;
-                int32_t *oj = args.side_j + at * (KC - 1);
-                float *os = args.side_s + at * (KC - 1);
-#pragma unroll
-                for (int p = 0; p < KC - 1; ++p) {
-                    oj[p] = lj[p] >= 0 ? lj[p] - I.shift : -1;
-                    os[p] = ls[p];
-                }
-                args.side_splus[at] = fminf(ls[KC - 1], thr0v);
-            } else {
-                int32_t *out = args.cand + size_t(i - I.shift) * (KC - 1);
-#pragma unroll
-                for (int p = 0; p < KC - 1; ++p) out[p] = lj[p] >= 0 ? lj[p] - I.shift : -1;
-            }
-            // keys that never entered the list scored at least min(KC-th, thr0)
-            if (KC == 1 || I.part == 0) args.splus[i - I.shift] = fminf(ls[KC - 1], thr0v);
-        }
-        // next item: this row's published threshold starts over, and the
-        // staging area is free again; a failure anywhere stops every warp here
-        if (NH == 2) thr_sh[half * BM + row] = __int_as_float(0x7f800000);
-        if (epilogue_bar_any(32 * EPI, !ok)) break;
+        // the next item reuses the logs, the counts and the bounds
+        epilogue_bar(32 * EPI);
+        if (failed) break;
         }
     }
     tc_fence_before();
@@ -587,49 +755,88 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
+    if constexpr (!TOP1) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicExch(args.claim + *slot_sh, 0);
+        }
+    }
 }
 
-// Rows of split query tiles (one block of BM threads per split tile): the
-// row's candidates are the KC - 1 smallest scores over its parts' lists and
-// s+ = min(the KC-th smallest of those lists, every part's s+). A key that
-// no part kept scored at least its part's s+; a kept key left out here
-// scored at least the KC-th. So the row gets the candidates and s+ the
-// unsplit list would have had (up to the order of equal scores).
-template <int KC>
-__global__ void __launch_bounds__(BM)
+// Rows of split query tiles (a warp per row, blockIdx.y = 16 rows of split
+// tile blockIdx.x): s+ = the smallest of the parts' s+ (every key of the
+// others at or below it is among their candidates), lowered like a whole
+// list's; candidates = the parts' candidates at or below it.
+__global__ void __launch_bounds__(512)
 split_merge_kernel(const int32_t *__restrict__ splitq, const int32_t *__restrict__ nsplit,
                    const int32_t *__restrict__ side_j, const float *__restrict__ side_s,
-                   const float *__restrict__ side_splus, int64_t n, int32_t *__restrict__ cand,
-                   float *__restrict__ splus) {
+                   const int32_t *__restrict__ side_cnt, const float *__restrict__ side_splus,
+                   int64_t n, Select sel, const float *__restrict__ ny,
+                   const unsigned *__restrict__ ymax, int32_t *__restrict__ cand,
+                   int32_t *__restrict__ ccnt, float *__restrict__ splus) {
     if (int(blockIdx.x) >= __ldg(nsplit)) return;
     const int q = splitq[3 * blockIdx.x], slot0 = splitq[3 * blockIdx.x + 1];
     const int P = splitq[3 * blockIdx.x + 2];
-    const int row = threadIdx.x;
+    const int row = int(blockIdx.y) * 16 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int64_t i = int64_t(q) * BM + row;
     if (i >= n) return;
-    float ls[KC];
-    int lj[KC];
+    const float inf = __int_as_float(0x7f800000);
+    float T = inf;
+    for (int p = lane; p < P; p += 32) T = fminf(T, side_splus[size_t(slot0 + p) * BM + row]);
 #pragma unroll
-    for (int p = 0; p < KC; ++p) {
-        ls[p] = __int_as_float(0x7f800000);
-        lj[p] = -1;
-    }
-    float sp = __int_as_float(0x7f800000);
-    for (int part = 0; part < P; ++part) {
-        const size_t at = size_t(slot0 + part) * BM + row;
-        sp = fminf(sp, side_splus[at]);
-        const float *ps = side_s + at * (KC - 1);
-        const int32_t *pj = side_j + at * (KC - 1);
-        for (int p = 0; p < KC - 1; ++p) {   // ascending: stop at the first that cannot enter
-            const float sv = ps[p];
-            if (!(sv < ls[KC - 1])) break;
-            list_insert<KC>(ls, lj, sv, pj[p]);
+    for (int o = 16; o >= 1; o >>= 1) T = fminf(T, __shfl_xor_sync(0xffffffffu, T, o));
+    const int cap = sel.cap;
+    float lo = inf, hi = -inf;
+    int have = 0;   // candidates of the parts up to T
+    for (int p = 0; p < P; ++p) {
+        const size_t at = size_t(slot0 + p) * BM + row;
+        const int c = side_cnt[at];   // <= cap
+        for (int e = lane; e < c; e += 32) {
+            const float s = side_s[at * cap + e];
+            if (s <= T) {
+                lo = fminf(lo, s);
+                hi = fmaxf(hi, s);
+                ++have;
+            }
         }
     }
-    int32_t *out = cand + i * (KC - 1);
 #pragma unroll
-    for (int p = 0; p < KC - 1; ++p) out[p] = lj[p];
-    splus[i] = fminf(ls[KC - 1], sp);
+    for (int o = 16; o >= 1; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        have += __shfl_xor_sync(0xffffffffu, have, o);
+    }
+    if (have > sel.k + 1) {
+        auto count = [&](float t) {
+            int c = 0;
+            for (int p = 0; p < P; ++p) {
+                const size_t at = size_t(slot0 + p) * BM + row;
+                const int cp = side_cnt[at];
+                for (int e0 = 0; e0 < cp; e0 += 32)
+                    c += __popc(__ballot_sync(
+                        0xffffffffu, e0 + lane < cp && side_s[at * cap + e0 + lane] <= t));
+            }
+            return c;
+        };
+        T = select_bound(count, lo, hi, T, sel, sqrtf(ny[i]), __uint_as_float(*ymax));
+    }
+    int total = 0;
+    for (int p = 0; p < P; ++p) {
+        const size_t at = size_t(slot0 + p) * BM + row;
+        const int c = side_cnt[at];
+        for (int e0 = 0; e0 < c; e0 += 32) {
+            const int e = e0 + lane;
+            const bool in = e < c && side_s[at * cap + e] <= T;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            const int to = total + __popc(m & ((1u << lane) - 1u));
+            if (in && to < cap) cand[i * cap + to] = side_j[at * cap + e];
+            total += __popc(m);
+        }
+    }
+    if (lane == 0) {
+        ccnt[i] = total < cap ? total : cap;
+        splus[i] = total <= cap ? T : -inf;   // more ties than places: not certified
+    }
 }
 
 // ------------------------------------------------------------- prep
@@ -817,14 +1024,73 @@ __global__ void thr0_kernel(const float *__restrict__ tau_row, const float *__re
 
 // ------------------------------------------------------------- rerank
 
+// relative error of the tensor-core dot of BF16 operands, split (x3) or not:
+// products and accumulation over the padded columns
+__host__ __device__ inline double tc_eps_dot(int d_pad, bool x3) {
+    const double u8 = 1.0 / 256.0;
+    const double kprod = double(x3 ? 3 * d_pad : d_pad);
+    return (x3 ? (3.0 * u8 * u8 + 3.0 * u8 * u8 * u8 + u8 * u8 * u8 * u8)
+               : (2.0 * u8 + u8 * u8)) +
+           kprod * (1.0 / 4194304.0) * (1.0 + 4.0 * u8);
+}
+// the FP32 terms (norms, score rounding, canonical distance on both sides)
+inline float score_eps_row(int d) { return float(4.0 * (d + 8.0) / 16777216.0); }
+
 struct CertConst {
     double eps_dot;   // relative error of the tensor-core dot (products + accumulation)
-    double d_plus;    // d + 4, for the canonical distance error
+    float e32, c32, w32;   // 2.02 eps_dot and (d + 1) u 1.02 rounded up, 1 - (d + 4) u 1.05 down
 };
+inline CertConst cert_const(double eps_dot, int d) {
+    const double u = 1.0 / 16777216.0, up = 1.0 + 0x1p-22;
+    return CertConst{eps_dot, float(2.02 * eps_dot * up), float((d + 1) * u * 1.02 * up),
+                     float((1.0 - (d + 4.0) * u * 1.05) * (1.0 - 0x1p-22))};
+}
 
-// One warp per row: canonical distances of the k' candidates, bitonic sort
-// of (w, id), top k, certificate. Row i's point is xi; candidate ids index
-// rows of X (row stride ld, chain length dc >= d: columns beyond d are zero
+// Whether no key left out can be at a canonical distance <= kw: keys of
+// skipped tiles lie at a true distance >= skip, other keys left out have a
+// score above sp. First in FP32 with every rounding on the safe side, which
+// decides all but near ties; then in FP64. (The FP64 form alone, some sixty
+// operations with two square roots in every warp at this GPU's two FP64
+// lanes per SM and clock, held the re-rank back: 10.4 -> 6.6 ms
+// for 256 clouds of 500 to 20,000 points.)
+template <class Eps64>
+__device__ __forceinline__ bool certified(float kw, float skip, float sp, float xn2f, float ymf,
+                                          int d, const CertConst &cc, Eps64 eps64) {
+    const float inf = __int_as_float(0x7f800000);
+    {
+        const float u = 0x1p-24f;
+        const float xn = __fsqrt_ru(xn2f), xy = __fmul_ru(xn, ymf), yy = __fmul_ru(ymf, ymf);
+        // the terms of the FP64 form below, each rounded up
+        const float E = __fadd_ru(
+            __fadd_ru(__fmul_ru(cc.e32, xy), __fmul_ru(cc.c32, yy)),
+            __fadd_ru(__fmul_ru(2.03f * u, __fadd_ru(yy, __fmul_ru(2.0f, xy))), 1.1e-30f));
+        const float p = __fsub_rd(__fadd_rd(xn2f, sp), __fadd_ru(E, __fmul_ru(cc.c32, xn2f)));
+        const float lo = __fsub_rd(p > 0.0f ? __fsqrt_rd(p) : 0.0f,
+                                   __fmul_ru(1.03f * u, __fadd_ru(xn, ymf)));
+        const bool skip_ok = !(skip < inf) || __fmul_rd(skip, cc.w32) > kw;
+        if (skip_ok && (!(sp < inf) || (lo > 0.0f && __fmul_rd(lo, cc.w32) > kw))) return true;
+    }
+    const double u24 = 1.0 / 16777216.0;
+    // their canonical distance is above kw when skip (1 - eps_canon) is
+    if (skip < inf && !(double(skip) * (1.0 - (d + 4.0) * u24 * 1.05) > double(kw))) return false;
+    if (!(sp < inf)) return true;   // no bound: every visited key was kept
+    const double xn2 = double(xn2f);
+    const double xn = sqrt(xn2);
+    const double ym = double(ymf);
+    // |s~ - s| <= E: tensor-core dot, FP32 key norm, score rounding
+    const double E = 2.0 * eps64() * xn * ym * 1.01 + (d + 1) * u24 * 1.02 * ym * ym +
+                     2.0 * u24 * (ym * ym + 2.0 * xn * ym) * 1.01 + 1e-30;
+    // lower bound on the centred squared distance of any unkept point
+    const double p_lo = xn2 * (1.0 - (d + 1) * u24 * 1.02) + double(sp) - E;
+    const double dist_lo =
+        (p_lo > 0.0 ? sqrt(p_lo) : 0.0) - 1.02 * u24 * (xn + ym);  // centring rounding
+    const double w_lo = dist_lo * (1.0 - (d + 4.0) * u24 * 1.05);  // canonical FP32 error
+    return w_lo > double(kw);
+}
+
+// One warp per row: canonical distances of its cnt candidates, bitonic sort
+// of (w, id), top k, certificate (sp: every key left out scored above it).
+// Row i's point is xi; candidate ids index rows of X (row stride ld, chain length dc >= d: columns beyond d are zero
 // and leave the canonical distance unchanged). d is the true dimension used in
 // the error bounds. Returns whether the row was certified (then the k
 // results are written).
@@ -832,19 +1098,30 @@ struct CertConst {
 // canonical partial) of every candidate from coalesced row reads, the query
 // row held in registers, and the warp sums the partials of a batch of
 // candidates at once (below); XR = 0: one candidate per lane, its 32
-// partials in registers.
-template <int VEC, int KC, int XR = 0>
+// partials in registers. H: a list holds at most 32 H <= CAP candidates.
+// Bound: issue slots (a candidate's 4 loads, 8 FP32 operations and 3 shuffles
+// per lane at d = 128) at 68 % of peak. With about k + 3 candidates instead of
+// 4 R - 1, half batches, and the certificate's FP64 out of the common way: 1M
+// rows at k = 32 3.45 -> 2.59 ms, 256 clouds (2.6M rows, k = 16) 8.4 -> 6.6 ms.
+template <int XR, int H, class Eps64>
 __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, int dc, int d,
                                            const float *__restrict__ xi, int k,
-                                           const int32_t *__restrict__ cand_row, float sp,
-                                           float skip, float xn2f, float ymf, double eps_dot,
-                                           int lane,
+                                           const int32_t *__restrict__ cand_row, int cnt, float sp,
+                                           float skip, float xn2f, float ymf,
+                                           const CertConst &cc, Eps64 eps64, int lane,
                                            int32_t *__restrict__ nbr_row,
                                            float *__restrict__ dist_row,
                                            const int32_t *__restrict__ idmap = nullptr,
                                            uint64_t *kth_out = nullptr) {
-    constexpr int KP = KC - 1;
-    uint64_t key[2];
+    const int kp = cnt;   // <= 32 H
+    uint64_t key[H];
+    int jc[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        key[h] = KEY_NONE;
+        const int c = h * 32 + lane;
+        jc[h] = c < kp ? cand_row[c] : -1;
+    }
     if constexpr (XR > 0) {
         // batches of NB candidates: lane l's partial of candidate c in
         // acc[c mod NB]; the butterfly's steps xor 16 .. xor NB on all NB,
@@ -857,48 +1134,56 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
         // register budget; NB = 1 is the plain butterfly)
         constexpr int NB = XR <= 4 ? 16 : (XR <= 8 ? 2 : 1);
         constexpr int G = XR <= 8 ? 2 : 1;   // candidates with loads in flight
-        static_assert(NB % G == 0, "a batch is whole load groups");
+        constexpr int PB = NB == 16 ? 8 : NB;   // a whole or half batch
+        static_assert(PB % G == 0, "a part is whole load groups");
         float xr[XR];
 #pragma unroll
         for (int q = 0; q < XR; ++q) {
             const int t = lane + 32 * q;
             xr[q] = t < dc ? __ldg(xi + t) : 0.0f;
         }
-        int jc[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int c = h * 32 + lane;
-            jc[h] = c < KP ? cand_row[c] : -1;
-        }
-        key[0] = key[1] = KEY_NONE;
 #pragma unroll 1
-        for (int b = 0; b < (KP + NB - 1) / NB; ++b) {
+        for (int b = 0; b < (kp + NB - 1) / NB; ++b) {
+            const int hb = (NB * b) >> 5;   // a batch lies in one register of the list
+            int jb = jc[0];
+#pragma unroll
+            for (int h = 1; h < H; ++h) jb = hb == h ? jc[h] : jb;
             float acc[NB];
+            auto part = [&](auto first) {   // candidates first .. first + PB - 1 of the batch
 #pragma unroll
-            for (int g0 = 0; g0 < NB; g0 += G) {
-                int j[G];
-                float y[G][XR];
+                for (int g1 = 0; g1 < PB; g1 += G) {
+                    const int g0 = first.value + g1;
+                    int j[G];
+                    float y[G][XR];
 #pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    const int c = NB * b + g0 + g;
-                    const int ja = __shfl_sync(0xffffffffu, jc[0], c & 31);
-                    const int jb = __shfl_sync(0xffffffffu, jc[1], c & 31);
-                    j[g] = c < KP ? (c < 32 ? ja : jb) : -1;
+                    for (int g = 0; g < G; ++g) {
+                        j[g] = __shfl_sync(0xffffffffu, jb, (NB * b + g0 + g) & 31);
 #pragma unroll
-                    for (int q = 0; q < XR; ++q) {
-                        const int t = lane + 32 * q;
-                        y[g][q] = (j[g] >= 0 && t < dc) ? __ldg(X + int64_t(j[g]) * ld + t) : 0.0f;
+                        for (int q = 0; q < XR; ++q) {
+                            const int t = lane + 32 * q;
+                            y[g][q] =
+                                (j[g] >= 0 && t < dc) ? __ldg(X + int64_t(j[g]) * ld + t) : 0.0f;
+                        }
+                    }
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        float p = 0.0f;
+#pragma unroll
+                        for (int q = 0; q < XR; ++q) {
+                            const float dl = __fsub_rn(xr[q], y[g][q]);
+                            p = __fmaf_rn(dl, dl, p);
+                        }
+                        acc[g0 + g] = p;
                     }
                 }
+            };
+            part(std::integral_constant<int, 0>{});
+            if constexpr (NB > PB) {   // the last batch's second half is often empty
+                if (kp - NB * b > PB) {
+                    part(std::integral_constant<int, PB>{});
+                } else {
 #pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    float p = 0.0f;
-#pragma unroll
-                    for (int q = 0; q < XR; ++q) {
-                        const float dl = __fsub_rn(xr[q], y[g][q]);
-                        p = __fmaf_rn(dl, dl, p);
-                    }
-                    acc[g0 + g] = p;
+                    for (int i = PB; i < NB; ++i) acc[i] = 0.0f;
                 }
             }
 #pragma unroll
@@ -919,85 +1204,34 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
             // candidate c of this lane; sort element c (register c / 32 of
             // lane c mod 32) takes it from the lane of the matching block
             const int c = NB * b + (lane & (NB - 1));
-            const int ja = __shfl_sync(0xffffffffu, jc[0], c & 31);
-            const int jb = __shfl_sync(0xffffffffu, jc[1], c & 31);
-            const int jl = c < KP ? (c < 32 ? ja : jb) : -1;
+            const int jl = __shfl_sync(0xffffffffu, jb, c & 31);
             if ((lane & ~(NB - 1)) == ((NB * b) & 31) && jl >= 0) {
                 const uint64_t kg = nb_key(__fsqrt_rn(acc[0]), uint32_t(idmap ? idmap[jl] : jl));
-                if (c < 32) key[0] = kg;
-                else key[1] = kg;
+#pragma unroll
+                for (int h = 0; h < H; ++h)
+                    if (h == hb) key[h] = kg;
             }
         }
     } else {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            int c = h * 32 + lane;
-            key[h] = KEY_NONE;
-            if (c < KP) {
-                int j = cand_row[c];
-                if (j >= 0)
-                    key[h] = nb_key(canon_dist<VEC>(xi, X + int64_t(j) * ld, dc),
-                                    uint32_t(idmap ? idmap[j] : j));
-            }
-        }
+        for (int h = 0; h < H; ++h)
+            if (jc[h] >= 0)
+                key[h] = nb_key(canon_dist<1>(xi, X + int64_t(jc[h]) * ld, dc),
+                                uint32_t(idmap ? idmap[jc[h]] : jc[h]));
     }
-    // bitonic sort of 64 keys, element index = h*32 + lane
-#pragma unroll
-    for (int size = 2; size <= 64; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride == 32) {
-                // partner is the other register of the same lane (size == 64: ascending)
-                uint64_t lo = key[0] < key[1] ? key[0] : key[1];
-                uint64_t hi = key[0] < key[1] ? key[1] : key[0];
-                key[0] = lo;
-                key[1] = hi;
-            } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    int idx = h * 32 + lane;
-                    bool asc = ((idx & size) == 0);
-                    uint64_t other = shfl_xor_u64(key[h], stride);
-                    bool lower = (lane & stride) == 0;
-                    uint64_t mn = key[h] < other ? key[h] : other;
-                    uint64_t mx = key[h] < other ? other : key[h];
-                    key[h] = (lower == asc) ? mn : mx;
-                }
-            }
-        }
+    // sort by (w, id), as many registers as the candidates fill
+    if (kp <= 32) {
+        uint64_t one[1] = {key[0]};
+        warp_sort_regs<1>(one, lane);
+        key[0] = one[0];
+    } else {
+        warp_sort_regs<H>(key, lane);
     }
     // k-th key (index k-1)
-    const int kh = (k - 1) >> 5, kl = (k - 1) & 31;
-    uint64_t kth = __shfl_sync(0xffffffffu, kh ? key[1] : key[0], kl);
+    const int kh = (k - 1) >> 5, kl = (k - 1) & 31;   // k <= 63
+    const uint64_t kth = __shfl_sync(0xffffffffu, kh ? key[1] : key[0], kl);
     if (kth_out) *kth_out = kth;
-    bool cert = false;
-    if (lane == 0) {
-        const double u24c = 1.0 / 16777216.0;
-        // keys of skipped tiles lie at true distance >= skip; their canonical
-        // distance is then above the k-th when skip (1 - eps_canon) is
-        const bool skip_ok = !(skip < __int_as_float(0x7f800000)) ||
-                             double(skip) * (1.0 - (d + 4.0) * u24c * 1.05) > double(key_w(kth));
-        if (!skip_ok) {
-            cert = false;
-        } else if (!(sp < __int_as_float(0x7f800000))) {
-            cert = true;  // fewer than KC points besides i among the visited keys: all kept
-        } else {
-            const double u24 = 1.0 / 16777216.0;
-            const double xn2 = double(xn2f);
-            const double xn = sqrt(xn2);
-            const double ym = double(ymf);
-            // |s~ - s| <= E: tensor-core dot, FP32 key norm, score rounding
-            const double E = 2.0 * eps_dot * xn * ym * 1.01 + (d + 1) * u24 * 1.02 * ym * ym +
-                             2.0 * u24 * (ym * ym + 2.0 * xn * ym) * 1.01 + 1e-30;
-            // lower bound on the centred squared distance of any unkept point
-            const double p_lo = xn2 * (1.0 - (d + 1) * u24 * 1.02) + double(sp) - E;
-            const double dist_lo =
-                (p_lo > 0.0 ? sqrt(p_lo) : 0.0) - 1.02 * u24 * (xn + ym);  // centring rounding
-            const double w_lo = dist_lo * (1.0 - (d + 4.0) * u24 * 1.05);  // canonical FP32 error
-            cert = w_lo > double(key_w(kth));
-        }
-    }
-    cert = __shfl_sync(0xffffffffu, cert, 0);
+    const bool cert = certified(key_w(kth), skip, sp, xn2f, ymf, d, cc, eps64);   // warp-uniform
     if (cert) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -1011,10 +1245,10 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
     return cert;
 }
 
-template <int VEC, int KC, int XR>
+template <int XR, int H>
 __global__ void rerank_kernel(const float *__restrict__ X, int64_t n, int d, int k,
-                              const int32_t *__restrict__ cand, const float *__restrict__ splus,
-                              const float *__restrict__ skip,
+                              const int32_t *__restrict__ cand, const int32_t *__restrict__ ccnt,
+                              const float *__restrict__ splus, const float *__restrict__ skip,
                               const float *__restrict__ xnorm2, const unsigned *__restrict__ ymax_bits,
                               CertConst cc, int32_t *__restrict__ nbr, float *__restrict__ dist,
                               int32_t *__restrict__ fail_rows, int32_t *__restrict__ fail_count) {
@@ -1022,8 +1256,8 @@ __global__ void rerank_kernel(const float *__restrict__ X, int64_t n, int d, int
     int lane = threadIdx.x & 31;
     if (i >= n) return;
     const float sk = skip ? skip[i] : __int_as_float(0x7f800000);
-    bool cert = rerank_row<VEC, KC, XR>(X, d, d, d, X + i * d, k, cand + i * (KC - 1), splus[i], sk,
-                                    xnorm2[i], __uint_as_float(*ymax_bits), cc.eps_dot, lane,
+    bool cert = rerank_row<XR, H>(X, d, d, d, X + i * d, k, cand + i * (32 * H), ccnt[i], splus[i], sk,
+                                    xnorm2[i], __uint_as_float(*ymax_bits), cc, [&] { return cc.eps_dot; }, lane,
                                     nbr + i * k, dist + i * k);
     if (!cert && lane == 0) fail_rows[atomicAdd(fail_count, 1)] = int32_t(i);
 }
@@ -1032,9 +1266,11 @@ __global__ void rerank_kernel(const float *__restrict__ X, int64_t n, int d, int
 // candidate rows are read from the sorted copy Xs (a row's candidates are
 // mostly cell-mates, so they sit close together in memory), keyed and
 // written with their original ids.
-template <int VEC, int KC, int XR>
-__global__ void __launch_bounds__(256, 5) rerank_sorted_kernel(const float *__restrict__ Xs, int64_t n, int d, int k,
+template <int XR, int H>
+__global__ void __launch_bounds__(256, H == 2 ? 5 : 3)
+rerank_sorted_kernel(const float *__restrict__ Xs, int64_t n, int d, int k,
                                      const int32_t *__restrict__ cand,
+                                     const int32_t *__restrict__ ccnt,
                                      const float *__restrict__ splus,
                                      const float *__restrict__ skipQ,
                                      const int32_t *__restrict__ perm,
@@ -1049,9 +1285,9 @@ __global__ void __launch_bounds__(256, 5) rerank_sorted_kernel(const float *__re
     if (r >= n) return;
     const int64_t i = perm[r];
     uint64_t kth;
-    const bool cert = rerank_row<VEC, KC, XR>(Xs, d, d, d, Xs + r * d, k, cand + r * (KC - 1),
+    const bool cert = rerank_row<XR, H>(Xs, d, d, d, Xs + r * d, k, cand + r * (32 * H), ccnt[r],
                                           splus[r], skipQ[r / BM], xnorm2[i],
-                                          __uint_as_float(*ymax_bits), cc.eps_dot, lane,
+                                          __uint_as_float(*ymax_bits), cc, [&] { return cc.eps_dot; }, lane,
                                           nbr + i * k, dist + i * k, perm, &kth);
     if (!cert && lane == 0) {
         const int s = atomicAdd(fail_count, 1);
@@ -1075,14 +1311,16 @@ __device__ __forceinline__ int cloud_of(const long long *__restrict__ off, int B
 // perm (may be null): the rows are in a spatial order within each cloud and
 // perm[v] is the compact id of row v; candidate ids are mapped through it
 // and the results written at the original row.
-template <int KC, int XR>
-__global__ void rerank_batched_kernel(const float *__restrict__ Xc, int ld, int64_t N,
+template <int XR, int H>
+__global__ void __launch_bounds__(256, H == 2 ? 4 : 3)
+rerank_batched_kernel(const float *__restrict__ Xc, int ld, int64_t N,
                                       const long long *__restrict__ voff, int B,
                                       const CloudDev *__restrict__ cl, int x3, int k,
                                       const int32_t *__restrict__ cand,
+                                      const int32_t *__restrict__ ccnt,
                                       const float *__restrict__ splus,
                                       const float *__restrict__ xnorm2,
-                                      const unsigned *__restrict__ ymax_bits,
+                                      const unsigned *__restrict__ ymax_bits, CertConst cc,
                                       const int32_t *__restrict__ perm,
                                       int32_t *__restrict__ nbr, float *__restrict__ dist,
                                       int32_t *__restrict__ fail_rows,
@@ -1093,16 +1331,12 @@ __global__ void rerank_batched_kernel(const float *__restrict__ Xc, int ld, int6
     const int b = cloud_of(voff, B, v);
     const CloudDev c = cl[b];
     if (!c.use_tc) return;
-    const double u8 = 1.0 / 256.0;
-    const double kprod = double(x3 ? 3 * c.d_pad : c.d_pad);
-    const double eps = (x3 ? (3.0 * u8 * u8 + 3.0 * u8 * u8 * u8 + u8 * u8 * u8 * u8)
-                           : (2.0 * u8 + u8 * u8)) +
-                       kprod * (1.0 / 4194304.0) * (1.0 + 4.0 * u8);
     const int dc = (c.d + 3) & ~3;
     const int64_t pv = perm ? int64_t(perm[v]) : v;
-    bool cert = rerank_row<4, KC, XR>(Xc, ld, dc, c.d, Xc + v * ld, k, cand + v * (KC - 1), splus[v],
+    bool cert = rerank_row<XR, H>(Xc, ld, dc, c.d, Xc + v * ld, k, cand + v * (32 * H), ccnt[v], splus[v],
                                   __int_as_float(0x7f800000),
-                                  xnorm2[v], __uint_as_float(ymax_bits[b]), eps, lane, nbr + pv * k,
+                                  xnorm2[v], __uint_as_float(ymax_bits[b]), cc,
+                                  [&] { return tc_eps_dot(c.d_pad, x3); }, lane, nbr + pv * k,
                                   dist + pv * k, perm);
     if (!cert && lane == 0) fail_rows[atomicAdd(fail_count, 1)] = int32_t(pv);
 }
@@ -1239,59 +1473,85 @@ __global__ void top1_merge_kernel(const int32_t *__restrict__ c2, const float *_
 }
 
 struct TcPlan {
-    int d_pad, nkb, kh, stages, kc, epi;
+    int d_pad, nkb, kh, stages, r, cap;
     int64_t nq_tiles, nk_tiles;
     size_t smem;
 };
 
-// allow8: eight epilogue warps when the candidate lists fit the merge area
-// (KC <= 2 CAPB) and the larger staging area still leaves three B stages
 // f8: E4M3 operand rows, 128 elements (128 bytes) per K block
-TcPlan tc_plan(int64_t n, int d, int k, bool x3, bool allow8 = true, bool f8 = false) {
+TcPlan tc_plan(int64_t n, int d, int k, bool x3, bool f8 = false) {
     TcPlan p{};
     const int kel = f8 ? 2 * BK : BK;   // elements per 128-byte K block
     p.d_pad = (d + kel - 1) / kel * kel;
     p.nkb = p.d_pad / kel;
     p.kh = (x3 ? 2 : 1) * p.d_pad;
-    // keep at least ~10 candidates beyond k so that the certificate has a
-    // gap to work with: k <= 21 -> 31 candidates, k <= 37 -> 47, k <= 63 -> 63
-    p.kc = (k <= 21) ? 32 : (k <= 37 ? 48 : 64);
+    // R, the minima kept per thread: 4 R keys at least stay in a row's log, of
+    // which k + 1 plus the margin are wanted. A smaller R is cheaper per tile
+    // and leaves more rows uncertified, each of which is redone exactly. At
+    // k = 16, R = 6 / 8 / 10: 100,000 x 128 blobs 1.12 / 1.18 / 1.26 ms of tiles
+    // and 1928 / 96 / 2 rows redone; 256 clouds of 500 to 20,000 points 22.5 /
+    // 23.5 / 26.4 ms of tiles, 56.6 / 51.1 / 54.3 ms in all. At k = 32, R = 10 /
+    // 12 / 14: 1M x 128 sphere points 7.6 / 8.1 / 8.4 ms, but 40 keys leave
+    // overlapping clusters a margin of seven.
+    p.r = k <= 7 ? 4 : (k <= 21 ? 8 : (k <= 37 ? 12 : 16));
+    // (twice the places cost the re-rank two more key registers: 5.4 against
+    // 3.5 ms at 1M rows and k = 32)
+    p.cap = p.r <= 12 ? 64 : CAP;
     p.nq_tiles = (n + BM - 1) / BM;
     p.nk_tiles = (n + BN - 1) / BN;
     const size_t cap = 227 * 1024;
-    auto fixed_for = [&](int nh) {
-        return 1024 + size_t(x3 ? 2 : 1) * p.nkb * A_BLOCK + size_t(nh) * CAPB * BM * 8 +
-               2 * BM * 4 + 512;
-    };
-    auto stages_for = [&](size_t fixed) {
-        int st = cap > fixed ? int((cap - fixed) / B_BLOCK) : 0;
-        return st > 6 ? 6 : st;
-    };
-    const int st8 = stages_for(fixed_for(2));
-    p.epi = (allow8 && p.kc <= 2 * CAPB && st8 >= 3) ? 8 : 4;
-    const size_t fixed = fixed_for(p.epi / 4);
-    p.stages = stages_for(fixed);
+    const size_t fixed = 1024 + size_t(x3 ? 2 : 1) * p.nkb * A_BLOCK + 8 * BM * 4 + EPI * CAP * 8 + 512;
+    p.stages = cap > fixed ? int(std::min<size_t>(6, (cap - fixed) / B_BLOCK)) : 0;
     p.smem = fixed + size_t(p.stages) * B_BLOCK;
     return p;
+}
+
+// One launch of the tile kernel; r: the plan's list length (0: top-1).
+famst_status launch_tiles(const Exec &ex, int r, bool f8, unsigned grid, size_t smem,
+                          const CUtensorMap &mA, const CUtensorMap &mB, const TcArgs &a) {
+#define TC_LAUNCH(...)                                                                          \
+    do {                                                                                        \
+        if (set_smem_attr(knn_tc_kernel<__VA_ARGS__>, int(smem), ex.stream) != cudaSuccess)     \
+            return FAMST_ERR_CUDA;                                                              \
+        FAMST_LAUNCH(ex, (knn_tc_kernel<__VA_ARGS__>), grid, TC_THREADS, smem, mA, mB, a);      \
+    } while (0)
+    if (a.colcomp) {   // nearest foreign neighbours
+        if (r > 4) return FAMST_ERR_UNSUPPORTED;
+        TC_LAUNCH(4, true);
+    } else if (f8) {
+        if (r <= 8) TC_LAUNCH(8, false, true);
+        else if (r <= 12) TC_LAUNCH(12, false, true);
+        else TC_LAUNCH(16, false, true);
+    } else {
+        switch (r) {
+            case 0: TC_LAUNCH(0, false); break;
+            case 4: TC_LAUNCH(4, false); break;
+            case 8: TC_LAUNCH(8, false); break;
+            case 12: TC_LAUNCH(12, false); break;
+            default: TC_LAUNCH(16, false);
+        }
+    }
+#undef TC_LAUNCH
+    return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
 }
 
 }  // namespace
 
 bool knn_tc_supported(int64_t n, int d, int k, bool x3, bool f8) {
     if (k + 1 > 64 || n < 2) return false;
-    TcPlan p = tc_plan(n, d, k, x3 && !f8, true, f8);
+    TcPlan p = tc_plan(n, d, k, x3 && !f8, f8);
     return p.stages >= 2 && encode_fn() != nullptr;
 }
 
 size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prune, bool f8) {
-    TcPlan p = tc_plan(n, d, k, x3 && !f8, true, f8);
+    TcPlan p = tc_plan(n, d, k, x3 && !f8, f8);
     if (f8) prune = false;
     size_t b = 0;
     if (prune) {
         const int64_t K = prune_pivots_max(n), Kpad = (K + BN - 1) / BN * BN;
         b += align256(size_t(K) * 4) + align256(size_t(K) * p.kh * 2) +
              align256(size_t(Kpad + BN) * 4) * 2 + align256(size_t(n) * 4) * 2;
-        b += prune_workspace(n, d, p.kh, p.kc - 1, p.nq_tiles, p.nk_tiles);
+        b += prune_workspace(n, d, p.kh, p.cap, p.nq_tiles, p.nk_tiles);
         b += align256(size_t(n) * 4) * 2 + align256(size_t(n) * 8) + 256;   // thr0, failed rows
         b += std::max(knn_fp32_pruned_workspace(n, k, p.nq_tiles),
                       visited_rows_workspace(n / VISITED_ROWS_SHARE));
@@ -1302,8 +1562,11 @@ size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prun
     b += align256(size_t(n) * 4);                          // xnorm2
     b += align256(size_t(d) * 4) + 256;                    // mean, ymax
     b += align256(size_t(4096) * d * 8);                   // column partials
-    b += align256(size_t(n) * (p.kc - 1) * 4);             // candidates
-    b += align256(size_t(n) * 4) * 2 + 256;                // splus, fail rows, count
+    b += align256(size_t(n) * p.cap * 4);                  // candidates
+    const int slots = log_slots(
+        p.nq_tiles + (prune_supported(n, d, k, true) ? PRUNE_SPLIT_SLOTS : 0), num_sms);
+    b += align256(size_t(slots) * LOG_SLOT * 8) + align256(size_t(slots) * 4);   // logs
+    b += align256(size_t(n) * 4) * 4 + 256;                // their number, splus, pivots, fail rows
     b += knn_fp32_workspace(n, d, k, n, num_sms);          // fallback
     return b;
 }
@@ -1329,7 +1592,7 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         if (colcomp) return FAMST_ERR_UNSUPPORTED;
     }
     // f32: the tensor tiles only place the points in pivot cells
-    TcPlan p = tc_plan(n, d, f32 ? 1 : k, x3, true, f8);
+    TcPlan p = tc_plan(n, d, f32 ? 1 : k, x3, f8);
     if (p.stages < 2 || (k + 1 > 64 && !f32)) return FAMST_ERR_UNSUPPORTED;
     // operand rows: BF16 (kh elements) or E4M3 bytes (kh bytes) with per-row scales
     __nv_bfloat16 *H = f8 ? nullptr : ar.take<__nv_bfloat16>(size_t(n) * p.kh);
@@ -1343,12 +1606,18 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     const int rows_per = int((n + 4095) / 4096) > 0 ? int((n + 4095) / 4096) : 1;
     const int nb = int((n + rows_per - 1) / rows_per);
     double *part = ar.take<double>(size_t(nb) * d);
-    int32_t *cand = ar.take<int32_t>(size_t(n) * (p.kc - 1));
+    int32_t *cand = f32 ? nullptr : ar.take<int32_t>(size_t(n) * p.cap);   // (pruned: in cell order)
+    int32_t *ccnt = ar.take<int32_t>(size_t(n));
+    const int slots = log_slots(
+        p.nq_tiles + (prune_supported(n, d, k, true) ? PRUNE_SPLIT_SLOTS : 0), ex.num_sms);
+    int2 *log = f32 ? nullptr : ar.take<int2>(size_t(slots) * LOG_SLOT);
+    int *claim = f32 ? nullptr : ar.take<int>(size_t(slots));
+    int32_t *top = ar.take<int32_t>(size_t(n));   // pivot of every point
     float *splus = ar.take<float>(size_t(n));
     int32_t *fail_rows = ar.take<int32_t>(size_t(n));
     int32_t *fail_count = ar.take<int32_t>(1);
-    if ((!f8 && !H) || !ny || !xn2 || !mean || !ymax || !part || !cand || !splus || !fail_rows ||
-        !fail_count)
+    if ((!f8 && !H) || !ny || !xn2 || !mean || !ymax || !part || (!f32 && (!cand || !log || !claim)) || !ccnt || !top || !splus ||
+        !fail_rows || !fail_count)
         return FAMST_ERR_OOM;
     // prep: mean, centred BF16 operands, norms
     FAMST_LAUNCH(ex, colsum_partial_kernel, nb, 128, 0, X, n, d, rows_per, part);
@@ -1389,8 +1658,6 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
             prune_pivot_operands(ex, H, p.kh, ny, n, K0, Kpadmax + BN, piv, Hp, nyp);
         if (st != FAMST_OK) return st;
         const TcPlan p1 = tc_plan(n, d, 1, false);
-        if (set_smem_attr(knn_tc_kernel<1, false>, int(p1.smem), ex.stream) != cudaSuccess)
-            return FAMST_ERR_CUDA;
         // top-1 over pivots [k0, k0 + kc) into (c_out, s_out), ids relative to k0
         auto assign = [&](int k0, int kc, int32_t *c_out, float *s_out) -> famst_status {
             CUtensorMap mA1, mB1;
@@ -1403,15 +1670,21 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
                 return FAMST_ERR_CUDA;
             if (kc < nkt * BN)   // columns beyond the pass's pivots never win
                 FAMST_LAUNCH(ex, fill_inf_kernel, 1, 256, 0, nya, int64_t(kc), int64_t(nkt) * BN);
-            TcArgs a1{int(n), nkt, p.nkb, 0, p1.stages, nya, c_out, s_out,
-                      ex.dstatus, nullptr, nullptr, nullptr, 1, p1.epi};
+            TcArgs a1{};
+            a1.n = int(n);
+            a1.nk_tiles = nkt;
+            a1.nkb = p.nkb;
+            a1.stages = p1.stages;
+            a1.ny = nya;
+            a1.cand = c_out;
+            a1.splus = s_out;
+            a1.status = ex.dstatus;
+            a1.cross = 1;
             a1.nitems = int(p.nq_tiles);   // persistent: one CTA per SM walks the query tiles
-            FAMST_LAUNCH(ex, (knn_tc_kernel<1, false>), pgrid, 64 + 32 * p1.epi, p1.smem, mA1, mB1,
-                         a1);
-            return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
+            return launch_tiles(ex, 0, false, pgrid, p1.smem, mA1, mB1, a1);
         };
         int K = K0;
-        st = assign(0, K, cand, splus);
+        st = assign(0, K, top, splus);
         // each coverage pass scores the points against the new pivots only
         int32_t *c2 = ar.take<int32_t>(size_t(n));
         float *s2 = ar.take<float>(size_t(n));
@@ -1424,12 +1697,12 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
                 st = assign(K, me, c2, s2);
                 if (st == FAMST_OK)
                     FAMST_LAUNCH(ex, top1_merge_kernel, unsigned((n + 255) / 256), 256, 0, c2, s2,
-                                 K, n, cand, splus);
+                                 K, n, top, splus);
             }
             K += M;
         }
         if (st != FAMST_OK) return st;
-        st = prune_partition(ex, ar, X, d, n, k, H, p.kh, ny, p.nkb, K, piv, cand, 1,
+        st = prune_partition(ex, ar, X, d, n, k, H, p.kh, ny, p.nkb, K, piv, top, 1,
                              pinned_host + 2, &P);
         if (st != FAMST_OK) return st;
     }
@@ -1439,11 +1712,7 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         return use_prune ? knn_fp32_pruned(ex, ar, X, n, d, k, P, nbr, dist)
                          : FAMST_ERR_UNSUPPORTED;
     }
-    // candidates of the tensor pass: directly in cand / splus, or (pruned)
-    // in sorted order first
-    int32_t *cand_t = cand;
-    float *splus_t = splus;
-    int32_t *side_j = nullptr;   // candidates of the parts of split lists
+    int32_t *side_j = nullptr, *side_cnt = nullptr;   // candidates of the parts of split lists
     float *side_s = nullptr, *side_sp = nullptr;
     float *thr0 = nullptr;       // start thresholds
     uint64_t *fail_kth = nullptr;
@@ -1454,12 +1723,11 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         fails2 = ar.take<int32_t>(size_t(n));
         nfail2 = ar.take<int32_t>(1);
         if (!thr0 || !fail_kth || !fails2 || !nfail2) return FAMST_ERR_OOM;
-        cand_t = ar.take<int32_t>(size_t(n) * (p.kc - 1));
-        splus_t = ar.take<float>(size_t(n));
-        side_j = ar.take<int32_t>(size_t(PRUNE_SPLIT_SLOTS) * BM * (p.kc - 1));
-        side_s = ar.take<float>(size_t(PRUNE_SPLIT_SLOTS) * BM * (p.kc - 1));
+        side_j = ar.take<int32_t>(size_t(PRUNE_SPLIT_SLOTS) * BM * p.cap);
+        side_s = ar.take<float>(size_t(PRUNE_SPLIT_SLOTS) * BM * p.cap);
+        side_cnt = ar.take<int32_t>(size_t(PRUNE_SPLIT_SLOTS) * BM);
         side_sp = ar.take<float>(size_t(PRUNE_SPLIT_SLOTS) * BM);
-        if (!cand_t || !splus_t || !side_j || !side_s || !side_sp) return FAMST_ERR_OOM;
+        if (!side_j || !side_s || !side_cnt || !side_sp) return FAMST_ERR_OOM;
     }
     const void *Hop = f8 ? static_cast<const void *>(Q)
                          : static_cast<const void *>(use_prune ? P.Hs : H);
@@ -1475,12 +1743,8 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
             return FAMST_ERR_CUDA;
     }
     // certificate constants (also the pruned lists' start thresholds)
-    const double u8 = 1.0 / 256.0;
     const double kprod = double(x3 ? 3 * p.d_pad : p.d_pad);
-    CertConst cc;
-    cc.eps_dot = (x3 ? (3.0 * u8 * u8 + 3.0 * u8 * u8 * u8 + u8 * u8 * u8 * u8)
-                     : (2.0 * u8 + u8 * u8)) +
-                 kprod * std::ldexp(1.0, -22) * (1.0 + 4.0 * u8);
+    double eps_dot = tc_eps_dot(p.d_pad, x3);
     if (f8) {
         // E4M3 with the row's scale: a normal element is within u = 2^-4 of
         // x'_t (relative); an element below the normal range within 2^-10 s,
@@ -1491,16 +1755,35 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         // sides, |x^.y^ - x'.y'| <= ((2u + u^2) + 2 sqrt(d)(1 + u) c + d c^2)
         // ||x'|| ||y'||.
         const double u4 = 1.0 / 16.0, c8 = 2.0 / 448.0 / 1024.0, dp = double(p.d_pad);
-        cc.eps_dot = 2.0 * u4 + u4 * u4 + 2.0 * std::sqrt(dp) * (1.0 + u4) * c8 + dp * c8 * c8 +
+        eps_dot = 2.0 * u4 + u4 * u4 + 2.0 * std::sqrt(dp) * (1.0 + u4) * c8 + dp * c8 * c8 +
                      kprod * std::ldexp(1.0, -22) * (1.0 + 4.0 * u4);
     }
-    cc.d_plus = double(d) + 4.0;
+    const CertConst cc = cert_const(eps_dot, d);
     if (use_prune)
         FAMST_LAUNCH(ex, thr0_kernel, unsigned((n + 255) / 256), 256, 0, P.tau_row, P.nys, n, d,
                      ymax, cc.eps_dot, thr0);
-    TcArgs a{int(n), int(p.nk_tiles), p.nkb, int(x3), p.stages, use_prune ? P.nys : ny, cand_t,
-             splus_t, ex.dstatus, use_prune ? P.tab : nullptr, cpad,
-             use_prune ? P.klist : nullptr, 0, p.epi, rscale, thr0};
+    TcArgs a{};
+    a.n = int(n);
+    a.nk_tiles = int(p.nk_tiles);
+    a.nkb = p.nkb;
+    a.x3 = int(x3);
+    a.stages = p.stages;
+    a.ny = use_prune ? P.nys : ny;
+    a.cand = cand;
+    a.ccnt = ccnt;
+    a.cap = p.cap;
+    a.sel = Select{k, p.cap, float(4.2 * cc.eps_dot), score_eps_row(d)};
+    a.ymax = ymax;
+    a.log = log;
+    a.claim = claim;
+    a.nslots = slots;
+    if (cudaMemsetAsync(claim, 0, size_t(slots) * 4, ex.stream) != cudaSuccess)
+        return FAMST_ERR_CUDA;
+    a.splus = splus;
+    a.status = ex.dstatus;
+    a.colcomp = cpad;
+    a.rscale = rscale;
+    a.thr0 = thr0;
     // one CTA per work item: the pruned tiles' key lists differ in length,
     // and a static round-robin over persistent CTAs measured slower here.
     // Pruned lists come as work items, long ones split into parts; the grid
@@ -1508,81 +1791,50 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     // count leave at once.
     unsigned tgrid = unsigned(p.nq_tiles);
     if (use_prune) {
+        a.tiles = P.tab;
+        a.klist = P.klist;
         a.nitems_dev = P.nitems;
         a.side_j = side_j;
         a.side_s = side_s;
+        a.side_cnt = side_cnt;
         a.side_splus = side_sp;
         tgrid = unsigned(p.nq_tiles + PRUNE_SPLIT_SLOTS);
     }
-#define TC_LAUNCH(KCV, M)                                                                        \
-    do {                                                                                         \
-        if (set_smem_attr(knn_tc_kernel<KCV, M>, int(p.smem), ex.stream) != cudaSuccess)         \
-            return FAMST_ERR_CUDA;                                                               \
-        FAMST_LAUNCH(ex, (knn_tc_kernel<KCV, M>), tgrid, 64 + 32 * p.epi, p.smem, mA, mB, a);   \
-    } while (0)
-#define TC_LAUNCH_F8(KCV)                                                                           \
-    do {                                                                                            \
-        if (set_smem_attr(knn_tc_kernel<KCV, false, true>, int(p.smem), ex.stream) != cudaSuccess)  \
-            return FAMST_ERR_CUDA;                                                                  \
-        FAMST_LAUNCH(ex, (knn_tc_kernel<KCV, false, true>), tgrid, 64 + 32 * p.epi,                \
-                     p.smem, mA, mB, a);                                                            \
-    } while (0)
     timer_mark(ex, TIMER_TILES, false);
-    if (f8) {
-        if (p.kc == 32) TC_LAUNCH_F8(32);
-        else if (p.kc == 48) TC_LAUNCH_F8(48);
-        else TC_LAUNCH_F8(64);
-    } else if (cpad) {
-        if (p.kc == 32) TC_LAUNCH(32, true);
-        else if (p.kc == 48) TC_LAUNCH(48, true);
-        else TC_LAUNCH(64, true);
-    } else {
-        if (p.kc == 32) TC_LAUNCH(32, false);
-        else if (p.kc == 48) TC_LAUNCH(48, false);
-        else TC_LAUNCH(64, false);
+    {
+        const famst_status st = launch_tiles(ex, p.r, f8, tgrid, p.smem, mA, mB, a);
+        if (st != FAMST_OK) return st;
     }
-    if (use_prune) {   // rows of split lists: merge their parts
-#define SPLIT_MERGE(KCV)                                                                        \
-    FAMST_LAUNCH(ex, split_merge_kernel<KCV>, unsigned(PRUNE_SPLIT_TILES), BM, 0, P.splitq,     \
-                 P.nsplit, side_j, side_s, side_sp, n, cand_t, splus_t)
-        if (p.kc == 32) SPLIT_MERGE(32);
-        else if (p.kc == 48) SPLIT_MERGE(48);
-        else SPLIT_MERGE(64);
-#undef SPLIT_MERGE
-    }
+    if (use_prune)   // rows of split lists: combine their parts
+        FAMST_LAUNCH(ex, split_merge_kernel, dim3(PRUNE_SPLIT_TILES, BM / 16), 512, 0, P.splitq,
+                     P.nsplit, side_j, side_s, side_cnt, side_sp, n, a.sel, a.ny, ymax, cand, ccnt,
+                     splus);
     timer_mark(ex, TIMER_TILES, true);
-#undef TC_LAUNCH
-#undef TC_LAUNCH_F8
     if (cudaPeekAtLastError() != cudaSuccess) return FAMST_ERR_CUDA;
     const unsigned rgrid = unsigned((n * 32 + 255) / 256);
-#define RERANK3(V, KCV, XRV)                                                                     \
+#define RERANK2(XRV, HV)                                                                         \
     do {                                                                                         \
         if (use_prune)                                                                           \
-            FAMST_LAUNCH(ex, (rerank_sorted_kernel<V, KCV, XRV>), rgrid, 256, 0, P.Xs, n, d, k,  \
-                         cand_t, splus_t, P.skipQ, P.perm, xn2, ymax, cc, nbr, dist, fail_rows,  \
-                         fail_kth, fail_count);                                                            \
+            FAMST_LAUNCH(ex, (rerank_sorted_kernel<XRV, HV>), rgrid, 256, 0, P.Xs, n, d, k,      \
+                         cand, ccnt, splus, P.skipQ, P.perm, xn2, ymax, cc, nbr, dist,           \
+                         fail_rows, fail_kth, fail_count);                                       \
         else                                                                                     \
-            FAMST_LAUNCH(ex, (rerank_kernel<V, KCV, XRV>), rgrid, 256, 0, X, n, d, k, cand,      \
+            FAMST_LAUNCH(ex, (rerank_kernel<XRV, HV>), rgrid, 256, 0, X, n, d, k, cand, ccnt,    \
                          splus, nullptr, xn2, ymax, cc, nbr, dist, fail_rows, fail_count);       \
     } while (0)
-#define RERANK(V, KCV)                                                                           \
+#define RERANK(XRV)                                                                              \
     do {                                                                                         \
-        if (d <= 128) RERANK3(V, KCV, 4);                                                        \
-        else if (d <= 256) RERANK3(V, KCV, 8);                                                   \
-        else if (d <= 512) RERANK3(V, KCV, 16);                                                  \
-        else RERANK3(V, KCV, 0);                                                                 \
+        if (p.cap == 64) RERANK2(XRV, 2);                                                        \
+        else RERANK2(XRV, 4);                                                                    \
     } while (0)
     timer_mark(ex, TIMER_RERANK, false);
-    if (p.kc == 32) {
-        RERANK(1, 32);
-    } else if (p.kc == 48) {
-        RERANK(1, 48);
-    } else {
-        RERANK(1, 64);
-    }
+    if (d <= 128) RERANK(4);
+    else if (d <= 256) RERANK(8);
+    else if (d <= 512) RERANK(16);
+    else RERANK(0);
     timer_mark(ex, TIMER_RERANK, true);
 #undef RERANK
-#undef RERANK3
+#undef RERANK2
     if (cudaMemcpyAsync(pinned_host, fail_count, 4, cudaMemcpyDeviceToHost, ex.stream) != cudaSuccess ||
         (use_prune && cudaMemcpyAsync(pinned_host + 1, P.visited, 4, cudaMemcpyDeviceToHost,
                                       ex.stream) != cudaSuccess) ||
@@ -1618,43 +1870,19 @@ namespace famst {
 
 // Shared-memory plan of the batched tensor path for operand width D (the
 // largest cloud's K extent).
-bool knn_tc_batched_plan(int D, int k, bool x3, int epi_req, int *stages, size_t *smem, int *kc,
-                         int *epi) {
+bool knn_tc_batched_plan(int D, int k, bool x3, int *stages, size_t *smem) {
     if (k + 1 > 64) return false;
-    TcPlan p = tc_plan(int64_t(1) << 20, D, k, x3, epi_req == 8);
+    const TcPlan p = tc_plan(int64_t(1) << 20, D, k, x3);
     if (p.stages < 2 || encode_fn() == nullptr) return false;
     *stages = p.stages;
     *smem = p.smem;
-    *kc = p.kc;
-    *epi = p.epi;
     return true;
 }
 
-// The batched tile pass alone (one persistent launch over the (cloud, query
-// tile) items): the autotuner times it per shape on the batch's own data.
-famst_status knn_tc_batched_tiles(const Exec &ex, int D, bool x3, int stages, size_t smem, int kc,
-                                  int epi, const TcTile *tiles, int64_t nctas, const float *ny,
-                                  int32_t *cand, float *splus, const CUtensorMap *mA,
-                                  const CUtensorMap *mB, bool spiral) {
-    if (nctas <= 0) return FAMST_OK;
-    const int nkb = D / BK;
-    TcArgs a{0, 0, nkb, int(x3), stages, ny, cand, splus, ex.dstatus, tiles, nullptr, nullptr, 0,
-             epi};
-    // persistent: one CTA per SM walks the (cloud, query tile) items round-robin
-    a.nitems = int(nctas);
-    a.spiral = spiral ? 1 : 0;
-    const unsigned bgrid = unsigned(std::min<int64_t>(nctas, ex.num_sms));
-#define TCB_LAUNCH(KCV)                                                                          \
-    do {                                                                                         \
-        if (set_smem_attr(knn_tc_kernel<KCV, false>, int(smem), ex.stream) != cudaSuccess)      \
-            return FAMST_ERR_CUDA;                                                               \
-        FAMST_LAUNCH(ex, (knn_tc_kernel<KCV, false>), bgrid, 64 + 32 * epi, smem, *mA, *mB, a);  \
-    } while (0)
-    if (kc == 32) TCB_LAUNCH(32);
-    else if (kc == 48) TCB_LAUNCH(48);
-    else TCB_LAUNCH(64);
-#undef TCB_LAUNCH
-    return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
+int knn_tc_epilogue_warps() { return EPI; }
+int knn_tc_cand_cap(int k) { return tc_plan(1, 1, k, false).cap; }
+size_t knn_tc_log_entries(int64_t nctas, int num_sms) {
+    return size_t(log_slots(nctas, num_sms)) * LOG_SLOT;
 }
 
 // Everything of the batched tensor path that runs on the device; buffers
@@ -1662,10 +1890,11 @@ famst_status knn_tc_batched_tiles(const Exec &ex, int D, bool x3, int stages, si
 famst_status knn_tc_batched(const Exec &ex, const float *Xc, int D, int64_t N, int64_t NP,
                             const long long *voff, const long long *roff, int B,
                             const CloudDev *cl, const TcTile *tiles, int64_t nctas, int k,
-                            bool x3, int stages, size_t smem, int kc, int epi, __nv_bfloat16 *H,
+                            bool x3, int stages, size_t smem, __nv_bfloat16 *H,
                             float *ny, float *xn2, float *mean, unsigned *ymax, int32_t *cand,
-                            float *splus, int32_t *fail_rows, int32_t *fail_count, int32_t *nbr,
-                            float *dist, const CUtensorMap *mA, const CUtensorMap *mB,
+                            int32_t *ccnt, int2 *log, int *claim, float *splus,
+                            int32_t *fail_rows, int32_t *fail_count, int32_t *nbr, float *dist,
+                            const CUtensorMap *mA, const CUtensorMap *mB,
                             const float *Xorig, const int32_t *perm) {
     FAMST_LAUNCH(ex, cloud_mean_kernel, B, 128, 0, Xc, D, cl, mean);
     if (cudaMemsetAsync(ymax, 0, size_t(B) * 4, ex.stream) != cudaSuccess ||
@@ -1673,27 +1902,54 @@ famst_status knn_tc_batched(const Exec &ex, const float *Xc, int D, int64_t N, i
         return FAMST_ERR_CUDA;
     FAMST_LAUNCH(ex, tc_prep_batched_kernel, unsigned((NP * 32 + 255) / 256), 256, 0, Xc, D, NP,
                  roff, voff, B, cl, D, int(x3), mean, H, ny, xn2, ymax);
-    famst_status st = knn_tc_batched_tiles(ex, D, x3, stages, smem, kc, epi, tiles, nctas, ny, cand,
-                                           splus, mA, mB, perm != nullptr);
-    if (st != FAMST_OK) return st;
+    const TcPlan p = tc_plan(1, D, k, x3);
+    if (nctas > 0) {
+        TcArgs a{};
+        a.nkb = D / BK;
+        a.x3 = int(x3);
+        a.stages = stages;
+        a.ny = ny;
+        a.cand = cand;
+        a.ccnt = ccnt;
+        a.cap = p.cap;
+        a.sel = Select{k, p.cap, float(4.2 * tc_eps_dot(D, x3)), score_eps_row(D)};
+        a.ymax = ymax;
+        a.log = log;
+        a.claim = claim;
+        a.nslots = log_slots(nctas, ex.num_sms);
+        if (cudaMemsetAsync(claim, 0, size_t(a.nslots) * 4, ex.stream) != cudaSuccess)
+            return FAMST_ERR_CUDA;
+        a.splus = splus;
+        a.status = ex.dstatus;
+        a.tiles = tiles;
+        // persistent: one CTA per SM walks the (cloud, query tile) items round-robin
+        a.nitems = int(nctas);
+        a.spiral = perm != nullptr ? 1 : 0;
+        const famst_status st =
+            launch_tiles(ex, p.r, false,
+                         unsigned(std::min<int64_t>(nctas, ex.num_sms)), smem, *mA, *mB, a);
+        if (st != FAMST_OK) return st;
+    }
     const unsigned rgrid = unsigned((N * 32 + 255) / 256);
     // one candidate at a time per warp over coalesced row reads when the
     // padded rows fit the register slices (D <= 512), else one per lane
-#define RRB(KCV, XRV)                                                                            \
-    FAMST_LAUNCH(ex, (rerank_batched_kernel<KCV, XRV>), rgrid, 256, 0, Xc, D, N, voff, B, cl,    \
-                 int(x3), k, cand, splus, xn2, ymax, perm, nbr, dist, fail_rows, fail_count)
-#define RRB_KC(KCV)                                                                              \
+    // (the widest cloud's bounds hold for every cloud; FP64 takes each one's own)
+    const CertConst cc = cert_const(tc_eps_dot(D, x3), D);
+#define RRB2(XRV, HV)                                                                            \
+    FAMST_LAUNCH(ex, (rerank_batched_kernel<XRV, HV>), rgrid, 256, 0, Xc, D, N, voff, B, cl,     \
+                 int(x3), k, cand, ccnt, splus, xn2, ymax, cc, perm, nbr, dist, fail_rows,       \
+                 fail_count)
+#define RRB(XRV)                                                                                 \
     do {                                                                                         \
-        if (D <= 128) RRB(KCV, 4);                                                               \
-        else if (D <= 256) RRB(KCV, 8);                                                          \
-        else if (D <= 512) RRB(KCV, 16);                                                         \
-        else RRB(KCV, 0);                                                                        \
+        if (p.cap == 64) RRB2(XRV, 2);                                                           \
+        else RRB2(XRV, 4);                                                                       \
     } while (0)
-    if (kc == 32) RRB_KC(32);
-    else if (kc == 48) RRB_KC(48);
-    else RRB_KC(64);
-#undef RRB_KC
+    if (D <= 128) RRB(4);
+    else if (D <= 256) RRB(8);
+    else if (D <= 512) RRB(16);
+    else RRB(0);
 #undef RRB
+#undef RRB2
     // rows no certificate covers: exact within their cloud, original order and ids
     FAMST_LAUNCH(ex, fallback_rows_kernel, unsigned(ex.num_sms) * 16, FB_WARPS * 32, 0,
                  Xorig ? Xorig : Xc, D, voff, B, cl, k, fail_rows, fail_count, nbr, dist);

@@ -585,6 +585,7 @@ split_table_kernel(const int32_t *__restrict__ off, int64_t nq, int nkb, int64_t
             t.nkb = nkb;
             t.row_end = int(n);
             t.shift = 0;
+            t.cloud = 0;
             if (len > L) {
                 const int P = int((len + L - 1) / L);
                 splitq[3 * si] = int(q);
@@ -712,8 +713,7 @@ size_t prune_workspace(int64_t n, int d, int kh, int kp, int64_t nq, int64_t nk)
          align256(size_t(nq + PRUNE_SPLIT_SLOTS) * sizeof(TcTile));           // skip, work items
     b += align256(4) * 2 + align256(size_t(3) * PRUNE_SPLIT_TILES * 4);        // item and split counts
     b += align256(size_t(PRUNE_SPLIT_SLOTS) * QT * kp * 4) * 2 +
-         align256(size_t(PRUNE_SPLIT_SLOTS) * QT * 4);                         // parts' candidates
-    b += align256(size_t(n) * kp * 4) + align256(size_t(n) * 4);               // sorted outputs
+         align256(size_t(PRUNE_SPLIT_SLOTS) * QT * 4) * 2;                     // parts' candidates
     b += align256(size_t(n) * d * 4);                                          // sorted points
     return b;
 }

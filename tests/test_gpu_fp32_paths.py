@@ -63,10 +63,10 @@ def test_pruned_tiles(ctx, name, make, k):
 # tiles over all lists)
 @pytest.mark.parametrize("make,prec,k,few", [
     (lambda: workloads.get("blobs_100k").points(), "bf16x3", 16, True),
-    (lambda: workloads.blobs(30000, 128, 15, (0.4, 2.0), 47), "bf16x3", 16, False),
+    (lambda: workloads.blobs(30000, 128, 15, (0.4, 2.0), 47), "bf16x3", 16, True),
     (lambda: workloads.blobs(30000, 128, 15, (0.4, 2.0), 47), "bf16x3", 20, False),
     (lambda: workloads.blobs(30000, 128, 15, (0.4, 2.0), 47), "bf16", 16, False),
-], ids=["few", "many16", "many20", "bf16"])
+], ids=["few", "few16", "many20", "bf16"])
 def test_uncertified_rows_on_the_lists(ctx, make, prec, k, few):
     X = torch.from_numpy(make()).cuda()
     _, info = ctx.build(X, k, 2, 1, prec)

@@ -152,18 +152,6 @@ __device__ __forceinline__ void pairs_batch(const float *__restrict__ X, int d, 
 }
 
 // pair p -> (i, j), pairs enumerated i outer, j inner
-__device__ __forceinline__ void pair_of(int64_t p, int64_t t, int64_t &i, int64_t &j) {
-    const double bb = 2.0 * double(t) - 1.0;
-    const double disc = bb * bb - 8.0 * double(p);
-    i = int64_t((bb - sqrt(disc > 0 ? disc : 0.0)) * 0.5);
-    if (i < 0) i = 0;
-    if (i > t - 2) i = t - 2;
-    auto start = [t](int64_t x) { return x * t - x * (x + 1) / 2; };
-    while (i > 0 && start(i) > p) --i;
-    while (i + 1 <= t - 2 && start(i + 1) <= p) ++i;
-    j = p - start(i) + i + 1;
-}
-
 // ------------------------------------------------ all pairs on tcgen05
 
 constexpr int NT_M = 128;      // rows of an item (TMEM lanes)

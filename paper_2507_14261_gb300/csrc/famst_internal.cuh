@@ -190,13 +190,27 @@ __device__ __forceinline__ uint64_t shfl_up_u64(uint64_t v, int delta) {
     return (uint64_t(hi) << 32) | lo;
 }
 
+// (two warp reductions of 32 bits instead of ten shuffles and compares)
 __device__ __forceinline__ uint64_t warp_min_u64(uint64_t v) {
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) {
-        uint64_t o = shfl_xor_u64(v, m);
-        v = o < v ? o : v;
-    }
-    return v;
+    const uint32_t hi = uint32_t(v >> 32);
+    const uint32_t mh = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_min_sync(0xffffffffu, hi == mh ? uint32_t(v) : 0xffffffffu);
+    return (uint64_t(mh) << 32) | ml;
+}
+
+// Pair p of the t (t - 1) / 2 pairs i < j in lexicographic order. Counted from
+// the last pair, the rows hold 1, 2, 3, ... pairs: the m-th row from the end
+// has m (m + 1) / 2 pairs after it. m from an FP32 root, corrected exactly
+// (the root in FP64 cost a warp some thirty operations at two lanes per SM
+// and clock: about 0.8 ms of the 500,000 pairs of 1000 components).
+__device__ __forceinline__ void pair_of(int64_t p, int64_t t, int64_t &i, int64_t &j) {
+    const int64_t r = t * (t - 1) / 2 - 1 - p;
+    int64_t m = int64_t(0.5f * (__fsqrt_rn(8.0f * float(r) + 1.0f) - 1.0f));
+    if (m > t - 2) m = t - 2;
+    while (m * (m + 1) / 2 > r) --m;
+    while ((m + 1) * (m + 2) / 2 <= r) ++m;
+    i = t - 2 - m;
+    j = t - 1 - (r - m * (m + 1) / 2);
 }
 
 // Bitonic sort of 32 H keys (element 32 h + lane), ascending.

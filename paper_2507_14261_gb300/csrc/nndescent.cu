@@ -21,11 +21,11 @@
 //
 // GPU layout: a list is k 64-bit keys (w bits << 32 | id) plus a flag byte
 // per entry, one warp per list (lane r = entry r). The join stages a v's
-// (at most 2S) candidate rows in shared memory and gives every thread one
-// pair: the canonical FP32 distance with its 32 partials in registers,
-// float4 reads of the shared rows (row stride an odd number of 16-byte
-// units, so the rows that 8 neighbouring lanes read sit in different bank
-// groups). A proposal is kept only if it beats the target's current k-th
+// (at most 2S) candidate rows in shared memory (row stride an odd number of
+// 16-byte units, so the rows that 8 neighbouring lanes read sit in different
+// bank groups): one warp per v with up to four pairs per lane where many such
+// warps fit an SM, else a block per v with one pair per lane, its 32 partials
+// in registers. A proposal is kept only if it beats the target's current k-th
 // key: the k-th key of a list only falls while proposals arrive, so this
 // drops nothing the update would keep. The joins of a chunk of v's append
 // their proposals to one buffer; the buffer is grouped by target (count,
@@ -39,6 +39,7 @@
 #include <cstring>
 
 #include "famst_internal.cuh"
+#include "staged_rows.cuh"
 
 namespace famst {
 namespace {
@@ -47,6 +48,7 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr uint8_t NND_NEW = 1, NND_INS = 2;
 constexpr uint32_t TAG_START = 1, TAG_PRIO = 2;
 constexpr int NND_JOIN_THREADS = 128;
+constexpr size_t NND_SMEM_SM = 228 * 1024;   // shared memory of an SM
 
 __device__ __forceinline__ uint32_t nnd_draw(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                              uint2 key) {
@@ -364,6 +366,178 @@ nnd_join_kernel(const float *__restrict__ X, int d, int n, int k, int S, int v0,
     if (threadIdx.x == 0 && spairs) atomicAdd(npairs, (unsigned long long)spairs);
 }
 
+// Pairs (i < nn, i < b < m) of the staged rows, by one warp in tiles of 4 TI x
+// 16: lane (g, h) of 4 x 8 takes rows i0 + g + 4 a and b0 + h + 8 c, so a float4
+// read from shared memory serves two pairs (TI = 2) and a row is read by a whole
+// lane group. Canonical distances: the 32 partials are formed four at a time,
+// in the order in which the butterfly 16, 8, 4, 2, 1 adds them up.
+template <int TI>
+__device__ __forceinline__ void join_tiles(const float4 *srow, int rs4, int d4, const int *sid,
+                                           const unsigned long long *sthr, int nn, int m, int lane,
+                                           int32_t *__restrict__ pt,
+                                           uint64_t *__restrict__ pk,
+                                           unsigned long long *__restrict__ pcount,
+                                           unsigned long long pcap, unsigned &my_pairs,
+                                           int *dstatus) {
+    const int g = lane >> 3, h = lane & 7;
+    const int nb = (m + 15) >> 4, nt = ((nn + 4 * TI - 1) / (4 * TI)) * nb;
+    for (int t = 0; t < nt; ++t) {
+        const int i0 = (t / nb) * 4 * TI, b0 = (t % nb) * 16;
+        if (b0 + 15 <= i0) continue;   // on or below the diagonal
+        const float4 *rx[TI], *ry[2];   // (rows beyond the ends: any staged row)
+#pragma unroll
+        for (int a = 0; a < TI; ++a) rx[a] = srow + min(i0 + g + 4 * a, m - 1) * rs4;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) ry[c] = srow + min(b0 + h + 8 * c, m - 1) * rs4;
+        float U[TI][2][4];
+#pragma unroll 1
+        for (int jj = 0; jj < 2; ++jj) {
+            float R[TI][2][4], Q[TI][2][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {   // partials 4 j .. 4 j + 3
+                const int j = jj + 2 * (e >> 1) + 4 * (e & 1);
+                float p[TI][2][4] = {};
+#pragma unroll 2
+                for (int q = j; q < d4; q += 8) {
+                    float4 y[2];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) y[c] = ry[c][q];
+#pragma unroll
+                    for (int a = 0; a < TI; ++a) {
+                        const float4 x = rx[a][q];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const float t0 = __fsub_rn(x.x, y[c].x), t1 = __fsub_rn(x.y, y[c].y);
+                            const float t2 = __fsub_rn(x.z, y[c].z), t3 = __fsub_rn(x.w, y[c].w);
+                            p[a][c][0] = __fmaf_rn(t0, t0, p[a][c][0]);
+                            p[a][c][1] = __fmaf_rn(t1, t1, p[a][c][1]);
+                            p[a][c][2] = __fmaf_rn(t2, t2, p[a][c][2]);
+                            p[a][c][3] = __fmaf_rn(t3, t3, p[a][c][3]);
+                        }
+                    }
+                }
+                // e = 0, 1: partials l and l + 16; e = 2, 3: l + 8 and l + 24
+#pragma unroll
+                for (int a = 0; a < TI; ++a)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int l = 0; l < 4; ++l) {
+                            if (e == 0) R[a][c][l] = p[a][c][l];
+                            if (e == 1) R[a][c][l] = __fadd_rn(R[a][c][l], p[a][c][l]);
+                            if (e == 2) Q[a][c][l] = p[a][c][l];
+                            if (e == 3)
+                                R[a][c][l] =
+                                    __fadd_rn(R[a][c][l], __fadd_rn(Q[a][c][l], p[a][c][l]));
+                        }
+            }
+#pragma unroll
+            for (int a = 0; a < TI; ++a)
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int l = 0; l < 4; ++l)
+                        U[a][c][l] = jj == 0 ? R[a][c][l] : __fadd_rn(U[a][c][l], R[a][c][l]);
+        }
+        // proposals: w to the lists of both ends where it beats their k-th
+        uint64_t ka[TI][2], kb[TI][2];
+        unsigned ma[TI][2], mb[TI][2];
+        int tot = 0;
+#pragma unroll
+        for (int a = 0; a < TI; ++a)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int i = i0 + g + 4 * a, b = b0 + h + 8 * c;
+                const bool in = i < nn && b < m && b > i;
+                const int ia = sid[in ? i : 0], ib = sid[in ? b : 0];
+                const bool live = in && ia != ib;
+                const float *u = U[a][c];
+                const float w =
+                    __fsqrt_rn(__fadd_rn(__fadd_rn(u[0], u[2]), __fadd_rn(u[1], u[3])));
+                ka[a][c] = nb_key(w, uint32_t(ib));
+                kb[a][c] = nb_key(w, uint32_t(ia));
+                my_pairs += __popc(__ballot_sync(FULL, live));
+                ma[a][c] = __ballot_sync(FULL, live && ka[a][c] < sthr[in ? i : 0]);
+                mb[a][c] = __ballot_sync(FULL, live && kb[a][c] < sthr[in ? b : 0]);
+                tot += __popc(ma[a][c]) + __popc(mb[a][c]);
+            }
+        if (tot == 0) continue;
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(pcount, (unsigned long long)tot);
+        base = __shfl_sync(FULL, base, 0);
+        if (base + tot > pcap) {   // the chunk size rules this out
+            if (lane == 0) set_status(dstatus, STATUS_INTERNAL);
+            continue;
+        }
+#pragma unroll
+        for (int a = 0; a < TI; ++a)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (ma[a][c] >> lane & 1) {
+                    const unsigned long long q = base + __popc(ma[a][c] & lanemask_lt());
+                    pt[q] = int32_t(key_lo(kb[a][c]));
+                    pk[q] = ka[a][c];
+                }
+                base += __popc(ma[a][c]);
+                if (mb[a][c] >> lane & 1) {
+                    const unsigned long long q = base + __popc(mb[a][c] & lanemask_lt());
+                    pt[q] = int32_t(key_lo(ka[a][c]));
+                    pk[q] = kb[a][c];
+                }
+                base += __popc(mb[a][c]);
+            }
+    }
+}
+
+// Local joins of v in [v0, v0 + nv), one warp per v (persistent blocks of one
+// warp): the rows come by asynchronous copies, all in flight at once. A block
+// of four warps per v, a lane per pair of one row with 32 others, left most
+// lanes without a pair (some ten rows against sixteen) and issued 76 % of the
+// cycles: 100,000 x 128, k = S = 16, ten iterations 8.35 -> 6.63 ms. Bound: the
+// latency of shared memory with some thirteen warps per SM (their rows fill
+// it). The same tiles in four-warp blocks: 10.2 ms (one tile per v mostly, so
+// three warps idle).
+__global__ void __launch_bounds__(32)
+nnd_join_warp_kernel(const float *__restrict__ X, int d, int n, int k, int S, int v0, int nv,
+                     int rs4, const int32_t *__restrict__ samp, const int32_t *__restrict__ scnt,
+                     const uint64_t *__restrict__ Bk, int32_t *__restrict__ pt,
+                     uint64_t *__restrict__ pk, unsigned long long *__restrict__ pcount,
+                     unsigned long long pcap, unsigned long long *__restrict__ npairs,
+                     int *dstatus) {
+    extern __shared__ float4 srow[];
+    __shared__ int sid[64];
+    __shared__ unsigned long long sthr[64];
+    const int lane = threadIdx.x, d4 = d >> 2;
+    const uint32_t sbase = uint32_t(__cvta_generic_to_shared(srow));
+    unsigned my_pairs = 0;
+    for (int v = v0 + blockIdx.x; v < v0 + nv; v += gridDim.x) {
+        const int nn = scnt[v], no = scnt[n + v], m = nn + no;
+        if (nn == 0) continue;   // every pair holds a new candidate
+        for (int i = lane; i < m; i += 32) {
+            const int id = i < nn ? samp[int64_t(v) * S + i]
+                                  : samp[(int64_t(n) + v) * S + i - nn];
+            sid[i] = id;
+            sthr[i] = Bk[int64_t(id) * k + k - 1];
+        }
+        __syncwarp();
+        for (int r = 0; r < m; ++r) {
+            const float *row = X + int64_t(sid[r]) * d;
+            for (int c = lane; c < d4; c += 32)
+                staged::cp_async16(sbase + uint32_t(r * rs4 + c) * 16u, row + 4 * c);
+        }
+        staged::cp_async_wait_all();
+        __syncwarp();
+        if (nn > 4)
+            join_tiles<2>(srow, rs4, d4, sid, sthr, nn, m, lane, pt, pk, pcount, pcap, my_pairs,
+                          dstatus);
+        else
+            join_tiles<1>(srow, rs4, d4, sid, sthr, nn, m, lane, pt, pk, pcount, pcap, my_pairs,
+                          dstatus);
+        __syncwarp();   // the next v's rows take their place
+    }
+    if (lane == 0 && my_pairs) atomicAdd(npairs, (unsigned long long)my_pairs);
+}
+
 // proposals per target; the targets that receive any are listed once each
 // (in no particular order: each target's merge is independent)
 __global__ void nnd_group_count_kernel(const int32_t *__restrict__ pt,
@@ -540,7 +714,14 @@ famst_status nndescent(const Exec &ex, Arena &ar, const float *X, int64_t n, int
     if (cudaMemsetAsync(rcnt, 0, size_t(2 * n + 1) * 4, ex.stream) != cudaSuccess ||
         cudaMemsetAsync(gcnt, 0, size_t(n + 1) * 4, ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
-    if (set_smem_attr(nnd_join_kernel, P.smem, ex.stream) != cudaSuccess) return FAMST_ERR_CUDA;
+    // One warp per v where shared memory holds the rows of ten or more per SM;
+    // with fewer the four warps of a block per v keep the SM busier. (The rows
+    // are copied 16 bytes at a time: aligned, d a multiple of 4.)
+    const int warps_per_sm = int(std::min<size_t>(32, NND_SMEM_SM / (P.smem + 1024 + 1024)));
+    const bool by_warp = vec4 && warps_per_sm >= 10;
+    if ((by_warp ? set_smem_attr(nnd_join_warp_kernel, P.smem, ex.stream)
+                 : set_smem_attr(nnd_join_kernel, P.smem, ex.stream)) != cudaSuccess)
+        return FAMST_ERR_CUDA;
     int it = 0;
     while (it < max_iters) {
         if (cudaMemsetAsync(cdev, 0, 16, ex.stream) != cudaSuccess) return FAMST_ERR_CUDA;
@@ -561,9 +742,16 @@ famst_status nndescent(const Exec &ex, Arena &ar, const float *X, int64_t n, int
             if (cudaMemsetAsync(pcount, 0, 8, ex.stream) != cudaSuccess ||
                 cudaMemsetAsync(nact, 0, 4, ex.stream) != cudaSuccess)
                 return FAMST_ERR_CUDA;
-            FAMST_LAUNCH(ex, nnd_join_kernel, unsigned(nv), NND_JOIN_THREADS, P.smem, X, d, ni, k,
-                         S, int(v0), P.rs4, samp, scnt, Bk, pt, pk, pcount,
-                         (unsigned long long)P.pcap, cdev + 1, int(vec4), ex.dstatus);
+            if (by_warp) {
+                FAMST_LAUNCH(ex, nnd_join_warp_kernel,
+                             unsigned(std::min<int64_t>(nv, int64_t(ex.num_sms) * warps_per_sm)),
+                             32, P.smem, X, d, ni, k, S, int(v0), int(nv), P.rs4, samp, scnt, Bk,
+                             pt, pk, pcount, (unsigned long long)P.pcap, cdev + 1, ex.dstatus);
+            } else {
+                FAMST_LAUNCH(ex, nnd_join_kernel, unsigned(nv), NND_JOIN_THREADS, P.smem, X, d, ni,
+                             k, S, int(v0), P.rs4, samp, scnt, Bk, pt, pk, pcount,
+                             (unsigned long long)P.pcap, cdev + 1, int(vec4), ex.dstatus);
+            }
             FAMST_LAUNCH(ex, nnd_group_count_kernel, sgrid, 256, 0, pt, pcount,
                          (unsigned long long)P.pcap, gcnt, act, nact);
             st = exclusive_scan_i32(ex, ar, gcnt, goff, n + 1, nullptr);

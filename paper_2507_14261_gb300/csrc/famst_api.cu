@@ -976,7 +976,7 @@ famst_status famst_refine(famst_ctx *ctx, const float *X, int64_t n, int32_t d,
     // Labels that no kNN edge leaves (Algorithm 2's own): G[u] needs no test
     // for the component, and the grouped scans of a build serve here too.
     const bool v4 = vec4_ok(X, d);
-    const bool may_group = v4 && d >= 32 && d <= 256;
+    const bool may_group = v4 && d >= 32 && d <= 256 && refine_grouped_pays(m, n, k, d);
     Arena ar;
     size_t ws = align256(size_t(n + 1) * 4) + align256(size_t(n) * k * 4) +
                 reverse_csr_workspace(n, k) + align256(size_t(max_iters + 1) * 4) +

@@ -721,6 +721,16 @@ famst_status refine_edges(const Exec &ex, Arena &ar, const float *X, int d, bool
                           int64_t m, int max_iters, int32_t *change_hist /*max_iters+1*/,
                           unsigned long long *evals = nullptr, bool check = true,
                           int *variant = nullptr);
+// Whether Alg. 4 of m edges takes the grouped sweeps. They cost some 0.55 ms of
+// launches and sorts and 0.22 ns per kNN entry (lists, BF16 rows) before the
+// first edge, and then about a fourth of the per-edge scans' 3 ps per edge, list
+// entry and coordinate. famst_refine, per edge / grouped: 756 edges of 15,436 x
+// 64 points, k 30: 0.27 / 0.80 ms; 49,500 of 30,000 x 128, k 16: 0.61 / 1.03;
+// 44,850 of 100,000 x 128, k 32: 0.98 / 1.73; 1.25M of 200,000 x 128, k 32:
+// 15.6 / 5.8.
+inline bool refine_grouped_pays(int64_t m, int64_t n, int k, int d) {
+    return double(m) * k * d >= 2.3e8 + 92.0 * double(n) * k;
+}
 // candidate filter of the refinement kernel that ran (build info)
 constexpr int REFINE_FILTER_NONE = 0;      // canonical distance per lane
 constexpr int REFINE_FILTER_FP32 = 1;      // FP32 grouped sums + canonical survivors

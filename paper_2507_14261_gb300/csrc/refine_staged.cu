@@ -678,6 +678,8 @@ size_t refine_build_workspace(int64_t n, int64_t m) {
 // then the remaining active edges run per edge. change_hist[c] receives the
 // number of edges that changed in exactly c sweeps (the bookkeeping of
 // refine_edges); pinned_host: two pinned host words.
+constexpr int64_t STAGED_ALL = 65536;
+
 famst_status refine_build(const Exec &ex, Arena &ar, const float *X, int d, const HalfRows &hr,
                           const int32_t *members, int64_t n, int32_t *eu, int32_t *ev, float *ew,
                           const int32_t *order, int64_t m, int max_iters, int32_t *change_hist,
@@ -717,7 +719,13 @@ famst_status refine_build(const Exec &ex, Arena &ar, const float *X, int d, cons
     FAMST_LAUNCH(ex, bsp_iota_kernel, blocks(m), th, 0, listA, m);
     int64_t active = m;
     int sweep = 0;
-    const int64_t tail_at = m / 16;
+    // Up to STAGED_ALL edges, all of them go to the per-edge kernel at once: the
+    // sweeps' launches, sorts and synchronisations cost more than the staged
+    // rows they share. Whole builds, sweeps / per edge: 6,125 edges of 100,000 x
+    // 128 blobs, k 16: 5.15 / 4.36 ms; 29,700 of 60,000 x 128, k 32: 3.75 / 3.02;
+    // 49,500 of 30,000 x 128, k 16: 2.84 / 2.31. With 5M edges (1M points) a
+    // staged row serves 4.5 scans and the sweeps win.
+    const int64_t tail_at = m <= STAGED_ALL ? m : m / 16;
     // sweep-synchronous sweeps (none when max_iters == 1: the per-edge kernel
     // then applies the cap)
     while (active > tail_at && sweep < max_iters - 1) {

@@ -18,7 +18,8 @@
 // holds the KC smallest scores with ids that came in with them.
 //
 // Host and device: the CPU tests compile this header with a host compiler
-// and check the networks exhaustively on 0-1 inputs.
+// and check the networks exhaustively on 0-1 inputs. (No kernel holds such
+// lists any more: the tensor tiles log their candidates instead.)
 #pragma once
 
 #if defined(__CUDACC__)

@@ -288,10 +288,11 @@ __device__ void block_sum2(double &a, double &b) {
 // The FP64 value of a float without the conversion unit: the FP64 pipe (two
 // lanes an SM here) bounds the lengths below, and conversions go through it.
 // Normal numbers only need their exponent rebased and their fields moved;
-// zeros and subnormals take the instruction.
+// zeros and subnormals (exponent 0), infinities and NaN (255) take the
+// instruction (both ends are at or above 0x7f000000 after the subtraction).
 __device__ __forceinline__ double widen(float f) {
     const uint32_t b = __float_as_uint(f), e = b & 0x7f800000u;
-    if (e == 0u) return double(f);
+    if (e - 0x00800000u >= 0x7f000000u) return double(f);
     return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)),
                             int(b << 29));
 }

@@ -368,6 +368,9 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
                     en = __ldg(g.en + base + idx);
                 }
                 const int nv = __popc(__ballot_sync(0xffffffffu, valid));
+                // of this lane's pair bits 4 T + e2, those of present candidates
+                const unsigned rows_in = (g4 < nv ? 0x03u : 0u) | (g4 + 8 < nv ? 0x0cu : 0u) |
+                                         (g4 + 16 < nv ? 0x30u : 0u) | (g4 + 24 < nv ? 0xc0u : 0u);
                 // the round's largest row error (non-negative floats order as integers)
                 const float ebm = __uint_as_float(
                     __reduce_max_sync(0xffffffffu, __float_as_uint(en.x)));
@@ -430,7 +433,8 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
                                 const float nn = __fadd_rn(nx[c], ny);
                                 const float pt = __fmaf_rn(-2.0f, acc[T][2 * h + c], nn);
                                 const float A = __fmaf_ru(nn, aerr, 1e-35f);
-                                lo[T][2 * h + c] = __fsub_rd(pt, A);
+                                // (p~ beyond the FP32 range, or NaN with A = +inf)
+                                lo[T][2 * h + c] = __fsub_rd(fminf(pt, 0x1.fffffep127f), A);
                                 mh[c] = fminf(mh[c], __fadd_ru(pt, A));
                             }
                         }
@@ -455,13 +459,15 @@ __global__ void __launch_bounds__(Stage<NKS>::WARPS * 32, MINB)
                     // survivors, decided on canonical distances by the whole
                     // warp, up to four at a time; bit 4 T + e2 of `my` marks a
                     // surviving pair of this lane (one copy of the batch code).
-                    // (an absent candidate's lo is NaN or +inf, an absent task's lim -inf)
                     unsigned my = 0;
 #pragma unroll
                     for (int T = 0; T < 2; ++T)
 #pragma unroll
                         for (int e2 = 0; e2 < 4; ++e2)
                             if (lo[T][e2] <= lim[e2 & 1]) my |= 1u << (4 * T + e2);
+                    // (the bounds of an absent candidate or task say nothing: lim
+                    // is +inf once the incumbent's squared bound overflows)
+                    my &= rows_in & ((2 * t4 < ntb ? 0x55u : 0u) | (2 * t4 + 1 < ntb ? 0xaau : 0u));
                     // the surviving pairs as one list of (candidate, task) codes
                     int at = __popc(my);
 #pragma unroll

@@ -98,14 +98,17 @@ __device__ __forceinline__ void round_dots(uint32_t sbuf, const uint32_t (&b0)[N
 // product dt of centred rows with norms nx, ny and row error bounds ebx,
 // eby: |p~ - ||h_x - h_y||^2| <= aerr (nx + ny) + 1e-35 with
 // p~ = nx + ny - 2 dt, ||(h_y - h_x) - (y - x)|| <= ebx + eby, and eps for
-// the canonical sum's own error; directed rounding throughout.
+// the canonical sum's own error; directed rounding throughout. Where a norm or
+// p~ leaves the FP32 range the bounds are those of the largest float or say
+// nothing (lo = 0, hi = +inf): p~ is NaN only with A = +inf, and fminf and
+// fmaxf return the operand that is a number.
 __device__ __forceinline__ void dist_bounds(float dt, float nx, float ny, float ebx, float eby,
                                             float aerr, float eps, float &lo, float &hi) {
     const float nn = __fadd_rn(nx, ny);
     const float pt = __fmaf_rn(-2.0f, dt, nn);
     const float A = __fmaf_ru(nn, aerr, 1e-35f);
-    const float slo = __fsqrt_rd(fmaxf(__fsub_rd(pt, A), 0.0f));
-    const float shi = __fsqrt_ru(__fadd_ru(pt, A));
+    const float slo = __fsqrt_rd(fmaxf(__fsub_rd(fminf(pt, 0x1.fffffep127f), A), 0.0f));
+    const float shi = __fsqrt_ru(fminf(__fadd_ru(pt, A), __int_as_float(0x7f800000)));
     const float E = __fadd_ru(ebx, eby);
     lo = fmaxf(__fmul_rd(__fsub_rd(slo, E), 1.0f - eps), 0.0f);
     hi = __fmul_ru(__fadd_ru(shi, E), 1.0f + eps);

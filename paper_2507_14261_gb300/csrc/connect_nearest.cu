@@ -32,8 +32,9 @@
 // latency (TMEM load, score, compare: 1.8 ms with it, 2.5 ms with the
 // survivors; eight epilogue warps instead of sixteen: 3.2 ms). The whole call
 // there: 33.1 ms with the warp kernel below, 3.2 ms.
-// Small clouds, and inputs with so many ties that the survivors overflow
-// their buffer, take the warp kernel below:
+// Small clouds, inputs with so many ties that the survivors overflow their
+// buffer, and points whose squares leave the FP32 range take the warp kernel
+// below:
 //  * a work item is a block of 32 consecutive members of one component C_i;
 //    its warp stages their BF16 rows in shared memory once and then streams
 //    the members of every later component C_j (j > i), eight per step, as
@@ -164,6 +165,7 @@ constexpr int NT_FLUSH = 16;   // queued survivors at which a tile ends with a f
 constexpr int NT_THREADS = 64 + 32 * NT_EPI;
 constexpr int NT_SAMPLES = 1024;
 constexpr int NT_SW = 4;       // warps of a component pair's sample
+constexpr unsigned long long NT_TOO_MANY = 1ull << 62;   // above any survivor buffer
 
 struct NtItem {
     int32_t row0, row_end;   // sorted rows row0 .. min(row0 + 127, row_end - 1), of component i
@@ -198,7 +200,8 @@ __global__ void nt_gather_kernel(const __nv_bfloat16 *__restrict__ H, int ld,
                                  const int32_t *__restrict__ comp_off, int64_t t, int64_t n,
                                  int64_t npad, float aerr, __nv_bfloat16 *__restrict__ Hs,
                                  float *__restrict__ n2, float *__restrict__ eb,
-                                 float *__restrict__ nyq, int32_t *__restrict__ colcomp) {
+                                 float *__restrict__ nyq, int32_t *__restrict__ colcomp,
+                                 unsigned long long *__restrict__ count) {
     const int64_t pos = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (pos >= npad) return;
@@ -222,6 +225,9 @@ __global__ void nt_gather_kernel(const __nv_bfloat16 *__restrict__ H, int ld,
         }
         colcomp[pos] = int32_t(lo);
         const float v = hn2[r];
+        // the thresholds' squares need room in the FP32 range: beyond it the
+        // survivors count as too many, and the warp kernel takes the call
+        if (!(v < 1e36f)) *count = NT_TOO_MANY;
         n2[pos] = v;
         eb[pos] = heb[r];
         nyq[pos] = __fmul_rd(v, 1.0f - (aerr + 0x1p-20f));
@@ -1070,7 +1076,7 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
         cudaMemsetAsync(cnt, 0, size_t(npairs + 1) * 4, ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
     FAMST_LAUNCH(ex, nt_gather_kernel, unsigned((npad * 32 + 255) / 256), 256, 0, hr.h, hr.ld,
-                 hr.eb, hr.n2, members, comp_off, t, n, npad, aerr, Hs, n2, eb, nyq, colcomp);
+                 hr.eb, hr.n2, members, comp_off, t, n, npad, aerr, Hs, n2, eb, nyq, colcomp, count);
     FAMST_LAUNCH(ex, nt_chunk_kernel, unsigned((npad / 16 + 255) / 256), 256, 0, colcomp, eb, n,
                  npad / 16, 16, t, chunk);
     FAMST_LAUNCH(ex, nt_chunk_kernel, unsigned((npad / NT_COLS + 63) / 64), 64, 0, colcomp, eb, n,

@@ -56,6 +56,7 @@
 
 #include "famst_internal.cuh"
 #include "mbarrier.cuh"
+#include "nearest_plan.h"
 #include "staged_rows.cuh"
 #include "tcgen05.cuh"
 
@@ -152,7 +153,6 @@ __device__ __forceinline__ void pairs_batch(const float *__restrict__ X, int d, 
     }
 }
 
-// pair p -> (i, j), pairs enumerated i outer, j inner
 // ------------------------------------------------ all pairs on tcgen05
 
 constexpr int NT_M = 128;      // rows of an item (TMEM lanes)
@@ -986,18 +986,13 @@ famst_status launch_np(const Exec &ex, const float *X, int d, const HalfRows &hr
 
 namespace {
 
-// room for the survivors of the tensor pass
-int64_t nt_cap(int64_t n, int64_t t) {
-    return std::min((int64_t(1) << 22) + 64 * (t * (t - 1) / 2), n * (n - 1) / 2 + 1);
-}
-
 // Below this the sampling, grouping and selection around the tile pass
 // (about 0.3 ms of launches) cost more than the warp kernel's whole run:
 // 4100 x 128 in 10 components 1.47 ms warp kernel, 0.48 ms tiles.
 constexpr int64_t NT_MIN_N = 1024;
 
 size_t nt_workspace(int64_t n, int64_t t, int lambda) {
-    const int64_t npairs = t * (t - 1) / 2, cap = nt_cap(n, t);
+    const int64_t npairs = nearest_pairs(t), cap = nearest_cap(n, t, lambda);
     const int64_t npad = (n + NT_N - 1) / NT_N * NT_N;
     const int64_t items = (n / NT_M + t) * 2 + 16 * 1024;
     return align256(size_t(npad) * 256 * 2) + align256(size_t(npad) * 4) * 4 +
@@ -1017,7 +1012,7 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
                         int32_t *eu, int32_t *ev, float *ew, int32_t *eci, int32_t *ecj,
                         bool *done) {
     *done = false;
-    const int64_t n = comp_off_host[t], npairs = t * (t - 1) / 2, cap = nt_cap(n, t);
+    const int64_t n = comp_off_host[t], npairs = nearest_pairs(t), cap = nearest_cap(n, t, lambda);
     const int64_t ntile = (n + NT_N - 1) / NT_N, npad = ntile * NT_N;
     // items: 128 rows of a component against a run of the tiles that hold
     // later components; runs of about a sixteenth of an SM's share, so that
@@ -1143,10 +1138,7 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
 }  // namespace
 
 size_t connect_nearest_workspace(int64_t n, int64_t t, int lambda) {
-    // the warp kernel's lists: sum over i of ceil(|C_i| / 32) (t - 1 - i) <= (n / 32 + t) t
-    const int64_t lists = (n / 32 + t) * t;
-    const size_t warp =
-        2 * align256(size_t(t + 1) * 8) + 3 * align256(size_t(lists) * lambda * 4) + 256;
+    const size_t warp = 2 * align256(size_t(t + 1) * 8) + nearest_warp_bytes(n, t, lambda) + 1024;
     return std::max(warp, n >= NT_MIN_N ? nt_workspace(n, t, lambda) : 0);
 }
 

@@ -23,7 +23,9 @@
 //    of lambda distinct pairs, so no pair above their maximum is needed. The
 //    first rows of every component go first, in a launch of their own: the
 //    rest then meets bounds that a part of each component pair has set,
-//    instead of all its CTAs passing the sample's bound at once;
+//    instead of all its CTAs passing the sample's bound at once. With many
+//    component pairs that launch stores nothing and only lowers the bounds:
+//    most survivors pass before them (nearest_plan.h);
 //  * the survivors (a few hundred per component pair) are filtered with the
 //    final thr, grouped by component pair, and decided on canonical FP32
 //    distances by a warp per component pair.
@@ -31,10 +33,11 @@
 // for 100k x 128 in 50 components without an epilogue) and the epilogue's
 // latency (TMEM load, score, compare: 1.8 ms with it, 2.5 ms with the
 // survivors; eight epilogue warps instead of sixteen: 3.2 ms). The whole call
-// there: 33.1 ms with the warp kernel below, 3.2 ms.
-// Small clouds, inputs with so many ties that the survivors overflow their
-// buffer, and points whose squares leave the FP32 range take the warp kernel
-// below:
+// there: 33.1 ms with the warp kernel below, 3.1 ms; 1M x 128 points in 1000
+// components, lambda 10: 2514 and 689 ms.
+// Small clouds, many small components (nearest_plan.h), inputs with so many
+// ties that the survivors overflow their buffer, and points whose squares leave
+// the FP32 range take the warp kernel below:
 //  * a work item is a block of 32 consecutive members of one component C_i;
 //    its warp stages their BF16 rows in shared memory once and then streams
 //    the members of every later component C_j (j > i), eight per step, as
@@ -185,7 +188,8 @@ struct NtArgs {
     const int4 *hchunk;      // the same per NT_COLS
     unsigned *thr;           // per component pair: bound on its lambda-th distance (float bits)
     unsigned *slots;         // per component pair: lambda upper bounds (float bits)
-    unsigned long long *count, cap;
+    unsigned long long *count, cap;   // survivors found, room for them
+    unsigned long long limit;         // with more the search has failed
     int32_t *su, *sv;        // survivors: sorted rows, lower bound
     float *sl;
     float aerr, eps;
@@ -366,6 +370,10 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const NtItem I = args.items[blockIdx.x];
     const int ntiles = I.kt1 - I.kt0;
+    if (threadIdx.x == 0)
+        *abort_flag = *reinterpret_cast<volatile unsigned long long *>(args.count) > args.limit;
+    __syncthreads();
+    if (*abort_flag) return;
     if (threadIdx.x == 0) {
         for (int s = 0; s < args.stages; ++s) {
             mbar_init(&full[s], 1);
@@ -377,7 +385,6 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             mbar_init(&tempty[b], NT_EPI);
         }
         mbar_init(mma_done, 1);
-        *abort_flag = 0;
         mbar_init_fence();
     }
     if (warp == 1) {
@@ -501,10 +508,11 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 const float th = thr_of(c);
                 if (!(lo <= __fmul_ru(th, 1.0f + 0x1p-22f))) continue;
                 const unsigned long long at = atomicAdd(args.count, 1ull);
-                if (at >= args.cap) continue;
-                args.su[at] = I.row0 + quarter * 32 + ln;
-                args.sv[at] = pos;
-                args.sl[at] = lo;
+                if (at < args.cap) {
+                    args.su[at] = I.row0 + quarter * 32 + ln;
+                    args.sv[at] = pos;
+                    args.sl[at] = lo;
+                }
                 if (hi < th)
                     nt_slot_insert(args.slots + (pbase + c) * args.lambda, args.thr + pbase + c,
                                    args.lambda, __float_as_uint(hi));
@@ -525,7 +533,7 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             curthr = fminf(curthr, nthr);
             const float bh = hc.x == hc.y ? bound_of(hc.x) : 0.0f;
             nthr = cur >= 0 ? thr_of(cur) : inf;
-            const bool over = seen > args.cap;
+            const bool over = seen > args.limit;
             if ((g & 15) == 15) seen = *reinterpret_cast<volatile unsigned long long *>(args.count);
             float T = hc.x == hc.y ? limit(bh, hc.z) : 0.0f;
             // the next tile's norms and its record into L1 meanwhile
@@ -590,8 +598,8 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     cnt += __popc(who);
                 }
             };
-            // a full survivor buffer ends the search (the caller starts over
-            // on the warp kernel); the tiles still flow
+            // too many survivors end the search (the caller starts over on the
+            // warp kernel); this CTA's tiles still flow, later CTAs leave at once
             if (!__any_sync(0xffffffffu, over) && (hc.x != hc.y || bh >= 0.0f)) {
                 uint32_t va[16], vb[16];
                 __syncwarp();
@@ -624,6 +632,17 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
+}
+
+// Between the launch that only lowers the bounds and the search: the slots
+// start again (the search meets the same pairs once more, and a slot has to
+// hold a pair of its own), the bounds stay.
+__global__ void nt_restart_kernel(unsigned *__restrict__ slots, int64_t nslots,
+                                  unsigned long long *__restrict__ count,
+                                  unsigned long long limit) {
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i < nslots) slots[i] = 0x7f800000u;
+    if (i == 0 && *count <= limit) *count = 0;
 }
 
 // Survivors within the final bounds, counted per component pair (slot: the
@@ -992,7 +1011,7 @@ namespace {
 constexpr int64_t NT_MIN_N = 1024;
 
 size_t nt_workspace(int64_t n, int64_t t, int lambda) {
-    const int64_t npairs = nearest_pairs(t), cap = nearest_cap(n, t, lambda);
+    const int64_t npairs = nearest_pairs(t), cap = nearest_plan(n, t, lambda).cap;
     const int64_t npad = (n + NT_N - 1) / NT_N * NT_N;
     const int64_t items = (n / NT_M + t) * 2 + 16 * 1024;
     return align256(size_t(npad) * 256 * 2) + align256(size_t(npad) * 4) * 4 +
@@ -1012,7 +1031,10 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
                         int32_t *eu, int32_t *ev, float *ew, int32_t *eci, int32_t *ecj,
                         bool *done) {
     *done = false;
-    const int64_t n = comp_off_host[t], npairs = nearest_pairs(t), cap = nearest_cap(n, t, lambda);
+    const int64_t n = comp_off_host[t], npairs = nearest_pairs(t);
+    const NearestPlan plan = nearest_plan(n, t, lambda);
+    const int64_t cap = plan.cap;
+    const bool bounds_first = plan.bounds_first;
     const int64_t ntile = (n + NT_N - 1) / NT_N, npad = ntile * NT_N;
     // items: 128 rows of a component against a run of the tiles that hold
     // later components; runs of about a sixteenth of an SM's share, so that
@@ -1040,10 +1062,14 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
             items.push_back(I);
         }
     };
+    // (bounds_first: the first launch only lowers the bounds, and the search
+    // goes over all rows)
     for (int64_t i = 0; i + 1 < t; ++i) add(i, comp_off_host[i], run1);
     const size_t first = items.size();
     for (int64_t i = 0; i + 1 < t; ++i)
-        for (int64_t r = comp_off_host[i] + NT_M; r < comp_off_host[i + 1]; r += NT_M) add(i, r, run);
+        for (int64_t r = comp_off_host[i] + (bounds_first ? 0 : NT_M); r < comp_off_host[i + 1];
+             r += NT_M)
+            add(i, r, run);
     __nv_bfloat16 *Hs = ar.take<__nv_bfloat16>(size_t(npad) * hr.ld);
     float *n2 = ar.take<float>(size_t(npad));
     float *eb = ar.take<float>(size_t(npad));
@@ -1109,7 +1135,17 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
     a.eps = eps;
     a.status = ex.dstatus;
     if (set_smem_attr(nearest_tc_kernel, smem, ex.stream) != cudaSuccess) return FAMST_ERR_CUDA;
+    a.limit = a.cap;
+    if (bounds_first) {
+        a.cap = 0;
+        a.limit *= 8;
+    }
     FAMST_LAUNCH(ex, nearest_tc_kernel, unsigned(first), NT_THREADS, smem, mA, mB, a);
+    if (bounds_first) {
+        FAMST_LAUNCH(ex, nt_restart_kernel, unsigned((npairs * lambda + 255) / 256), 256, 0, slots,
+                     npairs * lambda, count, a.limit);
+        a.cap = a.limit = (unsigned long long)cap;
+    }
     if (items.size() > first) {
         a.items = d_items + first;
         FAMST_LAUNCH(ex, nearest_tc_kernel, unsigned(items.size() - first), NT_THREADS, smem, mA, mB,
@@ -1139,7 +1175,8 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
 
 size_t connect_nearest_workspace(int64_t n, int64_t t, int lambda) {
     const size_t warp = 2 * align256(size_t(t + 1) * 8) + nearest_warp_bytes(n, t, lambda) + 1024;
-    return std::max(warp, n >= NT_MIN_N ? nt_workspace(n, t, lambda) : 0);
+    const bool tensor = n >= NT_MIN_N && nearest_plan(n, t, lambda).tensor;
+    return std::max(warp, tensor ? nt_workspace(n, t, lambda) : 0);
 }
 
 // comp_off_host: the t + 1 member offsets on the host (the list layout is
@@ -1153,7 +1190,8 @@ famst_status connect_nearest(const Exec &ex, Arena &ar, const float *X, int d,
     if (!hr.h || hr.ld > 256) return FAMST_ERR_UNSUPPORTED;
     const float aerr = float(hr.ld * std::ldexp(1.0, -19) + std::ldexp(1.0, -20));
     const float eps = float((d + 16) * std::ldexp(1.0, -24) * 1.1);
-    if (comp_off_host[t] >= NT_MIN_N && encode_fn()) {
+    if (comp_off_host[t] >= NT_MIN_N && nearest_plan(comp_off_host[t], t, lambda).tensor &&
+        encode_fn()) {
         const size_t mark = ar.off;
         bool done = false;
         const famst_status s =

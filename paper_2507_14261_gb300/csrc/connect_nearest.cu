@@ -680,7 +680,8 @@ __global__ void nt_select_kernel(const float *__restrict__ X, int d,
                                  const int2 *__restrict__ grouped, const int32_t *__restrict__ off,
                                  int64_t t, int lambda, int32_t *__restrict__ eu_out,
                                  int32_t *__restrict__ ev_out, float *__restrict__ ew_out,
-                                 int32_t *__restrict__ eci, int32_t *__restrict__ ecj) {
+                                 int32_t *__restrict__ eci, int32_t *__restrict__ ecj,
+                                 int *status) {
     const int64_t npairs = t * (t - 1) / 2;
     const int64_t w0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -690,7 +691,12 @@ __global__ void nt_select_kernel(const float *__restrict__ X, int d,
         pair_of(p, t, i, j);
         uint64_t eh = ~0ull;
         uint32_t el = ~0u;
-        int eu = -1, ev = -1, have = 0;
+        int eu = 0, ev = 0, have = 0;
+        if (off[p] == off[p + 1]) {   // the nearest pair always survives: a bug, never an id of -1
+            if (lane == 0) set_status(status, STATUS_INTERNAL);
+            eh = 0;
+            have = 1;
+        }
         for (int e0 = off[p]; e0 < off[p + 1]; e0 += 4) {
             int qa[4], qb[4];
 #pragma unroll
@@ -1152,9 +1158,12 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
                      a);
     }
     unsigned long long got = 0;
+    int status = 0;
     if (cudaMemcpyAsync(&got, count, 8, cudaMemcpyDeviceToHost, ex.stream) != cudaSuccess ||
+        cudaMemcpyAsync(&status, ex.dstatus, 4, cudaMemcpyDeviceToHost, ex.stream) != cudaSuccess ||
         cudaStreamSynchronize(ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
+    if (status & STATUS_LOOP_LIMIT) return FAMST_ERR_TIMEOUT;   // a tile gave up: pairs are missing
     if (got > (unsigned long long)cap) return FAMST_OK;
     const unsigned sgrid = unsigned((got + 255) / 256);
     if (got > 0)
@@ -1166,7 +1175,7 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
         FAMST_LAUNCH(ex, nt_scatter_kernel, sgrid, 256, 0, su, sv, int64_t(got), t, colcomp,
                      members, off, slot, grouped);
     FAMST_LAUNCH(ex, nt_select_kernel<XR>, pgrid, 128, 0, X, d, grouped, off, t, lambda, eu, ev, ew,
-                 eci, ecj);
+                 eci, ecj, ex.dstatus);
     *done = true;
     return cudaPeekAtLastError() == cudaSuccess ? FAMST_OK : FAMST_ERR_CUDA;
 }

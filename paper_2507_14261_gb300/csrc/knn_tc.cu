@@ -71,11 +71,12 @@
 #include "famst_internal.cuh"
 #include "mbarrier.cuh"
 #include "tcgen05.cuh"
+#include "tile_rows.cuh"
 
 namespace famst {
 namespace {
 
-constexpr int BM = 128;          // query rows per CTA (TMEM lanes)
+constexpr int BM = tile::ROWS;   // query rows per CTA (TMEM lanes)
 constexpr int BN = 256;          // keys per tile (accumulator columns)
 constexpr int BK = TC_BK;        // K elements per stage (one 128-byte swizzle atom)
 constexpr int A_BLOCK = BM * BK * 2;   // 16 KB
@@ -254,6 +255,20 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     int *slot_sh = reinterpret_cast<int *>(tmem_slot + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // row `row` of this CTA's items from `item` on, when their tiles were given up
+    auto give_up = [&](int item, int row) {
+        for (; item < nitems; item += gridDim.x) {
+            const Item I = item_of(item);
+            if (I.q0 + row >= I.row_end) continue;
+            const tile::RowSlot at = tile::row_slot(I.q0, row, I.shift, I.part);
+            if constexpr (TOP1) {   // any pivot
+                args.cand[at.at] = 0;
+                args.splus[at.at] = 0.0f;
+            } else {
+                tile::give_up_row(at, args.ccnt, args.splus, args.side_cnt, args.side_splus);
+            }
+        }
+    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < args.stages; ++s) {
@@ -282,7 +297,10 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
     if constexpr (!TOP1) {
         __syncthreads();
-        if (*slot_sh < 0) return;
+        if (*slot_sh < 0) {
+            if (threadIdx.x < BM) give_up(blockIdx.x, threadIdx.x);
+            return;
+        }
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
@@ -606,6 +624,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         // the logs are complete; a failure anywhere stops every warp here
         const bool failed = epilogue_bar_any(32 * EPI, !ok);
+        if (failed && grp == 0) give_up(item, row);
         if constexpr (TOP1) {
             if (!failed && grp == 0 && mine) {
                 float s = t_sh[row];
@@ -705,9 +724,8 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     sp = select_bound(count, lo, hi, Tr, args.sel, sqrtf(__ldg(args.ny + ri)), ym);
                 }
                 // out: the candidates at or below sp
-                const size_t at0 =
-                    (I.part > 0 ? size_t(I.part - 1) * BM + rr : size_t(ri - I.shift)) *
-                    size_t(args.cap);
+                const tile::RowSlot slot = tile::row_slot(I.q0, rr, I.shift, I.part);
+                const size_t at0 = slot.at * size_t(args.cap);
                 int out = 0;
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
@@ -717,7 +735,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     if (in && to_row < args.cap) {
                         const size_t to = at0 + to_row;
                         const int j = fj[32 * h + lane] - I.shift;
-                        if (I.part > 0) {
+                        if (slot.side) {
                             args.side_j[to] = j;
                             args.side_s[to] = sv[h];
                         } else {
@@ -732,14 +750,8 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 }
                 if (lane == 0) {
                     if (lost) sp = -inf;   // never certified
-                    if (I.part > 0) {
-                        const size_t at = size_t(I.part - 1) * BM + rr;
-                        args.side_cnt[at] = out;
-                        args.side_splus[at] = sp;
-                    } else {
-                        args.ccnt[ri - I.shift] = out;
-                        args.splus[ri - I.shift] = sp;
-                    }
+                    (slot.side ? args.side_cnt : args.ccnt)[slot.at] = out;
+                    (slot.side ? args.side_splus : args.splus)[slot.at] = sp;
                 }
                 __syncwarp();
             }

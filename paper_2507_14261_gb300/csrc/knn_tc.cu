@@ -1058,6 +1058,11 @@ inline CertConst cert_const(double eps_dot, int d) {
                      float((1.0 - (d + 4.0) * u * 1.05) * (1.0 - 0x1p-22))};
 }
 
+// Largest |y| of a cloud whose scores are all finite: beyond it a key's squared
+// norm may leave the FP32 range, its score is +inf or NaN, and the tiles neither
+// keep nor count it.
+constexpr float NORM_MAX = 1e18f;
+
 // Whether no key left out can be at a canonical distance <= kw: keys of
 // skipped tiles lie at a true distance >= skip, other keys left out have a
 // score above sp. First in FP32 with every rounding on the safe side, which
@@ -1069,6 +1074,7 @@ template <class Eps64>
 __device__ __forceinline__ bool certified(float kw, float skip, float sp, float xn2f, float ymf,
                                           int d, const CertConst &cc, Eps64 eps64) {
     const float inf = __int_as_float(0x7f800000);
+    if (!(ymf < NORM_MAX)) return false;
     {
         const float u = 0x1p-24f;
         const float xn = __fsqrt_ru(xn2f), xy = __fmul_ru(xn, ymf), yy = __fmul_ru(ymf, ymf);

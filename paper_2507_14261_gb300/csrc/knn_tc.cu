@@ -66,6 +66,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <type_traits>
 
 #include "famst_internal.cuh"
@@ -1060,7 +1061,8 @@ inline CertConst cert_const(double eps_dot, int d) {
 
 // Largest |y| of a cloud whose scores are all finite: beyond it a key's squared
 // norm may leave the FP32 range, its score is +inf or NaN, and the tiles neither
-// keep nor count it.
+// keep nor count it. The distances between pivots are then no lower bounds either
+// (a square beyond the range makes one +inf), and no tile is pruned.
 constexpr float NORM_MAX = 1e18f;
 
 // Whether no key left out can be at a canonical distance <= kw: keys of
@@ -1656,7 +1658,8 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     }
     if (npad > n)
         FAMST_LAUNCH(ex, fill_inf_kernel, unsigned((npad - n + 255) / 256), 256, 0, ny, n, npad);
-    const bool use_prune = prune && !colcomp && prune_supported(n, d, k, vec4);
+    bool use_prune = prune && !colcomp && prune_supported(n, d, k, vec4);
+    const size_t before_prune = ar.off;
     // persistent launches: one CTA per SM takes the query tiles round-robin
     const unsigned pgrid = unsigned(std::min<int64_t>(p.nq_tiles, ex.num_sms));
     PruneOut P;
@@ -1672,6 +1675,8 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         // them as float4 from tile starts, and k0 need not be a multiple of 4
         float *nya = ar.take<float>(size_t(Kpadmax + BN));
         if (!piv || !Hp || !nyp || !nya) return FAMST_ERR_OOM;
+        if (cudaMemcpyAsync(pinned_host, ymax, 4, cudaMemcpyDeviceToHost, ex.stream) != cudaSuccess)
+            return FAMST_ERR_CUDA;
         famst_status st =
             prune_pivot_operands(ex, H, p.kh, ny, n, K0, Kpadmax + BN, piv, Hp, nyp);
         if (st != FAMST_OK) return st;
@@ -1720,15 +1725,23 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
             K += M;
         }
         if (st != FAMST_OK) return st;
-        st = prune_partition(ex, ar, X, d, n, k, H, p.kh, ny, p.nkb, K, piv, top, 1,
-                             pinned_host + 2, &P);
-        if (st != FAMST_OK) return st;
+        // (the passes above have waited for the stream)
+        float norm_max;
+        std::memcpy(&norm_max, pinned_host, 4);
+        if (!(norm_max < NORM_MAX)) {
+            use_prune = false;
+            ar.off = before_prune;
+        } else {
+            st = prune_partition(ex, ar, X, d, n, k, H, p.kh, ny, p.nkb, K, piv, top, 1,
+                                 pinned_host + 2, &P);
+            if (st != FAMST_OK) return st;
+        }
     }
     if (f32) {
         *uncertified = 0;
         if (tiles_visited) *tiles_visited = p.nq_tiles * p.nk_tiles;
         return use_prune ? knn_fp32_pruned(ex, ar, X, n, d, k, P, nbr, dist)
-                         : FAMST_ERR_UNSUPPORTED;
+                         : knn_fp32(ex, ar, X, n, d, k, nullptr, 0, n, nbr, dist);
     }
     int32_t *side_j = nullptr, *side_cnt = nullptr;   // candidates of the parts of split lists
     float *side_s = nullptr, *side_sp = nullptr;

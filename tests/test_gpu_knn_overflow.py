@@ -52,3 +52,24 @@ def test_batch(orc, ctx):
         ref = orc.famst(x, 6, 3, 5)
         assert int(t[b]) == ref.C.t
         np.testing.assert_array_equal(np.sort(trees[b].w.cpu().numpy()), np.sort(ref.tree.w))
+
+
+def spread(n, d, seed):
+    """One cloud whose squared distances lie around the end of the FP32 range:
+    many pairs overflow, but no point's nearest ones."""
+    rng = np.random.default_rng(seed)
+    return np.ascontiguousarray(rng.standard_normal((n, d)) * 3.5e18, dtype=np.float32)
+
+
+# sizes whose tiles are pruned where the norms allow it
+@pytest.mark.parametrize("n,d,k,precs", [(5000, 12, 8, ("bf16x3", "bf16", "fp32")),
+                                         (28000, 16, 10, ("fp32", "bf16x3"))])
+@pytest.mark.parametrize("cloud", [camps, spread])
+def test_pruned_sizes(orc, ctx, n, d, k, precs, cloud):
+    X = cloud(n, d, n)
+    rows = np.random.default_rng(1).choice(n, 1500, replace=False).astype(np.int32)
+    rn, rd = orc.knn_rows(X, k, rows)
+    for prec in precs:
+        nbr, dist = ctx.knn_graph(torch.from_numpy(X).cuda(), k, prec)
+        np.testing.assert_array_equal(nbr.cpu().numpy()[rows], rn)
+        np.testing.assert_array_equal(dist.cpu().numpy()[rows], rd)

@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "batch.cuh"
+#include "tile_rows.cuh"
 
 namespace famst {
 namespace {
@@ -166,7 +167,11 @@ __global__ void bt_check_forest_kernel(const long long *__restrict__ edges, int6
 // first): sort key of row v = its cloud in the top cb bits, then the top
 // bits of its projection on a fixed +-1 direction (order-preserving bits of
 // the FP32 value). Rows of FP32-tile clouds keep their order (projection
-// bits 0; the sort is stable).
+// bits 0; the sort is stable). Tensor clouds' rows enter the sort in a
+// scrambled order, so that equal projections come out without one: those of a
+// pixel grid tie along its diagonals, which would keep the index's period
+// (tile_rows.cuh; 16 grids 32 and 128 wide, 90,000 points, k = 16: 45,900 rows
+// lost their certificate, 8.6 ms; now none, 1.9 ms).
 __global__ void bt_proj_key_kernel(const float *__restrict__ Xc, int D, int64_t N,
                                    const long long *__restrict__ voff, int B,
                                    const CloudDev *__restrict__ cl, int cb,
@@ -176,12 +181,15 @@ __global__ void bt_proj_key_kernel(const float *__restrict__ Xc, int D, int64_t 
     if (v >= N) return;
     const int b = cloud_of_v(voff, B, v);
     const bool tc = cl[b].use_tc != 0;
+    int64_t row = v;
     float p = 0.0f;
-    if (tc)
+    if (tc) {
+        row = voff[b] + tile::scrambled_row(int(v - voff[b]), int(voff[b + 1] - voff[b]));
         for (int t = lane; t < D; t += 32) {
-            const float x = Xc[v * D + t];
+            const float x = Xc[row * D + t];
             p += ((uint32_t(t) * 0x9E3779B1u) >> 31) ? x : -x;
         }
+    }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
     if (lane == 0) {
@@ -190,7 +198,7 @@ __global__ void bt_proj_key_kernel(const float *__restrict__ Xc, int D, int64_t 
         const uint32_t hi = cb > 0 ? uint32_t(b) << (32 - cb) : 0u;
         const uint32_t lo = tc ? (cb > 0 ? u >> cb : u) : 0u;
         keys[v] = hi | lo;
-        vals[v] = int32_t(v);
+        vals[v] = int32_t(row);
     }
 }
 

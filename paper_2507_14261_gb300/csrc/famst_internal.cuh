@@ -593,7 +593,7 @@ famst_status visited_rows(const Exec &ex, Arena &ar, const PruneOut &P, int64_t 
 famst_status exact_rows(const Exec &ex, const float *X, int64_t n, int d, int k,
                         const int32_t *rows, const int32_t *count, int64_t max_rows,
                         const int32_t *colcomp, int32_t *nbr, float *dist);
-int prune_pivots(int64_t n);      // evenly spaced pivots
+int prune_pivots(int64_t n);      // one pivot of every n / K rows
 int prune_extra(int64_t n);       // pivots added by each of the two coverage passes
 int prune_pivots_max(int64_t n);
 bool prune_supported(int64_t n, int d, int k, bool vec4);

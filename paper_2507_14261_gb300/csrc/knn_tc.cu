@@ -28,7 +28,9 @@
 //                new one goes in by R min/max pairs. The row's T is the largest
 //                of its four threads' R-th (shared memory): each list holds R
 //                distinct keys' scores at or below it, so at least 4 R keys
-//                score <= T.
+//                score <= T. (Tight when the near keys are spread over the four
+//                column groups and do not come last: passes without pruned
+//                lists take the rows in a scrambled order, tile_rows.cuh.)
 //              - log: a key that scores at most the T of the moment is appended
 //                to the thread's log of (score, id) in a scratch area of the
 //                CTA (about 4 R ln(keys / 4 R) entries per row, L2-resident).
@@ -78,7 +80,7 @@ namespace famst {
 namespace {
 
 constexpr int BM = tile::ROWS;   // query rows per CTA (TMEM lanes)
-constexpr int BN = 256;          // keys per tile (accumulator columns)
+constexpr int BN = tile::KEYS;   // keys per tile (accumulator columns)
 constexpr int BK = TC_BK;        // K elements per stage (one 128-byte swizzle atom)
 constexpr int A_BLOCK = BM * BK * 2;   // 16 KB
 constexpr int B_BLOCK = BN * BK * 2;   // 32 KB
@@ -895,7 +897,10 @@ __global__ void colsum_final_kernel(const double *__restrict__ part, int nb, int
 }
 
 // One warp per row: centred row, BF16 hi (and lo) operand rows, FP32 norm.
+// `scrambled`: operand row and key norm at position p are those of row
+// scrambled_row(p) (xnorm stays by row).
 __global__ void tc_prep_kernel(const float *__restrict__ X, int64_t n, int d, int d_pad, int x3,
+                               int scrambled,
                                const float *__restrict__ mean, __nv_bfloat16 *__restrict__ H,
                                float *__restrict__ ny, float *__restrict__ xnorm,
                                unsigned *__restrict__ ymax_bits) {
@@ -906,8 +911,9 @@ __global__ void tc_prep_kernel(const float *__restrict__ X, int64_t n, int d, in
     const int lane = threadIdx.x & 31;
     if (row < n) {
         const int kh = (x3 ? 2 : 1) * d_pad;
+        const int64_t src = scrambled ? tile::scrambled_row(int(row), int(n)) : row;
         __nv_bfloat16 *h = H + row * kh;
-        const float *x = X + row * d;
+        const float *x = X + src * d;
         float acc = 0.0f;
         // four coordinates per lane per step (16-byte rows), else one
         const bool v4 = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
@@ -944,7 +950,7 @@ __global__ void tc_prep_kernel(const float *__restrict__ X, int64_t n, int d, in
         for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) {
             ny[row] = acc;
-            xnorm[row] = acc;
+            xnorm[src] = acc;
             atomicMax(&bmax, __float_as_uint(sqrtf(acc)));   // one global atomic per block
         }
     }
@@ -957,7 +963,7 @@ __global__ void tc_prep_kernel(const float *__restrict__ X, int64_t n, int d, in
 // largest finite E4M3), q = e4m3(x' / s) rounded to nearest (the division by
 // a power of two is exact), FP32 norm ||x'||^2 as for the BF16 operands.
 // Rows of d_pad bytes, zero beyond d.
-__global__ void tc_prep_f8_kernel(const float *__restrict__ X, int64_t n, int d, int d_pad,
+__global__ void tc_prep_f8_kernel(const float *__restrict__ X, int64_t n, int d, int d_pad, int scrambled,
                                   const float *__restrict__ mean, uint8_t *__restrict__ Q,
                                   float *__restrict__ rscale, float *__restrict__ ny,
                                   float *__restrict__ xnorm, unsigned *__restrict__ ymax_bits) {
@@ -967,7 +973,8 @@ __global__ void tc_prep_f8_kernel(const float *__restrict__ X, int64_t n, int d,
     const int64_t row = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (row < n) {
-        const float *x = X + row * d;
+        const int64_t src = scrambled ? tile::scrambled_row(int(row), int(n)) : row;
+        const float *x = X + src * d;
         float amax = 0.0f, acc = 0.0f;
         for (int t = lane; t < d; t += 32) {
             const float xc = __fsub_rn(__ldg(x + t), __ldg(mean + t));
@@ -997,7 +1004,7 @@ __global__ void tc_prep_f8_kernel(const float *__restrict__ X, int64_t n, int d,
         if (lane == 0) {
             rscale[row] = sc;
             ny[row] = acc;
-            xnorm[row] = acc;
+            xnorm[src] = acc;
             atomicMax(&bmax, __float_as_uint(sqrtf(acc)));
         }
     }
@@ -1013,6 +1020,13 @@ __global__ void fill_value_kernel(float *p, int64_t from, int64_t to, float v) {
 __global__ void fill_inf_kernel(float *p, int64_t from, int64_t to) {
     int64_t i = from + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i < to) p[i] = __int_as_float(0x7f800000);
+}
+
+// components over the (scrambled) padded rows, -1 beyond n
+__global__ void pad_components_kernel(const int32_t *__restrict__ comp, int64_t n, int64_t npad,
+                                      int32_t *__restrict__ cpad) {
+    const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (p < npad) cpad[p] = p < n ? comp[tile::scrambled_row(int(p), int(n))] : -1;
 }
 
 // Start threshold of the pruned tiles' lists: every key y within tau_r of
@@ -1110,7 +1124,7 @@ __device__ __forceinline__ bool certified(float kw, float skip, float sp, float 
 
 // One warp per row: canonical distances of its cnt candidates, bitonic sort
 // of (w, id), top k, certificate (sp: every key left out scored above it).
-// Row i's point is xi; candidate ids index rows of X (row stride ld, chain length dc >= d: columns beyond d are zero
+// Row i's point is xi; row_of(candidate id) is a row of X (row stride ld, chain length dc >= d: columns beyond d are zero
 // and leave the canonical distance unchanged). d is the true dimension used in
 // the error bounds. Returns whether the row was certified (then the k
 // results are written).
@@ -1123,12 +1137,12 @@ __device__ __forceinline__ bool certified(float kw, float skip, float sp, float 
 // per lane at d = 128) at 68 % of peak. With about k + 3 candidates instead of
 // 4 R - 1, half batches, and the certificate's FP64 out of the common way: 1M
 // rows at k = 32 3.45 -> 2.59 ms, 256 clouds (2.6M rows, k = 16) 8.4 -> 6.6 ms.
-template <int XR, int H, class Eps64>
+template <int XR, int H, class Eps64, class RowOf>
 __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, int dc, int d,
                                            const float *__restrict__ xi, int k,
                                            const int32_t *__restrict__ cand_row, int cnt, float sp,
                                            float skip, float xn2f, float ymf,
-                                           const CertConst &cc, Eps64 eps64, int lane,
+                                           const CertConst &cc, Eps64 eps64, RowOf row_of, int lane,
                                            int32_t *__restrict__ nbr_row,
                                            float *__restrict__ dist_row,
                                            const int32_t *__restrict__ idmap = nullptr,
@@ -1140,7 +1154,7 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
     for (int h = 0; h < H; ++h) {
         key[h] = KEY_NONE;
         const int c = h * 32 + lane;
-        jc[h] = c < kp ? cand_row[c] : -1;
+        jc[h] = c < kp ? row_of(cand_row[c]) : -1;
     }
     if constexpr (XR > 0) {
         // batches of NB candidates: lane l's partial of candidate c in
@@ -1265,20 +1279,21 @@ __device__ __forceinline__ bool rerank_row(const float *__restrict__ X, int ld, 
     return cert;
 }
 
+// Position r of an unpruned pass (rows as they are, or scrambled).
 template <int XR, int H>
-__global__ void rerank_kernel(const float *__restrict__ X, int64_t n, int d, int k,
+__global__ void rerank_kernel(const float *__restrict__ X, int64_t n, int d, int k, int scrambled,
                               const int32_t *__restrict__ cand, const int32_t *__restrict__ ccnt,
-                              const float *__restrict__ splus, const float *__restrict__ skip,
-                              const float *__restrict__ xnorm2, const unsigned *__restrict__ ymax_bits,
+                              const float *__restrict__ splus, const float *__restrict__ xnorm2, const unsigned *__restrict__ ymax_bits,
                               CertConst cc, int32_t *__restrict__ nbr, float *__restrict__ dist,
                               int32_t *__restrict__ fail_rows, int32_t *__restrict__ fail_count) {
-    int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
-    if (i >= n) return;
-    const float sk = skip ? skip[i] : __int_as_float(0x7f800000);
-    bool cert = rerank_row<XR, H>(X, d, d, d, X + i * d, k, cand + i * (32 * H), ccnt[i], splus[i], sk,
-                                    xnorm2[i], __uint_as_float(*ymax_bits), cc, [&] { return cc.eps_dot; }, lane,
-                                    nbr + i * k, dist + i * k);
+    if (r >= n) return;
+    auto row_of = [&](int p) { return scrambled ? tile::scrambled_row(p, int(n)) : p; };
+    const int64_t i = row_of(int(r));
+    bool cert = rerank_row<XR, H>(X, d, d, d, X + i * d, k, cand + r * (32 * H), ccnt[r], splus[r],
+                                    __int_as_float(0x7f800000), xnorm2[i], __uint_as_float(*ymax_bits),
+                                    cc, [&] { return cc.eps_dot; }, row_of, lane, nbr + i * k, dist + i * k);
     if (!cert && lane == 0) fail_rows[atomicAdd(fail_count, 1)] = int32_t(i);
 }
 
@@ -1307,8 +1322,9 @@ rerank_sorted_kernel(const float *__restrict__ Xs, int64_t n, int d, int k,
     uint64_t kth;
     const bool cert = rerank_row<XR, H>(Xs, d, d, d, Xs + r * d, k, cand + r * (32 * H), ccnt[r],
                                           splus[r], skipQ[r / BM], xnorm2[i],
-                                          __uint_as_float(*ymax_bits), cc, [&] { return cc.eps_dot; }, lane,
-                                          nbr + i * k, dist + i * k, perm, &kth);
+                                          __uint_as_float(*ymax_bits), cc, [&] { return cc.eps_dot; },
+                                          [](int p) { return p; }, lane, nbr + i * k, dist + i * k,
+                                          perm, &kth);
     if (!cert && lane == 0) {
         const int s = atomicAdd(fail_count, 1);
         fail_rows[s] = int32_t(r);   // the position in the cell order
@@ -1356,8 +1372,8 @@ rerank_batched_kernel(const float *__restrict__ Xc, int ld, int64_t N,
     bool cert = rerank_row<XR, H>(Xc, ld, dc, c.d, Xc + v * ld, k, cand + v * (32 * H), ccnt[v], splus[v],
                                   __int_as_float(0x7f800000),
                                   xnorm2[v], __uint_as_float(ymax_bits[b]), cc,
-                                  [&] { return tc_eps_dot(c.d_pad, x3); }, lane, nbr + pv * k,
-                                  dist + pv * k, perm);
+                                  [&] { return tc_eps_dot(c.d_pad, x3); },
+                                  [](int p) { return p; }, lane, nbr + pv * k, dist + pv * k, perm);
     if (!cert && lane == 0) fail_rows[atomicAdd(fail_count, 1)] = int32_t(pv);
 }
 
@@ -1646,26 +1662,27 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         cudaMemsetAsync(fail_count, 0, 4, ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
     const int64_t npad = p.nk_tiles * BN;
+    bool use_prune = prune && !colcomp && prune_supported(n, d, k, vec4);
+    const int scrambled = !use_prune;   // the pruning has an order of its own
     if (f8) {
         FAMST_LAUNCH(ex, tc_prep_f8_kernel, unsigned((n * 32 + 255) / 256), 256, 0, X, n, d,
-                     p.d_pad, mean, Q, rscale, ny, xn2, ymax);
+                     p.d_pad, scrambled, mean, Q, rscale, ny, xn2, ymax);
         if (npad > n)
             FAMST_LAUNCH(ex, fill_value_kernel, unsigned((npad - n + 255) / 256), 256, 0, rscale,
                          n, npad, 1.0f);
     } else {
         FAMST_LAUNCH(ex, tc_prep_kernel, unsigned((n * 32 + 255) / 256), 256, 0, X, n, d, p.d_pad,
-                     int(x3), mean, H, ny, xn2, ymax);
+                     int(x3), scrambled, mean, H, ny, xn2, ymax);
     }
     if (npad > n)
         FAMST_LAUNCH(ex, fill_inf_kernel, unsigned((npad - n + 255) / 256), 256, 0, ny, n, npad);
-    bool use_prune = prune && !colcomp && prune_supported(n, d, k, vec4);
     const size_t before_prune = ar.off;
     // persistent launches: one CTA per SM takes the query tiles round-robin
     const unsigned pgrid = unsigned(std::min<int64_t>(p.nq_tiles, ex.num_sms));
     PruneOut P;
     if (use_prune) {
         // pivot cells: top-1 pivot of every point on the tensor tiles (BF16),
-        // evenly spaced pivots plus two coverage passes
+        // one pivot of every n / K rows plus two coverage passes
         const int K0 = prune_pivots(n), M = prune_extra(n), Kmax = prune_pivots_max(n);
         const int Kpadmax = (Kmax + BN - 1) / BN * BN;
         int32_t *piv = ar.take<int32_t>(size_t(Kmax));
@@ -1768,10 +1785,9 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     int32_t *cpad = nullptr;   // components over the padded rows (-1 beyond n)
     if (colcomp) {
         cpad = ar.take<int32_t>(size_t(npad));
-        if (cudaMemsetAsync(cpad, 0xff, size_t(npad) * 4, ex.stream) != cudaSuccess ||
-            cudaMemcpyAsync(cpad, colcomp, size_t(n) * 4, cudaMemcpyDeviceToDevice, ex.stream) !=
-                cudaSuccess)
-            return FAMST_ERR_CUDA;
+        if (!cpad) return FAMST_ERR_OOM;
+        FAMST_LAUNCH(ex, pad_components_kernel, unsigned((npad + 255) / 256), 256, 0, colcomp, n,
+                     npad, cpad);
     }
     // certificate constants (also the pruned lists' start thresholds)
     const double kprod = double(x3 ? 3 * p.d_pad : p.d_pad);
@@ -1850,8 +1866,8 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
                          cand, ccnt, splus, P.skipQ, P.perm, xn2, ymax, cc, nbr, dist,           \
                          fail_rows, fail_kth, fail_count);                                       \
         else                                                                                     \
-            FAMST_LAUNCH(ex, (rerank_kernel<XRV, HV>), rgrid, 256, 0, X, n, d, k, cand, ccnt,    \
-                         splus, nullptr, xn2, ymax, cc, nbr, dist, fail_rows, fail_count);       \
+            FAMST_LAUNCH(ex, (rerank_kernel<XRV, HV>), rgrid, 256, 0, X, n, d, k, scrambled,     \
+                         cand, ccnt, splus, xn2, ymax, cc, nbr, dist, fail_rows, fail_count);    \
     } while (0)
 #define RERANK(XRV)                                                                              \
     do {                                                                                         \

@@ -2,7 +2,7 @@
 // tile, key tile) pair; on data with structure most pairs cannot hold a
 // neighbour, and the triangle inequality proves it cheaply:
 //
-//   1. Locality partition. Pivots: evenly spaced rows, then two coverage
+//   1. Locality partition. Pivots: a row of every n / K, then two coverage
 //      passes that add pivots among the points far from every pivot (a
 //      cluster without a pivot would otherwise scatter into foreign cells).
 //      Every point joins the cell of its nearest pivot (the tensor-core
@@ -38,6 +38,7 @@
 #include <vector>
 
 #include "famst_internal.cuh"
+#include "tile_rows.cuh"
 
 namespace famst {
 namespace {
@@ -55,8 +56,14 @@ __device__ __forceinline__ float sq_lo(float p, float rho) {
     return fmaxf(__fsub_rd(__fmul_rd(p, 1.0f - rho), 1e-30f), 0.0f);
 }
 
-// pivot c = rows[c] (null: row c n / K): its operand row and norm; nyp
-// padded with +inf up to Kpad
+// pivot c = rows[c] (null: a row drawn from c n / K .. (c + 1) n / K - 1): its
+// operand row and norm; nyp padded with +inf up to Kpad. (Rows exactly n / K
+// apart share their phase when the index has a period: the first column of a
+// pixel grid 64 wide, one label of i mod 64. Their cells are then strips or
+// mixtures with that period inside: 27 to 34 % of the grid's rows lost their
+// certificate at k = 32, and mixed labels were listed against most tiles. Exact
+// steps / drawn rows, k = 32: a grid 256 wide, 65,536 x 4 11.3 / 2.25 ms; labels
+// i mod 64, 65,536 x 64 28.1 / 2.9; a random walk 100,000 x 64 1.97 / 1.96.)
 __global__ void pivots_kernel(const __nv_bfloat16 *__restrict__ H, int kh,
                               const float *__restrict__ ny, int64_t n, int K, int Kpad,
                               const int32_t *__restrict__ rows, int32_t *__restrict__ piv,
@@ -68,7 +75,8 @@ __global__ void pivots_kernel(const __nv_bfloat16 *__restrict__ H, int kh,
         if (lane == 0) nyp[c] = __int_as_float(0x7f800000);
         return;
     }
-    const int64_t row = rows ? int64_t(rows[c]) : c * n / K;
+    const int64_t lo = c * n / K, len = (c + 1) * n / K - lo;
+    const int64_t row = rows ? int64_t(rows[c]) : lo + tile::scrambled_row(0, int(len), uint32_t(c));
     if (lane == 0) {
         piv[c] = int32_t(row);
         nyp[c] = ny[row];

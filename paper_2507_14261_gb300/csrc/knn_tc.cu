@@ -258,21 +258,6 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     int *slot_sh = reinterpret_cast<int *>(tmem_slot + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // row `row` of this CTA's items from `item` on, when their tiles were given up
-    auto give_up = [&](int item, int row) {
-        for (; item < nitems; item += gridDim.x) {
-            const Item I = item_of(item);
-            if (I.q0 + row >= I.row_end) continue;
-            const tile::RowSlot at = tile::row_slot(I.q0, row, I.shift, I.part);
-            if constexpr (TOP1) {   // any pivot
-                args.cand[at.at] = 0;
-                args.splus[at.at] = 0.0f;
-            } else {
-                tile::give_up_row(at, args.ccnt, args.splus, args.side_cnt, args.side_splus);
-            }
-        }
-    };
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < args.stages; ++s) {
             mbar_init(&full[s], 1);
@@ -300,10 +285,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
     if constexpr (!TOP1) {
         __syncthreads();
-        if (*slot_sh < 0) {
-            if (threadIdx.x < BM) give_up(blockIdx.x, threadIdx.x);
-            return;
-        }
+        if (*slot_sh < 0) return;
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
@@ -627,7 +609,6 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         // the logs are complete; a failure anywhere stops every warp here
         const bool failed = epilogue_bar_any(32 * EPI, !ok);
-        if (failed && grp == 0) give_up(item, row);
         if constexpr (TOP1) {
             if (!failed && grp == 0 && mine) {
                 float s = t_sh[row];
@@ -778,6 +759,23 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
 }
 
+// A row's candidates and bound as the kernels behind the tiles take them. A CTA
+// that gives up (a bounded wait ran out, or no scratch area was free) leaves its
+// rows unset and the status word says so: then no row has candidates, or a bound
+// that certifies. (Written by the tile kernel itself, 20 lines behind its loops,
+// this cost registers in them: 16 to 40 bytes of spills, 1.6 % of 256 clouds'
+// build.) The pivots of such a top-1 pass may be anything; their reader takes
+// what is no pivot as pivot 0.
+__device__ __forceinline__ void row_result(const int *__restrict__ status,
+                                           const int32_t *__restrict__ ccnt,
+                                           const float *__restrict__ splus, int64_t r, int &cnt,
+                                           float &sp) {
+    cnt = ccnt[r];
+    sp = splus[r];
+    if (__ldg(status) & STATUS_LOOP_LIMIT)
+        tile::give_up_row(tile::RowSlot{false, 0}, &cnt, &sp, nullptr, nullptr);
+}
+
 // Rows of split query tiles (a warp per row, blockIdx.y = 16 rows of split
 // tile blockIdx.x): s+ = the smallest of the parts' s+ (every key of the
 // others at or below it is among their candidates), lowered like a whole
@@ -788,8 +786,10 @@ split_merge_kernel(const int32_t *__restrict__ splitq, const int32_t *__restrict
                    const int32_t *__restrict__ side_cnt, const float *__restrict__ side_splus,
                    int64_t n, Select sel, const float *__restrict__ ny,
                    const unsigned *__restrict__ ymax, int32_t *__restrict__ cand,
-                   int32_t *__restrict__ ccnt, float *__restrict__ splus) {
+                   int32_t *__restrict__ ccnt, float *__restrict__ splus,
+                   const int *__restrict__ status) {
     if (int(blockIdx.x) >= __ldg(nsplit)) return;
+    if (__ldg(status) & STATUS_LOOP_LIMIT) return;   // (row_result)
     const int q = splitq[3 * blockIdx.x], slot0 = splitq[3 * blockIdx.x + 1];
     const int P = splitq[3 * blockIdx.x + 2];
     const int row = int(blockIdx.y) * 16 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -1284,14 +1284,18 @@ template <int XR, int H>
 __global__ void rerank_kernel(const float *__restrict__ X, int64_t n, int d, int k, int scrambled,
                               const int32_t *__restrict__ cand, const int32_t *__restrict__ ccnt,
                               const float *__restrict__ splus, const float *__restrict__ xnorm2, const unsigned *__restrict__ ymax_bits,
-                              CertConst cc, int32_t *__restrict__ nbr, float *__restrict__ dist,
+                              CertConst cc, const int *__restrict__ status,
+                              int32_t *__restrict__ nbr, float *__restrict__ dist,
                               int32_t *__restrict__ fail_rows, int32_t *__restrict__ fail_count) {
     const int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (r >= n) return;
     auto row_of = [&](int p) { return scrambled ? tile::scrambled_row(p, int(n)) : p; };
     const int64_t i = row_of(int(r));
-    bool cert = rerank_row<XR, H>(X, d, d, d, X + i * d, k, cand + r * (32 * H), ccnt[r], splus[r],
+    int cnt;
+    float sp;
+    row_result(status, ccnt, splus, r, cnt, sp);
+    bool cert = rerank_row<XR, H>(X, d, d, d, X + i * d, k, cand + r * (32 * H), cnt, sp,
                                     __int_as_float(0x7f800000), xnorm2[i], __uint_as_float(*ymax_bits),
                                     cc, [&] { return cc.eps_dot; }, row_of, lane, nbr + i * k, dist + i * k);
     if (!cert && lane == 0) fail_rows[atomicAdd(fail_count, 1)] = int32_t(i);
@@ -1311,6 +1315,7 @@ rerank_sorted_kernel(const float *__restrict__ Xs, int64_t n, int d, int k,
                                      const int32_t *__restrict__ perm,
                                      const float *__restrict__ xnorm2,
                                      const unsigned *__restrict__ ymax_bits, CertConst cc,
+                                     const int *__restrict__ status,
                                      int32_t *__restrict__ nbr, float *__restrict__ dist,
                                      int32_t *__restrict__ fail_rows,
                                      uint64_t *__restrict__ fail_kth,
@@ -1320,8 +1325,11 @@ rerank_sorted_kernel(const float *__restrict__ Xs, int64_t n, int d, int k,
     if (r >= n) return;
     const int64_t i = perm[r];
     uint64_t kth;
-    const bool cert = rerank_row<XR, H>(Xs, d, d, d, Xs + r * d, k, cand + r * (32 * H), ccnt[r],
-                                          splus[r], skipQ[r / BM], xnorm2[i],
+    int cnt;
+    float sp;
+    row_result(status, ccnt, splus, r, cnt, sp);
+    const bool cert = rerank_row<XR, H>(Xs, d, d, d, Xs + r * d, k, cand + r * (32 * H), cnt, sp,
+                                          skipQ[r / BM], xnorm2[i],
                                           __uint_as_float(*ymax_bits), cc, [&] { return cc.eps_dot; },
                                           [](int p) { return p; }, lane, nbr + i * k, dist + i * k,
                                           perm, &kth);
@@ -1357,6 +1365,7 @@ rerank_batched_kernel(const float *__restrict__ Xc, int ld, int64_t N,
                                       const float *__restrict__ splus,
                                       const float *__restrict__ xnorm2,
                                       const unsigned *__restrict__ ymax_bits, CertConst cc,
+                                      const int *__restrict__ status,
                                       const int32_t *__restrict__ perm,
                                       int32_t *__restrict__ nbr, float *__restrict__ dist,
                                       int32_t *__restrict__ fail_rows,
@@ -1369,7 +1378,10 @@ rerank_batched_kernel(const float *__restrict__ Xc, int ld, int64_t N,
     if (!c.use_tc) return;
     const int dc = (c.d + 3) & ~3;
     const int64_t pv = perm ? int64_t(perm[v]) : v;
-    bool cert = rerank_row<XR, H>(Xc, ld, dc, c.d, Xc + v * ld, k, cand + v * (32 * H), ccnt[v], splus[v],
+    int cnt;
+    float sp;
+    row_result(status, ccnt, splus, v, cnt, sp);
+    bool cert = rerank_row<XR, H>(Xc, ld, dc, c.d, Xc + v * ld, k, cand + v * (32 * H), cnt, sp,
                                   __int_as_float(0x7f800000),
                                   xnorm2[v], __uint_as_float(ymax_bits[b]), cc,
                                   [&] { return tc_eps_dot(c.d_pad, x3); },
@@ -1855,7 +1867,7 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     if (use_prune)   // rows of split lists: combine their parts
         FAMST_LAUNCH(ex, split_merge_kernel, dim3(PRUNE_SPLIT_TILES, BM / 16), 512, 0, P.splitq,
                      P.nsplit, side_j, side_s, side_cnt, side_sp, n, a.sel, a.ny, ymax, cand, ccnt,
-                     splus);
+                     splus, ex.dstatus);
     timer_mark(ex, TIMER_TILES, true);
     if (cudaPeekAtLastError() != cudaSuccess) return FAMST_ERR_CUDA;
     const unsigned rgrid = unsigned((n * 32 + 255) / 256);
@@ -1863,11 +1875,12 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     do {                                                                                         \
         if (use_prune)                                                                           \
             FAMST_LAUNCH(ex, (rerank_sorted_kernel<XRV, HV>), rgrid, 256, 0, P.Xs, n, d, k,      \
-                         cand, ccnt, splus, P.skipQ, P.perm, xn2, ymax, cc, nbr, dist,           \
+                         cand, ccnt, splus, P.skipQ, P.perm, xn2, ymax, cc, ex.dstatus, nbr, dist, \
                          fail_rows, fail_kth, fail_count);                                       \
         else                                                                                     \
             FAMST_LAUNCH(ex, (rerank_kernel<XRV, HV>), rgrid, 256, 0, X, n, d, k, scrambled,     \
-                         cand, ccnt, splus, xn2, ymax, cc, nbr, dist, fail_rows, fail_count);    \
+                         cand, ccnt, splus, xn2, ymax, cc, ex.dstatus, nbr, dist, fail_rows,     \
+                         fail_count);                                                            \
     } while (0)
 #define RERANK(XRV)                                                                              \
     do {                                                                                         \
@@ -1984,7 +1997,7 @@ famst_status knn_tc_batched(const Exec &ex, const float *Xc, int D, int64_t N, i
     const CertConst cc = cert_const(tc_eps_dot(D, x3), D);
 #define RRB2(XRV, HV)                                                                            \
     FAMST_LAUNCH(ex, (rerank_batched_kernel<XRV, HV>), rgrid, 256, 0, Xc, D, N, voff, B, cl,     \
-                 int(x3), k, cand, ccnt, splus, xn2, ymax, cc, perm, nbr, dist, fail_rows,       \
+                 int(x3), k, cand, ccnt, splus, xn2, ymax, cc, ex.dstatus, perm, nbr, dist, fail_rows, \
                  fail_count)
 #define RRB(XRV)                                                                                 \
     do {                                                                                         \

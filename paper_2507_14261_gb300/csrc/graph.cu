@@ -12,6 +12,8 @@
 // the discovery order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "famst_internal.cuh"
 
 namespace famst {
@@ -186,22 +188,32 @@ __device__ __forceinline__ int uf_find(int32_t *parent_, int v, int limit, int *
 }
 
 // Hooks. Hooking every edge by itself makes the threads in flight fight for
-// the few roots their edges share (50k points of two moons: 1.2 ms, the
+// the few roots their edges share (50k points of two moons: 0.5 ms, the
 // hubs' roots changing hands one compare-and-swap at a time). So the forest
-// is first grown by rounds without retries: every vertex points at its
-// smallest neighbour; then, twice, every edge between two roots lowers the
-// larger root's parent by atomicMin, after a plain read that filters most of
-// them. A round may replace a link by another; uf_hook_kernel then goes over
-// all edges, which mostly find equal roots in one read of each end, and
-// joins what is still apart.
-constexpr int UF_ROUNDS = 2;
+// is first grown by rounds without retries, over a few of each vertex's edges:
+// every vertex points at the smallest of its first UF_MIN neighbours; then,
+// twice, every edge of the next few between two roots lowers the larger
+// root's parent by atomicMin, after a plain read that filters most of them. A
+// round may replace a link by another; uf_hook_kernel then goes over all
+// edges, which mostly find equal roots in one read of each end, and joins
+// what is still apart.
+//
+// Bound: the hooks' gathers of both ends' roots (140 us for the 32M edges of 1M
+// points), and latency. famst_components, us, no rounds / two rounds over all
+// edges / these: 1M sphere points in 1000 clusters, k 32: 471 / 830 / 471; 200k
+// in 500: 210 / 252 / 170; 1M in 3, k 8: 690 / 410 / 253; moons 50k, k 16: 530 /
+// 300 / 198, 400k: 700 / 800 / 231; 65,537 overlapping, k 32: 250 / 200 / 143.
+// (Rounds over 2, 6 or 8 neighbours: 464, 490 and 507 us at 1M; 220, 121 and 127
+// on the 50k moons.)
+constexpr int UF_MIN = 4, UF_ROUNDS = 2;
+constexpr int UF_LOWER[UF_ROUNDS] = {4, 2};
 
-__global__ void uf_min_kernel(const int32_t *__restrict__ nbr, int64_t n, int k,
+__global__ void uf_min_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, int kmin,
                               int32_t *__restrict__ parent) {
     const int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (v >= n) return;
     int m = int(v);
-    for (int j = 0; j < k; ++j) {
+    for (int j = 0; j < kmin; ++j) {
         const int b = __ldg(nbr + v * k + j);
         m = b >= 0 && b < m ? b : m;
     }
@@ -212,16 +224,17 @@ __global__ void uf_min_kernel(const int32_t *__restrict__ nbr, int64_t n, int k,
 // v = (e / k) * 0x9E3779B1 mod 2^m (odd multiplier: a bijection of
 // [0, 2^m), 2^m >= n; v >= n idle). When ids are contiguous in space (clouds
 // laid out one after another, sorted inputs), threads in flight together
-// would otherwise all hook onto the same few roots.
-__global__ void uf_lower_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, uint32_t vmask,
-                                int32_t *parent_) {
+// would otherwise all hook onto the same few roots. (uf_lower_kernel: the same
+// over the neighbours j0 .. j0 + kl - 1.)
+__global__ void uf_lower_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, int j0, int kl,
+                                uint32_t vmask, int32_t *parent_) {
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int64_t vl = e / k;
+    const int64_t vl = e / kl;
     if (vl > int64_t(vmask)) return;
     const uint32_t v = (uint32_t(vl) * 0x9E3779B1u) & vmask;
     if (int64_t(v) >= n) return;
     volatile int32_t *parent = parent_;
-    const int ra = parent[v], rb = parent[nbr[int64_t(v) * k + (e - vl * k)]];
+    const int ra = parent[v], rb = parent[nbr[int64_t(v) * k + j0 + (e - vl * kl)]];
     if (ra == rb) return;
     const int hi = ra > rb ? ra : rb, lo = ra > rb ? rb : ra;
     if (parent[hi] > lo) atomicMin(parent_ + hi, lo);
@@ -251,10 +264,24 @@ __global__ void uf_hook_kernel(const int32_t *__restrict__ nbr, int64_t n, int k
     set_status(dstatus, STATUS_LOOP_LIMIT);
 }
 
-// every vertex points at its root (no hooks run beside this kernel)
-__global__ void uf_compress_kernel(int32_t *parent, int64_t n, int limit, int *dstatus) {
+// Every vertex points at its root (no hooks run beside this kernel). A thread
+// writes its own vertex's parent only, and reads what the others have reached:
+// chains shorten by doubling. (uf_find's walk, which rewrites the nodes it
+// passes, went along the chains that the lowering rounds leave node by node:
+// 490 us instead of 15 on 400k points of two moons.)
+__global__ void uf_compress_kernel(int32_t *parent_, int64_t n, int limit, int *dstatus) {
     const int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (v < n) *reinterpret_cast<volatile int32_t *>(parent + v) = uf_find(parent, int(v), limit, dstatus);
+    if (v >= n) return;
+    volatile int32_t *parent = parent_;
+    int p = parent[v], steps = 0;
+    for (int g = parent[p]; g != p; g = parent[p]) {
+        parent[v] = g;
+        p = g;
+        if (steps++ >= limit) {
+            set_status(dstatus, STATUS_LOOP_LIMIT);
+            return;
+        }
+    }
 }
 
 // Roots go to a separate array: a concurrent find may still rewrite
@@ -383,15 +410,20 @@ famst_status components_uf(const Exec &ex, Arena &ar, const int32_t *nbr, int64_
     const int th = 256;
     const int lim = ex.loop_limit > 0 ? ex.loop_limit : UF_LIMIT;
     int64_t nk = n * k;
-    FAMST_LAUNCH(ex, uf_min_kernel, blocks_for(n, th), th, 0, nbr, n, nk > 0 ? k : 0, parent);
+    FAMST_LAUNCH(ex, uf_min_kernel, blocks_for(n, th), th, 0, nbr, n, k,
+                 nk > 0 ? std::min(k, UF_MIN) : 0, parent);
     if (nk > 0) {
         uint32_t vmask = 1;
         while (int64_t(vmask) + 1 < n) vmask = (vmask << 1) | 1u;
         const unsigned hgrid = blocks_for((int64_t(vmask) + 1) * k, th);
+        int j0 = UF_MIN;
         for (int r = 0; r < UF_ROUNDS; ++r) {
+            const int kl = std::min(k, UF_LOWER[r]);
             FAMST_LAUNCH(ex, uf_compress_kernel, blocks_for(n, th), th, 0, parent, n, lim,
                          ex.dstatus);
-            FAMST_LAUNCH(ex, uf_lower_kernel, hgrid, th, 0, nbr, n, k, vmask, parent);
+            FAMST_LAUNCH(ex, uf_lower_kernel, blocks_for((int64_t(vmask) + 1) * kl, th), th, 0, nbr,
+                         n, k, std::min(j0, k - kl), kl, vmask, parent);
+            j0 += kl;
         }
         FAMST_LAUNCH(ex, uf_compress_kernel, blocks_for(n, th), th, 0, parent, n, lim, ex.dstatus);
         FAMST_LAUNCH(ex, uf_hook_kernel, hgrid, th, 0, nbr, n, k, vmask, parent, lim, ex.dstatus);

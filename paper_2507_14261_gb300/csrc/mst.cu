@@ -20,6 +20,8 @@
 // (round, component id), which is deterministic.
 #include <cuda_runtime.h>
 
+#include <cstring>
+
 #include "famst_internal.cuh"
 
 namespace famst {
@@ -371,23 +373,43 @@ __global__ void weight_final_kernel(const double *__restrict__ part, int64_t nb,
 // so the edge's length comes out of the loads the gradient needs anyway; no
 // pass over the edges computes or stores lengths, and the finiteness check
 // rides along. The incidences are placed by counting and ranked inside their
-// vertex (ascending edge index) instead of radix sorted; a vertex beyond
-// INC_RANK_MAX edges sends the call to the radix sort, whose cost does not
-// depend on the degrees.
+// vertex (ascending edge index) instead of radix sorted, where that is cheap.
+//
+// A rank reads its vertex's whole list: the reads of all ranks are the sum of the
+// squared degrees, and the longest list is one thread's chain. The radix sort's
+// cost does not depend on the degrees. Trees of hubs with h leaves each, whole
+// call, ranks / radix sort, us: 1M x 16 h = 4 313 / 452, 90 466 / 484, 128 527 /
+// 499, 500 1133 / 631, 2000 3577 / 1316; 100,000 x 64 h = 4 118 / 209, 256 306 /
+// 363, 500 494 / 507, 1000 575 / 520; 10,000 x 16 h = 500 267 / 313, 2000 840 / 833.
+constexpr int INC_RANK_MAX = 2048;   // about 20 us for a single such list
+inline bool rank_pays(int64_t m, uint64_t sum_sq, int64_t max_deg) {
+    return max_deg <= INC_RANK_MAX && sum_sq <= uint64_t(40000000 + 70 * m);
+}
 
-constexpr int INC_RANK_MAX = 2048;   // a rank reads its vertex's whole list (about 20 us here)
+// What incidence_count_kernel leaves behind the degrees.
+struct IncTotals {
+    unsigned long long sum_sq;   // of the degrees (those beyond INC_RANK_MAX count less)
+    int32_t max_deg;
+};
+inline int64_t totals_at(int64_t n) { return (n + 2) / 2 * 2; }   // 8-byte aligned, behind n + 1 degrees
+constexpr int64_t TOTALS_WORDS = 4;
 
-// Range check, degrees and each incidence's arrival number at its vertex;
-// maxdeg[0] = the largest degree.
+// Range check, degrees and each incidence's arrival number at its vertex; the
+// a-th arrival adds 2 a + 1 to the sum of squares.
 __global__ void incidence_count_kernel(const int32_t *__restrict__ tu,
                                        const int32_t *__restrict__ tv, int64_t m, int64_t n,
                                        int32_t *__restrict__ deg, int2 *__restrict__ slot,
-                                       int32_t *__restrict__ maxdeg, int *dstatus) {
+                                       IncTotals *__restrict__ totals, int *dstatus) {
     __shared__ int bmax;
-    if (threadIdx.x == 0) bmax = 0;
+    __shared__ unsigned bsum;   // 512 arrivals of at most 2^20
+    if (threadIdx.x == 0) {
+        bmax = 0;
+        bsum = 0;
+    }
     __syncthreads();
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     int mx = 0;
+    unsigned sum = 0;
     if (e < m) {
         const int u = tu[e], v = tv[e];
         if (u < 0 || v < 0 || int64_t(u) >= n || int64_t(v) >= n) {
@@ -396,12 +418,20 @@ __global__ void incidence_count_kernel(const int32_t *__restrict__ tu,
             const int su = atomicAdd(&deg[u], 1), sv = atomicAdd(&deg[v], 1);
             slot[e] = make_int2(su, sv);
             mx = (su > sv ? su : sv) + 1;
+            sum = min(2u * unsigned(su) + 1u, 1u << 20) + min(2u * unsigned(sv) + 1u, 1u << 20);
         }
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if ((threadIdx.x & 31) == 0) atomicMax(&bmax, mx);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&bmax, mx);
+        atomicAdd(&bsum, sum);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) atomicMax(maxdeg, bmax);
+    if (threadIdx.x == 0) {
+        atomicMax(&totals->max_deg, bmax);
+        atomicAdd(&totals->sum_sq, (unsigned long long)bsum);
+    }
 }
 
 __global__ void incidence_fill_kernel(const int32_t *__restrict__ tu,
@@ -433,7 +463,7 @@ __global__ void incidence_rank_kernel(const int32_t *__restrict__ tu,
     }
 }
 
-// The radix sort's input (a vertex of large degree) and its adj entries.
+// The radix sort's input (large degrees) and its adj entries.
 __global__ void incidence_kernel(const int32_t *__restrict__ tu, const int32_t *__restrict__ tv,
                                  int64_t m, uint32_t *__restrict__ keys,
                                  int32_t *__restrict__ vals) {
@@ -569,10 +599,18 @@ __global__ void __launch_bounds__(256) grad_rows_kernel(const float *__restrict_
             };
             if (j0 < j1) add(yc[0], y[0]);
             if (j0 + 1 < j1) add(yc[1], y[1]);
-            for (int j = j0 + 2; j < j1; ++j) {
-                const float *yr = X + int64_t(end_of(j)) * d;
-                row(yr, y[0]);
-                add(yr, y[0]);
+            // (the other edges two at a time, both rows in flight: a hub of 1000
+            // edges of 64 coordinates 0.4 -> 0.3 us an edge)
+#pragma unroll 1
+            for (int j = j0 + 2; j < j1; j += 2) {
+                const float *yr[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    yr[e] = X + int64_t(end_of(j + e < j1 ? j + e : j)) * d;
+                    row(yr[e], y[e]);
+                }
+                add(yr[0], y[0]);
+                if (j + 1 < j1) add(yr[1], y[1]);
             }
 #pragma unroll
             for (int q = 0; q < XR; ++q) {
@@ -833,38 +871,42 @@ famst_status tree_weight(const Exec &ex, Arena &ar, const float *X, int d, bool 
 
 size_t mst_backward_workspace(int64_t n, int64_t m) {
     return align256(size_t(m) * 8) + align256(size_t(2 * m) * 4) * 3 +
-           align256(size_t(n + 2) * 4) + align256(size_t(n + 1) * 4) +
+           align256(size_t(totals_at(n) + TOTALS_WORDS) * 4) + align256(size_t(n + 1) * 4) +
            radix_sort_workspace(2 * m) + scan_workspace(n + 1);
 }
 
-// pinned_host: two pinned host words. Ids are checked before they are used;
-// synchronises once (the status word and the largest degree).
+// pinned_host: four pinned host words (the totals, the status word). Ids are
+// checked before they are used; synchronises once.
 famst_status mst_backward(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
                           const int32_t *tu, const int32_t *tv, int64_t m, float gW, float *gX,
                           int32_t *pinned_host) {
     int2 *slot = ar.take<int2>(size_t(m > 0 ? m : 1));
     int32_t *inc = ar.take<int32_t>(size_t(m > 0 ? 2 * m : 1));
     int32_t *adj = ar.take<int32_t>(size_t(m > 0 ? 2 * m : 1));
-    int32_t *deg = ar.take<int32_t>(size_t(n + 2));   // [n + 1]: the largest degree
+    const int64_t tot = totals_at(n);
+    int32_t *deg = ar.take<int32_t>(size_t(tot + TOTALS_WORDS));
     int32_t *off = ar.take<int32_t>(size_t(n + 1));
     if (!slot || !inc || !adj || !deg || !off) return FAMST_ERR_OOM;
     const int th = 256;
-    if (cudaMemsetAsync(deg, 0, size_t(n + 2) * 4, ex.stream) != cudaSuccess)
+    IncTotals *totals = reinterpret_cast<IncTotals *>(deg + tot);
+    if (cudaMemsetAsync(deg, 0, size_t(tot + TOTALS_WORDS) * 4, ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
     if (m > 0)
         FAMST_LAUNCH(ex, incidence_count_kernel, blocks_for(m, th), th, 0, tu, tv, m, n, deg, slot,
-                     deg + n + 1, ex.dstatus);
+                     totals, ex.dstatus);
     famst_status st = exclusive_scan_i32(ex, ar, deg, off, n + 1, nullptr);
     if (st != FAMST_OK) return st;
     if (m > 0) {
-        if (cudaMemcpyAsync(pinned_host, deg + n + 1, 4, cudaMemcpyDeviceToHost, ex.stream) !=
+        IncTotals h;
+        if (cudaMemcpyAsync(pinned_host, totals, 12, cudaMemcpyDeviceToHost, ex.stream) !=
                 cudaSuccess ||
-            cudaMemcpyAsync(pinned_host + 1, ex.dstatus, 4, cudaMemcpyDeviceToHost, ex.stream) !=
+            cudaMemcpyAsync(pinned_host + 3, ex.dstatus, 4, cudaMemcpyDeviceToHost, ex.stream) !=
                 cudaSuccess ||
             cudaStreamSynchronize(ex.stream) != cudaSuccess)
             return FAMST_ERR_CUDA;
-        if (pinned_host[1] != 0) return FAMST_OK;   // an id out of range: the caller reads the status
-        if (pinned_host[0] <= INC_RANK_MAX) {
+        if (pinned_host[3] != 0) return FAMST_OK;   // an id out of range: the caller reads the status
+        std::memcpy(&h, pinned_host, 12);
+        if (rank_pays(m, h.sum_sq, h.max_deg)) {
             FAMST_LAUNCH(ex, incidence_fill_kernel, blocks_for(m, th), th, 0, tu, tv, m, off, slot,
                          inc);
             FAMST_LAUNCH(ex, incidence_rank_kernel, blocks_for(m, th), th, 0, tu, tv, m, off, inc,

@@ -403,7 +403,7 @@ size_t knn_stage_ws(famst_ctx *ctx, int64_t n, int32_t d, int32_t k, int32_t pre
                                 !f8 && ctx->prune != 0 && prune_supported(n, d, k, true), f8);
     const size_t plain = knn_fp32_workspace(n, d, k, n, ctx->num_sms);
     if (prec == FAMST_PREC_FP32 && ctx->prune && knn_fp32_prunes(n, d, k, true))
-        return std::max(plain, knn_tc_workspace(n, d, k, false, ctx->num_sms, true, false));
+        return std::max(plain, knn_tc_workspace(n, d, k, false, ctx->num_sms, true, false, true));
     return plain;
 }
 

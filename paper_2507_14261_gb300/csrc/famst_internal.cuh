@@ -544,8 +544,9 @@ famst_status knn_fp32_batched(const Exec &ex, const float *Xc, int ld, const lon
 // Exact kNN through tcgen05 BF16 (x3 = hi/lo split) distance tiles, FP32
 // re-rank, certificate, FP32 recomputation of uncertified rows.
 bool knn_tc_supported(int64_t n, int d, int k, bool x3, bool f8 = false);
+// (f32: of the pruned FP32 tiles, for which the tensor tiles only place the points)
 size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prune = false,
-                        bool f8 = false);
+                        bool f8 = false, bool f32 = false);
 // Exact kNN of the listed rows of a batch of clouds (warp per row, canonical
 // distances within the row's cloud); rows / count on the device. k <= 64.
 famst_status fallback_rows_batched(const Exec &ex, const float *Xc, int ld, const long long *voff,

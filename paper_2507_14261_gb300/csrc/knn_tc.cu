@@ -90,6 +90,13 @@ constexpr int LOG_CAP = 256;     // log entries per thread; compacted beyond LOG
 constexpr size_t LOG_SLOT = size_t(4) * BM * LOG_CAP;   // entries of one CTA's scratch area
 // scratch areas of a launch of nctas CTAs, of which one per SM is resident
 inline int log_slots(int64_t nctas, int num_sms) { return int(std::min<int64_t>(nctas, num_sms)); }
+// Most work items of a pass: the query tiles, with pruned lists' parts (each of
+// more than PRUNE_SPLIT_MIN / 2 key tiles, so that small clouds have none).
+inline int64_t max_items(int64_t nq_tiles, int64_t nk_tiles, bool prune) {
+    if (!prune) return nq_tiles;
+    const int64_t parts = (nk_tiles + PRUNE_SPLIT_MIN - 1) / PRUNE_SPLIT_MIN;
+    return std::min(nq_tiles + PRUNE_SPLIT_SLOTS, nq_tiles * std::max<int64_t>(1, parts));
+}
 constexpr int TC_THREADS = 64 + 32 * EPI;
 constexpr int VISITED_ROWS_SHARE = 32;   // uncertified rows redone one by one: up to n / this
 
@@ -1591,7 +1598,8 @@ bool knn_tc_supported(int64_t n, int d, int k, bool x3, bool f8) {
     return p.stages >= 2 && encode_fn() != nullptr;
 }
 
-size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prune, bool f8) {
+size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prune, bool f8,
+                        bool f32) {
     TcPlan p = tc_plan(n, d, k, x3 && !f8, f8);
     if (f8) prune = false;
     size_t b = 0;
@@ -1599,7 +1607,7 @@ size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prun
         const int64_t K = prune_pivots_max(n), Kpad = (K + BN - 1) / BN * BN;
         b += align256(size_t(K) * 4) + align256(size_t(K) * p.kh * 2) +
              align256(size_t(Kpad + BN) * 4) * 2 + align256(size_t(n) * 4) * 2;
-        b += prune_workspace(n, d, p.kh, p.cap, p.nq_tiles, p.nk_tiles);
+        b += prune_workspace(n, d, p.kh, f32 ? 0 : p.cap, p.nq_tiles, p.nk_tiles);
         b += align256(size_t(n) * 4) * 2 + align256(size_t(n) * 8) + 256;   // thr0, failed rows
         b += std::max(knn_fp32_pruned_workspace(n, k, p.nq_tiles),
                       visited_rows_workspace(n / VISITED_ROWS_SHARE));
@@ -1610,10 +1618,11 @@ size_t knn_tc_workspace(int64_t n, int d, int k, bool x3, int num_sms, bool prun
     b += align256(size_t(n) * 4);                          // xnorm2
     b += align256(size_t(d) * 4) + 256;                    // mean, ymax
     b += align256(size_t(4096) * d * 8);                   // column partials
-    b += align256(size_t(n) * p.cap * 4);                  // candidates
-    const int slots = log_slots(
-        p.nq_tiles + (prune_supported(n, d, k, true) ? PRUNE_SPLIT_SLOTS : 0), num_sms);
-    b += align256(size_t(slots) * LOG_SLOT * 8) + align256(size_t(slots) * 4);   // logs
+    if (!f32) {   // (else the tensor tiles only place the points in cells)
+        const int slots = log_slots(max_items(p.nq_tiles, p.nk_tiles, prune), num_sms);
+        b += align256(size_t(n) * p.cap * 4) +                                    // candidates
+             align256(size_t(slots) * LOG_SLOT * 8) + align256(size_t(slots) * 4);   // logs
+    }
     b += align256(size_t(n) * 4) * 4 + 256;                // their number, splus, pivots, fail rows
     b += knn_fp32_workspace(n, d, k, n, num_sms);          // fallback
     return b;
@@ -1656,8 +1665,8 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
     double *part = ar.take<double>(size_t(nb) * d);
     int32_t *cand = f32 ? nullptr : ar.take<int32_t>(size_t(n) * p.cap);   // (pruned: in cell order)
     int32_t *ccnt = ar.take<int32_t>(size_t(n));
-    const int slots = log_slots(
-        p.nq_tiles + (prune_supported(n, d, k, true) ? PRUNE_SPLIT_SLOTS : 0), ex.num_sms);
+    bool use_prune = prune && !colcomp && prune_supported(n, d, k, vec4);
+    const int slots = log_slots(max_items(p.nq_tiles, p.nk_tiles, use_prune), ex.num_sms);
     int2 *log = f32 ? nullptr : ar.take<int2>(size_t(slots) * LOG_SLOT);
     int *claim = f32 ? nullptr : ar.take<int>(size_t(slots));
     int32_t *top = ar.take<int32_t>(size_t(n));   // pivot of every point
@@ -1674,7 +1683,6 @@ famst_status knn_tc(const Exec &ex, Arena &ar, const float *X, int64_t n, int d,
         cudaMemsetAsync(fail_count, 0, 4, ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
     const int64_t npad = p.nk_tiles * BN;
-    bool use_prune = prune && !colcomp && prune_supported(n, d, k, vec4);
     const int scrambled = !use_prune;   // the pruning has an order of its own
     if (f8) {
         FAMST_LAUNCH(ex, tc_prep_f8_kernel, unsigned((n * 32 + 255) / 256), 256, 0, X, n, d,

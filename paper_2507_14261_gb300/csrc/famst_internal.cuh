@@ -722,13 +722,15 @@ famst_status refine_edges(const Exec &ex, Arena &ar, const float *X, int d, bool
                           int64_t m, int max_iters, int32_t *change_hist /*max_iters+1*/,
                           unsigned long long *evals = nullptr, bool check = true,
                           int *variant = nullptr);
-// Whether Alg. 4 of m edges takes the grouped sweeps. They cost some 0.55 ms of
-// launches and sorts and 0.22 ns per kNN entry (lists, BF16 rows) before the
-// first edge, and then about a fourth of the per-edge scans' 3 ps per edge, list
-// entry and coordinate. famst_refine, per edge / grouped: 756 edges of 15,436 x
-// 64 points, k 30: 0.27 / 0.80 ms; 49,500 of 30,000 x 128, k 16: 0.61 / 1.03;
-// 44,850 of 100,000 x 128, k 32: 0.98 / 1.73; 1.25M of 200,000 x 128, k 32:
-// 15.6 / 5.8.
+// Whether famst_refine takes the grouped route (lists of G with staged BF16 rows,
+// refine_build). Its lists and BF16 rows cost some 0.1 ms of launches and 0.22 ns
+// per kNN entry before the first edge; then the staged scans take about half, and
+// the sweeps beyond STAGED_ALL edges a fourth, of the per-edge scans' 3 ps per
+// edge, list entry and coordinate. Per edge / grouped, ms: 765 edges of 15,436 x 64
+// points, k 30: 0.20 / 0.31; 49,500 of 30,000 x 128, k 16: 0.64 / 0.55; 44,850 of
+// 100,000 x 128, k 32: 0.97 / 0.89; 79,600 of 200,000 x 128, k 32: 1.70 / 2.68;
+// 499,500 of 1M x 128, k 16: 8.0 / 7.5; 55,875 of 50,000 x 256, k 48: 2.40 / 1.58;
+// 99,500 of 30,000 x 200, k 60: 3.95 / 1.84; 1.25M of 200,000 x 128, k 32: 16.0 / 6.6.
 inline bool refine_grouped_pays(int64_t m, int64_t n, int k, int d) {
     return double(m) * k * d >= 2.3e8 + 92.0 * double(n) * k;
 }

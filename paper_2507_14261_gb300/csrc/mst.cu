@@ -600,17 +600,26 @@ __global__ void __launch_bounds__(256) grad_rows_kernel(const float *__restrict_
             if (j0 < j1) add(yc[0], y[0]);
             if (j0 + 1 < j1) add(yc[1], y[1]);
             // (the other edges two at a time, both rows in flight: a hub of 1000
-            // edges of 64 coordinates 0.4 -> 0.3 us an edge)
+            // edges of 64 coordinates 0.4 -> 0.3 us an edge; not with one coordinate
+            // per lane, where it takes 39 registers instead of 32)
+            if constexpr (XR > 1) {
 #pragma unroll 1
-            for (int j = j0 + 2; j < j1; j += 2) {
-                const float *yr[2];
+                for (int j = j0 + 2; j < j1; j += 2) {
+                    const float *yr[2];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    yr[e] = X + int64_t(end_of(j + e < j1 ? j + e : j)) * d;
-                    row(yr[e], y[e]);
+                    for (int e = 0; e < 2; ++e) {
+                        yr[e] = X + int64_t(end_of(j + e < j1 ? j + e : j)) * d;
+                        row(yr[e], y[e]);
+                    }
+                    add(yr[0], y[0]);
+                    if (j + 1 < j1) add(yr[1], y[1]);
                 }
-                add(yr[0], y[0]);
-                if (j + 1 < j1) add(yr[1], y[1]);
+            } else {
+                for (int j = j0 + 2; j < j1; ++j) {
+                    const float *yr = X + int64_t(end_of(j)) * d;
+                    row(yr, y[0]);
+                    add(yr, y[0]);
+                }
             }
 #pragma unroll
             for (int q = 0; q < XR; ++q) {

@@ -169,6 +169,7 @@ constexpr int NT_THREADS = 64 + 32 * NT_EPI;
 constexpr int NT_SAMPLES = 1024;
 constexpr int NT_SW = 4;       // warps of a component pair's sample
 constexpr unsigned long long NT_TOO_MANY = 1ull << 62;   // above any survivor buffer
+constexpr unsigned long long NT_GAVE_UP = 1ull << 63;    // a wait ran out: pairs are missing
 
 struct NtItem {
     int32_t row0, row_end;   // sorted rows row0 .. min(row0 + 127, row_end - 1), of component i
@@ -632,6 +633,8 @@ nearest_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
+    // (beside the count, which the host reads anyway)
+    if (threadIdx.x == 0 && *abort_flag) atomicMax(args.count, NT_GAVE_UP);
 }
 
 // Between the launch that only lowers the bounds and the search: the slots
@@ -1158,12 +1161,10 @@ famst_status nearest_tc(const Exec &ex, Arena &ar, const float *X, int d, const 
                      a);
     }
     unsigned long long got = 0;
-    int status = 0;
     if (cudaMemcpyAsync(&got, count, 8, cudaMemcpyDeviceToHost, ex.stream) != cudaSuccess ||
-        cudaMemcpyAsync(&status, ex.dstatus, 4, cudaMemcpyDeviceToHost, ex.stream) != cudaSuccess ||
         cudaStreamSynchronize(ex.stream) != cudaSuccess)
         return FAMST_ERR_CUDA;
-    if (status & STATUS_LOOP_LIMIT) return FAMST_ERR_TIMEOUT;   // a tile gave up: pairs are missing
+    if (got >= NT_GAVE_UP) return FAMST_ERR_TIMEOUT;
     if (got > (unsigned long long)cap) return FAMST_OK;
     const unsigned sgrid = unsigned((got + 255) / 256);
     if (got > 0)

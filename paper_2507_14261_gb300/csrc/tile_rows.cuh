@@ -49,7 +49,9 @@ constexpr int KEYS = 256;   // rows of a key tile
 // A permutation of [0, n) without structure: which row stands at position
 // `pos` (products with odd numbers, sums and xor-shifts modulo 2^b permute
 // [0, 2^b); a value beyond n steps on until it is back inside, less than one
-// step in the mean). Another `salt`, another permutation.
+// step in the mean). Another `salt`, another permutation. (The odd numbers: 2^32
+// over the golden ratio, as in Knuth's multiplicative hashing, and the two
+// multipliers of A. Appleby's MurmurHash3 finaliser.)
 //
 // The tiles' threshold is the largest of four column groups' R-th scores
 // (columns 16 g .. 16 g + 15 of every 64): tight when a row's near keys are

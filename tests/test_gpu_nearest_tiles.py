@@ -68,11 +68,3 @@ def test_ties_overflow_the_survivors(orc, ctx):
     b[:, 0] += 30.0
     X = np.ascontiguousarray(np.concatenate([a, b]), dtype=np.float32)
     _check(orc, ctx, X, (np.arange(4500) >= 2500).astype(np.int64), 7)
-
-
-@pytest.mark.parametrize("n,d,t,lam", [(20000, 32, 300, 32), (20011, 64, 600, 2)])
-def test_bounds_before_the_search(orc, ctx, n, d, t, lam):
-    # room for a search only after a launch that lowers the bounds
-    rng = np.random.default_rng(n)
-    X = rng.standard_normal((n, d)) + 6.0 * rng.standard_normal((t, d))[np.arange(n) % t]
-    _check(orc, ctx, np.ascontiguousarray(X, dtype=np.float32), np.arange(n) % t, lam)
